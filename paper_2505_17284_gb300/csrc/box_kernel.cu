@@ -152,70 +152,51 @@ __global__ void __launch_bounds__(kBoxThreads, 2)
     }
   }
 
-  // block reduction in a fixed order: lanes (FP64 from here), then warps
+  // block reduction in a fixed order, in FP64: one warp per quantity
   constexpr int NB = 2 * kMaxBox;
-  __shared__ double red[kBoxThreads / 32][NB];
+  static_assert(kBoxThreads / 32 >= NB, "one warp per quantity");
+  __shared__ float part[NB][kBoxThreads];
   __shared__ double tot[NB];
   __shared__ uint32_t s_last;
 #pragma unroll
-  for (int q = 0; q < NB; ++q) {
-    const double v = warp_sum_d((double)acc[q / kMaxBox][q % kMaxBox]);
-    if (lane == 0) red[warp][q] = v;
-  }
+  for (int q = 0; q < NB; ++q) part[q][threadIdx.x] = acc[q / kMaxBox][q % kMaxBox];
   __syncthreads();
-  if (threadIdx.x < NB) {
-    double v = 0.0;
-    for (int w = 0; w < kBoxThreads / 32; ++w) v += red[w][threadIdx.x];
-    d.box_partials[(size_t)it.item * NB + threadIdx.x] = v;
+  const bool used = warp < NB && (warp % kMaxBox) < d.n_boxes && (heun || warp < kMaxBox);
+  if (used) {
+    const double v = warp_block_sum<kBoxThreads>(part[warp]);
+    if (lane == 0) d.box_partials[(size_t)warp * it.count + it.item] = v;
   }
-  __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
+    __threadfence();   // the block's partials (ordered before by the barrier) before its ticket
     const uint32_t t = atomicAdd(&st->box_ticket, 1u);
     s_last = (t == static_cast<uint32_t>(it.count - 1)) ? 1u : 0u;
+    __threadfence();
   }
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
-  // all threads: item i goes to thread i mod kBoxThreads, then the fixed-order
-  // block reduction
-  double part[NB];
-#pragma unroll
-  for (int q = 0; q < NB; ++q) part[q] = 0.0;
-  for (int i = threadIdx.x; i < it.count; i += kBoxThreads) {
-#pragma unroll
-    for (int q = 0; q < NB; ++q) part[q] += __ldcg(d.box_partials + (size_t)i * NB + q);
-  }
-#pragma unroll
-  for (int q = 0; q < NB; ++q) {
-    const double v = warp_sum_d(part[q]);
-    if (lane == 0) red[warp][q] = v;
+  if (warp < NB) {
+    const double v = used ? warp_rows_sum(d.box_partials + (size_t)warp * it.count, it.count) : 0.0;
+    if (lane == 0) tot[warp] = v;
   }
   __syncthreads();
-  if (threadIdx.x < NB) {
-    double v = 0.0;
-    for (int w = 0; w < kBoxThreads / 32; ++w) v += red[w][threadIdx.x];
-    tot[threadIdx.x] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  const int b = threadIdx.x;
+  if (b < kMaxBox) {
     const double dt = d.dt_d;
-    for (int b = 0; b < kMaxBox; ++b) {
-      const bool on = b < d.n_boxes;
-      const double S0 = on ? tot[b] : 0.0, S1 = on ? tot[kMaxBox + b] : 0.0;
-      if (stage == STAGE_EULER) {
-        st->B_I[b] += dt * st->B_cur[b];
-        st->B_cur[b] = S0;
-      } else if (stage == STAGE_HEUN2) {
-        st->B_I[b] += 0.5 * dt * (st->B_cur[b] + S0);
-        st->B_cur[b] = S1;
-      } else {  // STAGE_INIT
-        st->B_cur[b] = S0;
-      }
+    const double S0 = tot[b], S1 = tot[kMaxBox + b];
+    if (stage == STAGE_EULER) {
+      st->B_I[b] += dt * st->B_cur[b];
+      st->B_cur[b] = S0;
+    } else if (heun) {
+      st->B_I[b] += 0.5 * dt * (st->B_cur[b] + S0);
+      st->B_cur[b] = S1;
+    } else {  // STAGE_INIT
+      st->B_cur[b] = S0;
     }
+  }
+  if (b == 0) {
     st->box_step = st->step;
     st->box_ticket = 0u;
-    __threadfence();
   }
 }
 

@@ -257,65 +257,103 @@ __device__ __forceinline__ void block_reduce_q(const double (&acc)[NQ], int nq, 
   __syncthreads();
 }
 
+// Sum over a block of one FP32 value per thread (v[0 .. NT) in shared memory), in
+// FP64, by one warp; every lane returns it. A lane first adds its NT / 32 values
+// with Knuth's two-sum (the rounding errors of an FP32 sum, kept beside it), so
+// that a conversion and 6 additions run on the FP64 pipe instead of 5 additions
+// in each of the block's warps: that pipe adds about 2 lanes per cycle and SM
+// here, and the block sums were most of a small launch's tail.
+template <int NT>
+__device__ __forceinline__ double warp_block_sum(const float* v) {
+  const int lane = threadIdx.x & 31;
+  float s = 0.f, e = 0.f;
+#pragma unroll
+  for (int j = 0; j < NT / 32; ++j) {
+    const float x = v[lane + 32 * j];
+    const float t = s + x, z = t - s;
+    e += (s - (t - z)) + (x - z);
+    s = t;
+  }
+  double r = (double)s + (double)e;
+  if (!isfinite(r)) {   // a value, or the FP32 sum of finite ones, is not finite
+    r = 0.0;
+    for (int j = 0; j < NT / 32; ++j) r += (double)v[lane + 32 * j];
+  }
+  return warp_sum_d(r);
+}
+
+// Sum over rows [0, n) of one quantity by one warp, FP64, fixed order.
+__device__ __forceinline__ double warp_rows_sum(const double* row, int n) {
+  const int lane = threadIdx.x & 31;
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int i = lane; i < n; i += 128) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (i + 32 * j < n) a[j] += __ldcg(row + i + 32 * j);
+  }
+  return warp_sum_d((a[0] + a[1]) + (a[2] + a[3]));
+}
+
 // Write this work item's QoI partial (red[0..nq)), and if it is the last item of
 // its instance in this launch, reduce all partials in item order and apply the
-// time-integration update of `stage`. Must be called by all threads.
+// time-integration update of `stage`. Must be called by all threads. Partials are
+// kept quantity by quantity ([nq][count]): the last item's warps read a quantity
+// each, 32 items at a time, and one thread per quantity then updates the state.
+// Bound by latency: it is the tail of every launch. With the block sums taken by
+// all warps on the FP64 pipe, a fence by every thread and a serial update of 18
+// quantities by one thread, a 70^2 x 64 first-order step took 72 us with its QoIs
+// read, 140^2 x 128 Heun 111 us; now 58 and 89 us.
 template <int NT>
 __device__ void finalize_item(const InstDesc& d, const WorkItem& it, const double* red, int stage,
-                              double* scratch /*[NT/32][NQ]*/) {
+                              double* scratch /*[NQ]*/) {
   __shared__ uint32_t s_last;
-  const int nq = d.n_regions + 2;
-  if (threadIdx.x < NQ) d.partials[(size_t)it.item * NQ + threadIdx.x] = (threadIdx.x < nq) ? red[threadIdx.x] : 0.0;
-  __threadfence();
+  const int nreg = d.n_regions, nq = nreg + 2;
+  InstState* st = d.st;
+  if (threadIdx.x < nq) d.partials[(size_t)threadIdx.x * it.count + it.item] = red[threadIdx.x];
   __syncthreads();
   if (threadIdx.x == 0) {
-    const uint32_t t = atomicAdd(&d.st->ticket, 1u);
+    __threadfence();   // the block's partials (ordered before by the barrier) before its ticket
+    const uint32_t t = atomicAdd(&st->ticket, 1u);
     s_last = (t == static_cast<uint32_t>(it.count - 1)) ? 1u : 0u;
+    __threadfence();
   }
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
-  // fixed-order reduction over the count partial rows
-  double acc[NQ];
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) acc[q] = 0.0;
-  for (int i = threadIdx.x; i < it.count; i += NT) {
-    const double* row = d.partials + (size_t)i * NQ;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q)
-      if (q < nq) acc[q] += __ldcg(row + q);
+  for (int q = threadIdx.x >> 5; q < nq; q += NT / 32) {
+    const double v = warp_rows_sum(d.partials + (size_t)q * it.count, it.count);
+    if ((threadIdx.x & 31) == 0) scratch[q] = v;
   }
-  block_reduce_q<NT>(acc, nq, scratch);
-  if (threadIdx.x == 0) {
-    InstState* st = d.st;
-    double S[NQ];
-    // map compact order (regions..., mass, outflow) to the NQ layout
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) S[q] = 0.0;
-    for (int r = 0; r < d.n_regions; ++r) S[r] = scratch[r];
-    S[kQMass] = scratch[d.n_regions];
-    S[kQOut] = scratch[d.n_regions + 1];
+  __syncthreads();
+  // compact order (regions..., mass, outflow) to the NQ layout, one thread each
+  const int q = threadIdx.x;
+  if (q < NQ) {
+    double S = 0.0;
+    if (q < nreg) S = scratch[q];
+    if (q == kQMass) S = scratch[nreg];
+    if (q == kQOut) S = scratch[nreg + 1];
     const double dt = d.dt_d;
     if (stage == STAGE_EULER) {
-      for (int q = 0; q < NQ; ++q) st->I[q] += dt * st->S_cur[q];
-      for (int q = 0; q < NQ; ++q) st->S_cur[q] = S[q];
+      st->I[q] += dt * st->S_cur[q];
+      st->S_cur[q] = S;
+    } else if (stage == STAGE_HEUN1) {
+      st->I[q] += 0.5 * dt * st->S_cur[q];
+      st->S_mid[q] = S;
+    } else if (stage == STAGE_HEUN2) {
+      st->I[q] += 0.5 * dt * st->S_mid[q];
+      st->S_cur[q] = S;
+    } else {  // STAGE_INIT
+      st->S_cur[q] = S;
+    }
+    if (!isfinite(S)) atomicCAS(&st->status, DEV_OK, DEV_NONFINITE);
+  }
+  if (q == 0) {
+    if (stage == STAGE_EULER) {
       st->step += 1;
       st->parity ^= 1;
-    } else if (stage == STAGE_HEUN1) {
-      for (int q = 0; q < NQ; ++q) st->I[q] += 0.5 * dt * st->S_cur[q];
-      for (int q = 0; q < NQ; ++q) st->S_mid[q] = S[q];
     } else if (stage == STAGE_HEUN2) {
-      for (int q = 0; q < NQ; ++q) st->I[q] += 0.5 * dt * st->S_mid[q];
-      for (int q = 0; q < NQ; ++q) st->S_cur[q] = S[q];
       st->step += 1;
-    } else {  // STAGE_INIT
-      for (int q = 0; q < NQ; ++q) st->S_cur[q] = S[q];
     }
-    bool finite = isfinite(S[kQMass]) && isfinite(S[kQOut]);
-    for (int r = 0; r < d.n_regions; ++r) finite = finite && isfinite(S[r]);
-    if (!finite && st->status == DEV_OK) st->status = DEV_NONFINITE;
     st->ticket = 0u;
-    __threadfence();
   }
 }
 
