@@ -140,18 +140,20 @@ typedef void (*rt_free_fn)(void* ptr, void* ctx);
  *     arithmetic is FP32 either way, QoI accumulation FP64).
  *   dt > 0: target step; N_t = ceil(t_end/dt - 1e-9) and dt = t_end/N_t.
  *   dt <= 0: Cartesian 0.5*min(dx,dy); triangles 0.9*min_i 2 A_i / P_i.
- *   tile_x, tile_y: Cartesian tile: cells per strip in x (16: runs of 2 cells per
- *     warp; 32: runs of 4, which needs chunk-uniform directions with 2 ordinates
- *     per lane) and rows per segment (at most 256); 0 = chosen by the library.
- *   variant: Cartesian kernel variant. 0 = chosen by the library; 1 = per-lane
+ *   tile_x, tile_y: Cartesian tile: cells per work item in x (16, or 32, which needs
+ *     chunk-uniform directions in chunks of 64 ordinates when asked for) and rows per
+ *     segment (at most 256); 0 = chosen by the library.
+ *   variant: directions of the Cartesian kernel. 0 = chosen by the library; 1 = per-lane
  *     flow directions (any quadrature); 2 = chunk-uniform directions, usable when
- *     every chunk of ordinates has one sign of xi and one of eta (the product
+ *     every chunk of 128 or 64 ordinates has one sign of xi and one of eta (the product
  *     quadrature's quadrants are contiguous); RT_EINVAL if it is not. The
  *     library takes chunk-uniform directions where the chunks allow them, except
- *     where only 32-cell strips would (2 ordinates per lane) on a grid of at most
- *     1e5 cells: there the per-lane variant measured faster.
+ *     where only chunks of 64 would on a grid of at most 1e5 cells.
  *   vec: Cartesian ordinates per lane (1, 2 or 4; 0 = chosen by the library);
  *     RT_EINVAL if the quadrature does not allow it (see rt_info_t for the choice).
+ *     With per-lane directions, a number asks for the general kernel (the one that
+ *     rt_cart_stage_noalloc runs); 0 lets the library take the streaming kernel where the
+ *     ordinates allow it (it always takes four per lane).
  *   alloc/free/alloc_ctx: device allocator (NULL = cudaMalloc/cudaFree).
  *   stream: cudaStream_t for every launch and copy. */
 typedef struct {
@@ -219,7 +221,8 @@ typedef struct {
   int32_t variant;   /* kernel variant in use: Cartesian 1 per-lane, 2 chunk-uniform directions;
                         triangles 3 first order with each chunk's rows staged in shared memory,
                         0 otherwise (rows gathered from global memory) */
-  int32_t vec;       /* ordinates per lane */
+  int32_t vec;       /* ordinates per lane (Cartesian: 0 if per-lane directions run in the streaming
+                        kernel, which takes four) */
   int32_t regrouped; /* Cartesian: 1 if the ordinates are stored regrouped by direction quadrant, each
                         quadrant padded with zero-weight ordinates to whole chunks (done when the
                         caller's order does not give sign-uniform chunks and the padding adds at most
@@ -312,7 +315,8 @@ rt_status rt_set_state(rt_solver* s, const void* host, size_t bytes);
 /* Test hooks, not for production use: key "wait_limit_cycles" bounds every
  * device-side wait (default about two seconds of SM clock); key "drop_load"
  * (value q >= 0) makes the Cartesian kernel skip its q-th tile load, so that the
- * wait for it runs out and the launch reports RT_ETIMEOUT. value < 0 clears.
+ * wait for it runs out and the launch reports RT_ETIMEOUT (the streaming kernel has
+ * no such wait: it reports RT_ETIMEOUT at once for any q). value < 0 clears.
  * Key "tri_staged" (first-order triangle solvers): 1 runs the stage with the
  * kernel that stages each chunk's rows in shared memory (the default), 0 with
  * the kernel that gathers neighbour rows from global memory; RT_EINVAL for
@@ -327,8 +331,8 @@ const char* rt_last_error(void);
 /* ---------------------------------------------------------------------------
  * Autotuner (Cartesian meshes). The paper has no counterpart: it chooses among
  * the library's own kernel configurations. For the problem and options given,
- * each candidate (strip width 16 or 32 cells, segment length in {auto, 16, 24,
- * ..., 64} rows, per-lane or chunk-uniform directions; only those the
+ * each candidate (strip width 16 or 32 cells, segment length in {auto, 4, 6, 8, 12,
+ * 16, 24, ..., 64} rows, per-lane or chunk-uniform directions; only those the
  * quadrature and shared memory allow, and opts->variant/vec if set) is built
  * as a full solver with rt_create, advanced one step, then timed with CUDA
  * events over `steps` further steps (at most N_t - 1) on opts->stream, and

@@ -28,8 +28,9 @@ def device_key() -> str:
 
 
 def shape_key(problem, M: int, order: int, integrator: int, storage: int) -> str:
+    # "stream": the kernel family; entries tuned for kernels that are gone are not used
     m = problem.mesh
-    return f"{device_key()}|cart{m.nx}x{m.ny}|M{M}|o{order}|i{integrator}|s{storage}"
+    return f"{device_key()}|stream|cart{m.nx}x{m.ny}|M{M}|o{order}|i{integrator}|s{storage}"
 
 
 def _load() -> dict:

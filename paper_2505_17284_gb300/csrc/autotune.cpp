@@ -25,7 +25,7 @@ extern "C" rt_status rt_autotune(const rt_mesh* mesh, const rt_materials* mat, c
 
   struct Cand { int tile_x, tile_y, variant; };
   std::vector<Cand> cands;
-  const int lys[] = {0, 16, 24, 32, 40, 48, 56, 64};
+  const int lys[] = {0, 4, 6, 8, 12, 16, 24, 32, 40, 48, 56, 64};
   for (int tx : {16, 32})
     for (int var : {0, 1}) {
       if (tx == 32 && var == 1) continue;   // 32-cell strips exist for chunk-uniform directions only

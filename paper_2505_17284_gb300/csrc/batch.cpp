@@ -225,7 +225,9 @@ rt_status rebuild(rt_batch* b) {
     const Slot& S = b->slots[i];
     if (!S.used || S.held || S.done >= S.inst.n_steps) continue;
     const Instance& I = S.inst;
-    by_variant[std::make_tuple(I.kind, I.order, I.integrator, I.run, I.cvec, I.vec, I.uni)].push_back(i);
+    // (the Cartesian kernels do not depend on I.vec)
+    const int vec = I.kind == RT_MESH_CARTESIAN ? 0 : I.vec;
+    by_variant[std::make_tuple(I.kind, I.order, I.integrator, I.run, I.cvec, vec, I.uni)].push_back(i);
     b->members.push_back(i);
   }
   std::vector<WorkItem> items, box_items;

@@ -371,389 +371,7 @@ __device__ __forceinline__ void cart_tile(const InstDesc& d, const WorkItem& it,
                                      x0, ya, nrows, TX, bacc);
 }
 
-// One row pull of the chunk-uniform tile: pull e (chunk c, row i of the chunk)
-// into ring slot `slot`, completing full[slot]. Only tiles that touch the y
-// sides of the domain (YB) pull rows outside it: the wrapped row on a periodic
-// axis, else nothing (the ghost values are set in registers); interior tiles
-// skip those tests, since the issuing thread is on the ring's critical path.
-template <typename L, bool YB>
-struct UniPull {
-  const InstDesc* d;
-  uint8_t* ring;
-  uint64_t* full;
-  int* slot_pull;   // [NS] last pull issued into each slot (read by the drain)
-  const CUtensorMap* map_halo;
-  const CUtensorMap* map_base;
-  int x0, ya, yb;
-
-  __device__ __forceinline__ void issue(int e, int c, int i, int slot) const {
-    constexpr int H = L::H, C = L::C;
-    const int dy = d->cdir_y[c];
-    const int p = ((dy > 0) ? ya : yb - 1) + dy * (i - H);
-    uint8_t* dst = ring + slot * L::slot_bytes;
-    bool halo = true;
-    int pl = p;
-    if constexpr (YB) {
-      if (p < 0 || p >= d->ny) {
-        halo = d->periodic_y != 0;
-        if (halo) pl = wrap_index(p, d->ny);
-      }
-    }
-    const bool base = L::base_bytes > 0 && (i >= H + 1);   // Heun stage 2: psi^n of the row completed here
-    const uint32_t bytes = (halo ? L::halo_bytes : 0) + (base ? L::base_bytes : 0);
-    slot_pull[slot] = e;
-    if ((int64_t)e == d->drop_load) return;   // test hook: that pull never completes
-    if (bytes == 0) {
-      mbar_arrive(&full[slot]);
-      return;
-    }
-    mbar_arrive_expect_tx(&full[slot], bytes);
-    if (halo) tma_load_3d(dst, map_halo, &full[slot], c * C, x0 - H, pl);
-    if (base) tma_load_3d(dst + L::halo_bytes, map_base, &full[slot], c * C, x0, p - dy);
-  }
-};
-
-// Chunk-uniform variant. When every chunk of C ordinates has one sign of xi and
-// one of eta (the product quadrature's quadrants are contiguous, so its chunks
-// are), the whole CTA shares the flow direction of a chunk. Each chunk then
-// walks its rows along the flow in y (upwind row first): the face between two
-// consecutive rows comes from the row already seen, so a row is completed one
-// row after it arrives, and the window carries only the previous row, its
-// difference to the row before, and the face value below it.
-//
-// Pipeline. Pull q of the tile (all chunks in order) lands in ring slot q mod NS
-// and completes full[slot]. Pull q - 1 is needed until every warp has finished
-// pull q; after the CTA barrier that closes row q, thread 0 issues pull
-// q - 1 + NS into its slot. (Releasing slots per warp with shared-memory
-// atomics or mbarrier arrivals, so that warps run apart, measured slower on
-// sm_103a than this one barrier per row.) The waits are bounded; the barrier
-// also carries a failed wait, so all warps stop together, drain the loads in
-// flight and report the timeout.
-// Register window of one row of the chunk-uniform tile, per lane: the row's
-// values c, their difference to the row before along the flow d, and the face
-// value g between the row before and this row.
-template <int R, int V2>
-struct UniRow {
-  float2 c[R][V2], d[R][V2], g[R][V2];
-};
-
-template <int ORDER, int R, int V, int STAGE, typename T, bool XB, bool YB>
-__device__ __forceinline__ void cart_tile_uni(const InstDesc& d, const WorkItem& it, InstState* st,
-                                              uint8_t* smem) {
-  using L = CartCfg<ORDER, R, V, STAGE, T>;
-  constexpr int H = L::H, TX = L::TX, C = L::C, NS = L::NS, NL = L::NL;
-  constexpr int V2 = V / 2;   // ordinate pairs per lane: arithmetic runs on float pairs
-  static_assert(NS >= 3, "the ring must hold two resident rows plus one load in flight");
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-  const int parity = (STAGE == STAGE_EULER) ? st->parity : 0;
-  [[maybe_unused]] const uint32_t salt = sr_salt(st->step, STAGE);   // BF16 stochastic rounding
-  const int in_buf = (STAGE == STAGE_EULER) ? parity : (STAGE == STAGE_HEUN1 ? 0 : 1);
-  const int out_buf = (STAGE == STAGE_EULER) ? (1 - parity) : (STAGE == STAGE_HEUN1 ? 1 : 0);
-  const float* __restrict__ phi_in = d.phi[in_buf];
-  float* __restrict__ phi_out = d.phi[out_buf];
-  T* __restrict__ psi_out = reinterpret_cast<T*>(d.psi[out_buf]);
-  const CUtensorMap* map_halo = &d.tm_psi_halo[in_buf];
-  const CUtensorMap* map_base = &d.tm_psi_center;
-
-  const int nx = d.nx, ny = d.ny, Mpad = d.Mpad;
-  const int x0 = it.a * TX;
-  const int ya = it.b * d.ly;
-  const int yb = min(ny, ya + d.ly);
-  const int nrows = yb - ya;
-  const int Lc = nrows + H + 1;     // rows pulled per chunk, in flow order: H before the tile, 1 after
-  const int total = d.n_chunks * Lc;
-
-  uint8_t* ring = smem;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + L::ring_bytes);
-  int* slot_pull = reinterpret_cast<int*>(full + NS);   // [NS]
-  float2* tile_ab = reinterpret_cast<float2*>(smem + L::ring_bytes + 128);   // (a, b) per cell
-  float* tile_acc = reinterpret_cast<float*>(tile_ab + d.ly * TX);
-  double* red = reinterpret_cast<double*>(smem + L::ring_bytes + 128 + cart_tile_bytes(TX, d.ly));
-  const int64_t limit = d.wait_limit;
-  static_assert(NS * (8 + 4) <= 128, "ring control block must fit its 128 bytes");
-  const UniPull<L, YB> pull{&d, ring, full, slot_pull, map_halo, map_base, x0, ya, yb};
-
-  if (tid == 0) {
-    for (int s = 0; s < NS; ++s) {
-      mbar_init(&full[s], 1);
-      slot_pull[s] = -1;
-    }
-    fence_barrier_init();
-    fence_tensormap_acquire(map_halo);
-    prefetch_tensormap(map_halo);
-    if (STAGE == STAGE_HEUN2) {
-      fence_tensormap_acquire(map_base);
-      prefetch_tensormap(map_base);
-    }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    for (int e = 0, c = 0, i = 0; e < min(NS, total); ++e) {
-      pull.issue(e, c, i, e);
-      if (++i == Lc) { i = 0; ++c; }
-    }
-  }
-  const float dt = d.dt;
-  for (int i = tid; i < nrows * TX; i += kCartThreads) {
-    const int r = i / TX, xl = i - r * TX;
-    const int gx = x0 + xl;
-    float a = 1.f, b = 0.f;
-    if (gx < nx) {
-      const size_t cell = (size_t)(ya + r) * nx + gx;
-      const int m = d.mat[cell];
-      a = 1.f - dt * d.sig_t[m];
-      b = dt * (d.sig_s2pi[m] * phi_in[cell] + d.q_src[m]);
-    }
-    tile_ab[i] = make_float2(a, b);
-    tile_acc[i] = 0.f;
-  }
-  __syncthreads();
-
-  float bacc = 0.f;
-  const float ly_f = (float)d.dy_d, lx_f = (float)d.dx_d;
-  const int xl0 = warp * R;
-  bool ok = true;
-  int q = 0;           // global pull index
-  int slot = 0;        // ring slot of pull q
-  uint32_t ph = 0;     // phase parity of full[slot] for pull q
-  int pslot = NS - 1;  // ring slot of pull q - 1
-  // chunk and row of pull q - 1 + NS, issued after row q (advanced once per pull from q = 1)
-  int nc = 0, ni = NS;
-  while (ni >= Lc) { ni -= Lc; ++nc; }
-
-  for (int c = 0; c < d.n_chunks && ok; ++c) {
-    auto chunk = [&](auto dir) {
-      constexpr int DXS = decltype(dir)::value;   // sign of xi in this chunk
-      const int k0 = c * C + lane * V;
-      [[maybe_unused]] const uint32_t gkey = sr_gkey(k0 >> 2, salt);   // BF16 rounding: the lane's group of 4
-      const int dys = d.cdir_y[c];
-      const int s0 = (DXS > 0) ? xl0 : xl0 + R - 1;   // this warp's first cell along the flow
-      float2 w2[V2], ax2[V2], ay2[V2];
-#pragma unroll
-      for (int v = 0; v < V2; ++v) {
-        w2[v] = make_float2(d.w[k0 + 2 * v], d.w[k0 + 2 * v + 1]);
-        ax2[v] = make_float2(dt * fabsf(d.xi[k0 + 2 * v]) * d.inv_dx, dt * fabsf(d.xi[k0 + 2 * v + 1]) * d.inv_dx);
-        ay2[v] = make_float2(dt * fabsf(d.eta[k0 + 2 * v]) * d.inv_dy, dt * fabsf(d.eta[k0 + 2 * v + 1]) * d.inv_dy);
-      }
-      // psi^- of the rows before the tile in flow order (entering through that side)
-      const float gy_up = (dys > 0) ? d.ghost[2] : d.ghost[3];
-      const int start = (dys > 0) ? ya : yb - 1;
-      // lane's element of cell position s0 within a slot, in bytes
-      const int lofs = ((s0 + H) * C + lane * V) * (int)sizeof(T);
-      constexpr int PSTEP = DXS * C * (int)sizeof(T);   // next cell along the flow
-      // output row pointer (row `start`, cell s0) and its step per completed row
-      T* op = psi_out + ((size_t)start * nx + (x0 + s0)) * Mpad + k0;
-      const ptrdiff_t ostep = (ptrdiff_t)dys * nx * Mpad;
-      const ptrdiff_t mstep = (ptrdiff_t)DXS * Mpad;
-      const float2* tab = tile_ab + (start - ya) * TX + s0;
-      const int tstep = dys * TX;
-      float* tacc = tile_acc + (start - ya) * TX + xl0 + lane / (32 / R);
-      int jrow = start;    // row completed next
-      int p = start - dys * H;
-
-      // Row i of the chunk (row p of the grid) into window X; Y holds the row
-      // before it, which is completed here. The two windows swap roles from row
-      // to row, so no register is copied.
-      auto row = [&](const int i, UniRow<R, V2>& X, const UniRow<R, V2>& Y) -> bool {
-        const bool wok = mbar_wait_bounded(&full[slot], ph, limit);
-        const uint8_t* cur = ring + slot * L::slot_bytes + lofs;
-        bool p_in = true;
-        if constexpr (YB) p_in = d.periodic_y || (p >= 0 && p < ny);
-        if (YB && !p_in) {
-          const float gv = (i < H) ? gy_up : 0.f;   // after the tile only the first-order face sees it
-#pragma unroll
-          for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int v = 0; v < V2; ++v) X.c[r][v] = make_float2(gv, gv);
-        } else {
-#pragma unroll
-          for (int r = 0; r < R; ++r) lds_vec2<T, V>(reinterpret_cast<const T*>(cur + r * PSTEP), X.c[r]);
-        }
-        // face between the previous row (upwind) and row p
-        if constexpr (ORDER == 2) {
-          bool second = true;
-          if constexpr (YB) {
-            const int pp = p - dys;
-            if (!d.periodic_y && (pp >= 0 && pp < ny) != p_in) second = false;   // domain boundary face: first order
-          }
-#pragma unroll
-          for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int v = 0; v < V2; ++v) {
-              X.d[r][v] = sub2(X.c[r][v], Y.c[r][v]);
-              const float2 ext = __ffma2_rn(make_float2(0.5f, 0.5f),
-                                            minmod2r(X.d[r][v], Y.d[r][v], relu2(X.d[r][v]), relu2(Y.d[r][v])), Y.c[r][v]);
-              X.g[r][v] = (!YB || second) ? ext : Y.c[r][v];
-            }
-        } else {
-#pragma unroll
-          for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int v = 0; v < V2; ++v) X.g[r][v] = Y.c[r][v];
-        }
-        // completion of the previous row (its slot, pull q - 1, is still resident)
-        if (i >= H + 1) {
-          const uint8_t* prv = ring + pslot * L::slot_bytes + lofs;
-          float2 u[NL][V2];
-#pragma unroll
-          for (int m = 0; m < NL; ++m) {
-            if (m >= H && m < H + R) {
-              // the warp's own cells of the previous row are still in the window (loaded one row ago)
-#pragma unroll
-              for (int v = 0; v < V2; ++v) u[m][v] = Y.c[m - H][v];
-            } else {
-              lds_vec2<T, V>(reinterpret_cast<const T*>(prv + (m - H) * PSTEP), u[m]);
-            }
-            if constexpr (XB) {
-              const int gpos = x0 + s0 + DXS * (m - H);
-              if (gpos < 0 || gpos >= nx) {
-                if (d.periodic_x) {
-                  // periodic: the wrapped cell of the same row, from the input state
-                  lds_vec2<T, V>(reinterpret_cast<const T*>(d.psi[in_buf]) + ((size_t)jrow * nx + wrap_index(gpos, nx)) * Mpad + k0,
-                                 u[m]);
-                } else {
-                  // entering ordinates see psi^- of the side, leaving ones nothing (only
-                  // first-order faces read it)
-                  const float gside = (gpos < 0) ? d.ghost[0] : d.ghost[1];
-                  const bool enter = (gpos < 0) == (DXS > 0);
-#pragma unroll
-                  for (int v = 0; v < V2; ++v) u[m][v] = enter ? make_float2(gside, gside) : make_float2(0.f, 0.f);
-                }
-              }
-            }
-          }
-          // faces m = -1 .. R-1 along x (outgoing face of upwind cell m); first order on domain faces
-          float2 F[R + 1][V2];
-          if constexpr (ORDER == 2) {
-            float2 D[NL][V2], RD[NL][V2];   // D[m] = u[m] - u[m-1], RD = max(D, 0)
-#pragma unroll
-            for (int m = 1; m < NL; ++m)
-#pragma unroll
-              for (int v = 0; v < V2; ++v) {
-                D[m][v] = sub2(u[m][v], u[m - 1][v]);
-                RD[m][v] = relu2(D[m][v]);
-              }
-#pragma unroll
-            for (int m = -1; m < R; ++m) {
-              bool second = true;
-              if constexpr (XB) {
-                const int ga = x0 + s0 + DXS * m, gb = ga + DXS;
-                if (!d.periodic_x && !((ga >= 0 && ga < nx) && (gb >= 0 && gb < nx))) second = false;
-              }
-#pragma unroll
-              for (int v = 0; v < V2; ++v)
-                F[m + 1][v] = second ? __ffma2_rn(make_float2(0.5f, 0.5f),
-                                                  minmod2r(D[m + H + 1][v], D[m + H][v], RD[m + H + 1][v], RD[m + H][v]),
-                                                  u[m + H][v])
-                                     : u[m + H][v];
-            }
-          } else {
-#pragma unroll
-            for (int m = -1; m < R; ++m)
-#pragma unroll
-              for (int v = 0; v < V2; ++v) F[m + 1][v] = u[m + H][v];
-          }
-          float contrib[R];
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            const float2 ab = tab[DXS * r];
-            const float2 ta2 = make_float2(ab.x, ab.x), tb2 = make_float2(ab.y, ab.y);
-            [[maybe_unused]] float2 bse[V2];
-            if constexpr (STAGE == STAGE_HEUN2)
-              lds_vec2<T, V>(reinterpret_cast<const T*>(cur - H * C * (int)sizeof(T) + L::halo_bytes + r * PSTEP), bse);
-            float2 out[V2];
-            float2 pw2 = make_float2(0.f, 0.f);
-            [[maybe_unused]] uint2 rb4;
-            if constexpr (sizeof(T) == 2) rb4 = sr_bits4((uint32_t)(jrow * nx + (x0 + s0 + DXS * r)), gkey);
-#pragma unroll
-            for (int v = 0; v < V2; ++v) {
-              const float2 div = __ffma2_rn(ax2[v], sub2(F[r + 1][v], F[r][v]), __fmul2_rn(ay2[v], sub2(X.g[r][v], Y.g[r][v])));
-              float2 t = sub2(__ffma2_rn(ta2, Y.c[r][v], tb2), div);
-              if constexpr (STAGE == STAGE_HEUN2) t = __fmul2_rn(make_float2(0.5f, 0.5f), __fadd2_rn(bse[v], t));
-              if constexpr (sizeof(T) == 2) t = Store<T>::round_sr2(t, ((k0 + 2 * v) & 2) ? rb4.y : rb4.x);
-              out[v] = t;
-              pw2 = __ffma2_rn(w2[v], t, pw2);
-            }
-            contrib[r] = 0.f;
-            const int gx = x0 + s0 + DXS * r;
-            if (!XB || gx < nx) {
-              stg_vec2<T, V>(op + r * mstep, out);
-              contrib[r] = pw2.x + pw2.y;
-              if (XB || YB) {
-#pragma unroll
-                for (int v = 0; v < V; ++v) {
-                  const float o = (v & 1) ? out[v / 2].y : out[v / 2].x;
-                  const float wv = (v & 1) ? w2[v / 2].y : w2[v / 2].x;
-                  const float xiv = d.xi[k0 + v], etav = d.eta[k0 + v];
-                  if (XB && !d.periodic_x && gx == 0) bacc += ly_f * (wv * -xiv * (xiv < 0.f ? o : (xiv > 0.f ? d.ghost[0] : 0.f)));
-                  if (XB && !d.periodic_x && gx == nx - 1) bacc += ly_f * (wv * xiv * (xiv > 0.f ? o : (xiv < 0.f ? d.ghost[1] : 0.f)));
-                  if (YB && !d.periodic_y && jrow == 0) bacc += lx_f * (wv * -etav * (etav < 0.f ? o : (etav > 0.f ? d.ghost[2] : 0.f)));
-                  if (YB && !d.periodic_y && jrow == ny - 1) bacc += lx_f * (wv * etav * (etav > 0.f ? o : (etav < 0.f ? d.ghost[3] : 0.f)));
-                }
-              }
-            }
-          }
-          float phys[R];
-#pragma unroll
-          for (int r = 0; r < R; ++r) phys[r] = (DXS > 0) ? contrib[r] : contrib[R - 1 - r];
-          const float sphi = multi_warp_sum<R>(phys, lane);
-          if ((lane & (32 / R - 1)) == 0) *tacc += sphi;
-          op += ostep;
-          tab += tstep;
-          tacc += tstep;
-          jrow += dys;
-        }
-        if (__syncthreads_or(!wok)) return false;   // a wait ran out somewhere: every warp stops here
-        if (tid == 0 && q >= 1 && q - 1 + NS < total) {
-          fence_proxy_async_smem();
-          pull.issue(q - 1 + NS, nc, ni, pslot);
-        }
-        if (q >= 1 && ++ni == Lc) { ni = 0; ++nc; }
-        pslot = slot;
-        if (++slot == NS) { slot = 0; ph ^= 1u; }
-        ++q;
-        p += dys;
-        return true;
-      };
-
-      UniRow<R, V2> A, B;
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-#pragma unroll
-        for (int v = 0; v < V2; ++v) B.c[r][v] = B.d[r][v] = B.g[r][v] = make_float2(0.f, 0.f);
-      for (int i = 0; i < Lc; i += 2) {
-        if (!row(i, A, B)) { ok = false; break; }
-        if (i + 1 < Lc && !row(i + 1, B, A)) { ok = false; break; }
-      }
-    };
-    if (d.cdir_x[c] > 0) chunk(std::integral_constant<int, 1>{});
-    else chunk(std::integral_constant<int, -1>{});
-  }
-  __syncthreads();
-  if (!ok) {
-    if (tid == 0) {
-      // drain: the last pull issued into each slot may still be in flight
-      for (int s = 0; s < NS; ++s) {
-        const int e = slot_pull[s];
-        if (e < 0 || (int64_t)e == d.drop_load) continue;
-        mbar_wait_bounded(&full[s], (uint32_t)((e / NS) & 1), limit);
-      }
-      atomicCAS(&st->status, DEV_OK, DEV_TIMEOUT);
-      st->timeout_where = ((int64_t)blockIdx.x << 32) | (int64_t)q;
-    }
-    return;
-  }
-  cart_epilogue<STAGE, kCartThreads>(d, it, phi_out, tile_acc, red, reinterpret_cast<float*>(ring), L::ring_bytes / 4,
-                                     x0, ya, nrows, TX, bacc);
-}
-
-template <int ORDER, int R, int V, int STAGE, typename T, bool XB, bool YB>
-__device__ __noinline__ void cart_tile_uni_edge(const InstDesc* dp, const WorkItem it, InstState* st, uint8_t* smem) {
-  cart_tile_uni<ORDER, R, V, STAGE, T, XB, YB>(*dp, it, st, smem);
-}
-
-template <int ORDER, int R, int V, int STAGE, typename T, bool UNI>
+template <int ORDER, int R, int V, int STAGE, typename T>
 __global__ void __launch_bounds__(kCartThreads, (R * V >= 8 ? 2 : 3))
     cart_stage_kernel(const InstDesc* __restrict__ descs, const WorkItem* __restrict__ items) {
   using L = CartCfg<ORDER, R, V, STAGE, T>;
@@ -769,24 +387,11 @@ __global__ void __launch_bounds__(kCartThreads, (R * V >= 8 ? 2 : 3))
   const int ya = it.b * d.ly;
   const bool xb = (x0 - L::H < 0) || (x0 + L::TX + L::H > d.nx);
   const bool yb = (ya - L::H < 0) || (ya + d.ly + L::H > d.ny);
-  if constexpr (UNI) {
-    // tiles on the domain boundary run out of line, so that their extra state
-    // (ghost values, wrapped rows and cells) does not raise the register
-    // pressure of the interior tiles
-    if (xb) {
-      if (yb) cart_tile_uni_edge<ORDER, R, V, STAGE, T, true, true>(&d, it, st, smem);
-      else cart_tile_uni_edge<ORDER, R, V, STAGE, T, true, false>(&d, it, st, smem);
-    } else {
-      if (yb) cart_tile_uni_edge<ORDER, R, V, STAGE, T, false, true>(&d, it, st, smem);
-      else cart_tile_uni<ORDER, R, V, STAGE, T, false, false>(d, it, st, smem);
-    }
-  } else {
-    if (xb) cart_tile<ORDER, R, V, STAGE, T, true>(d, it, st, smem, yb);
-    else cart_tile<ORDER, R, V, STAGE, T, false>(d, it, st, smem, yb);
-  }
+  if (xb) cart_tile<ORDER, R, V, STAGE, T, true>(d, it, st, smem, yb);
+  else cart_tile<ORDER, R, V, STAGE, T, false>(d, it, st, smem, yb);
 }
 
-template <int ORDER, int R, int V, int STAGE, typename T, bool UNI>
+template <int ORDER, int R, int V, int STAGE, typename T>
 static cudaError_t prepare_one(int ly_max) {
   // Raise the dynamic shared-memory limit of this kernel variant. The attribute
   // belongs to the current device, so the limit already raised is kept per
@@ -800,7 +405,7 @@ static cudaError_t prepare_one(int ly_max) {
   if (e != cudaSuccess) return e;
   const bool tracked = dev >= 0 && dev < kDev;
   if (tracked && smem <= s_limit[dev].load(std::memory_order_acquire)) return cudaSuccess;
-  e = cudaFuncSetAttribute(cart_stage_kernel<ORDER, R, V, STAGE, T, UNI>,
+  e = cudaFuncSetAttribute(cart_stage_kernel<ORDER, R, V, STAGE, T>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (tracked) {
@@ -811,35 +416,36 @@ static cudaError_t prepare_one(int ly_max) {
   return cudaSuccess;
 }
 
-template <int ORDER, int R, int V, int STAGE, typename T, bool UNI>
+template <int ORDER, int R, int V, int STAGE, typename T>
 static cudaError_t launch_one(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int ly_max,
                               cudaStream_t stream) {
-  cudaError_t e = prepare_one<ORDER, R, V, STAGE, T, UNI>(ly_max);
+  cudaError_t e = prepare_one<ORDER, R, V, STAGE, T>(ly_max);
   if (e != cudaSuccess) return e;
-  cart_stage_kernel<ORDER, R, V, STAGE, T, UNI>
+  cart_stage_kernel<ORDER, R, V, STAGE, T>
       <<<n_items, kCartThreads, cart_smem_for<ORDER, R, V, STAGE, T>(ly_max), stream>>>(d_desc, d_items);
   return cudaGetLastError();
 }
 
-// Instantiation units: per storage type T and direction family U, the variants
-// order {1, 2} x (run length R, ordinates per lane V) x stage, with (R, V) in
-// {(2, 1), (2, 2), (2, 4)} for U = false and {(2, 2), (2, 4), (4, 2)} for U = true.
-#define RTK_CART_STAGES(X, O, RR, VV, U, TT) \
-  X(O, RR, VV, STAGE_EULER, U, TT) X(O, RR, VV, STAGE_HEUN1, U, TT) X(O, RR, VV, STAGE_HEUN2, U, TT)
-#define RTK_CART_DEFINE_UNIT(NAME, TT, U, ...)                                                              \
-  cudaError_t cart_prepare_##NAME(int stage, int order, int run, int vec, int ly_max) {                      \
-    RTK_CART_UNIT_LIST(RTK_CART_P_, TT, U)                                                                  \
+// Instantiation units: per storage type, the variants order {1, 2} x ordinates per
+// lane {1, 2, 4} x stage.
+#define RTK_CART_ALL(X, TT)                                                                           \
+  RTK_CART_VECS(X, 1, STAGE_EULER, TT) RTK_CART_VECS(X, 1, STAGE_HEUN1, TT) RTK_CART_VECS(X, 1, STAGE_HEUN2, TT) \
+  RTK_CART_VECS(X, 2, STAGE_EULER, TT) RTK_CART_VECS(X, 2, STAGE_HEUN1, TT) RTK_CART_VECS(X, 2, STAGE_HEUN2, TT)
+#define RTK_CART_VECS(X, O, ST, TT) X(O, 1, ST, TT) X(O, 2, ST, TT) X(O, 4, ST, TT)
+#define RTK_CART_DEFINE_UNIT(NAME, TT)                                                                      \
+  cudaError_t cart_prepare_##NAME(int stage, int order, int vec, int ly_max) {                              \
+    RTK_CART_ALL(RTK_CART_P_, TT)                                                                           \
     return cudaErrorInvalidValue;                                                                           \
   }                                                                                                         \
   cudaError_t cart_launch_##NAME(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage,   \
-                                 int order, int run, int vec, int ly_max, cudaStream_t stream) {            \
-    RTK_CART_UNIT_LIST(RTK_CART_L_, TT, U)                                                                  \
+                                 int order, int vec, int ly_max, cudaStream_t stream) {                     \
+    RTK_CART_ALL(RTK_CART_L_, TT)                                                                           \
     return cudaErrorInvalidValue;                                                                           \
   }
-#define RTK_CART_P_(O, RR, VV, ST, U, TT) \
-  if (order == O && run == RR && vec == VV && stage == ST) return prepare_one<O, RR, VV, ST, TT, U>(ly_max);
-#define RTK_CART_L_(O, RR, VV, ST, U, TT)                                  \
-  if (order == O && run == RR && vec == VV && stage == ST)                 \
-    return launch_one<O, RR, VV, ST, TT, U>(d_desc, d_items, n_items, ly_max, stream);
+#define RTK_CART_P_(O, VV, ST, TT) \
+  if (order == O && vec == VV && stage == ST) return prepare_one<O, 2, VV, ST, TT>(ly_max);
+#define RTK_CART_L_(O, VV, ST, TT)                   \
+  if (order == O && vec == VV && stage == ST)        \
+    return launch_one<O, 2, VV, ST, TT>(d_desc, d_items, n_items, ly_max, stream);
 
 }  // namespace rtk

@@ -407,8 +407,8 @@ static int choose_cart_vec(const rt_quadrature* quad, int Mpad) {
 }
 
 // Chunk-uniform check: for chunks of 32V ordinates, every chunk has one sign of
-// xi and one of eta (zeros fit either). Fills the per-chunk directions.
-static bool chunks_uniform(const rt_quadrature* quad, int Mpad, int V, int8_t* dx, int8_t* dy) {
+// xi and one of eta (zeros fit either).
+static bool chunks_uniform(const rt_quadrature* quad, int Mpad, int V) {
   const int C = 32 * V;
   if (Mpad % C != 0 || Mpad / C > kMaxUniChunks) return false;
   for (int c = 0; c < Mpad / C; ++c) {
@@ -425,13 +425,65 @@ static bool chunks_uniform(const rt_quadrature* quad, int Mpad, int V, int8_t* d
         else if (sy != ky) return false;
       }
     }
-    dx[c] = (int8_t)(sx < 0 ? -1 : 1);
-    dy[c] = (int8_t)(sy < 0 ? -1 : 1);
   }
   return true;
 }
 
-// Resident CTAs per SM of the Cartesian stage kernel at segment length ly: the
+// Ordinate chunks of the streaming Cartesian kernel: windows of 32 consecutive
+// ordinates, each with one sign of eta, and with one sign of xi in every aligned
+// group of four (a lane's ordinates; zeros fit either sign). The ordinates are cut
+// into runs of one sign of eta, or of one sign of both where that takes no more
+// windows (or where a lane would mix signs of xi), and each run is covered by
+// windows that start on a 16-byte boundary of psi. Empty when that takes more than
+// half as many windows again as whole chunks would: the kernel computes whole
+// windows, so the general kernel does less work then.
+static std::vector<int4> plan_stream_chunks(const rt_quadrature* quad, int Mpad, int storage) {
+  auto sgn = [](double v) { return v > 0 ? 1 : (v < 0 ? -1 : 0); };
+  const int M = (int)quad->M;
+  const int align = storage == RT_BF16 ? 8 : 4;
+  auto cover = [&](bool both) {
+    std::vector<int4> out;
+    int k = 0;
+    while (k < M) {
+      int sx = 0, sy = 0, e = k;
+      for (; e < M; ++e) {   // the run of ordinates k .. e-1
+        const int x = sgn(quad->xi[e]), y = sgn(quad->eta[e]);
+        if ((sy && y && y != sy) || (both && sx && x && x != sx)) break;
+        sy = sy ? sy : y;
+        sx = sx ? sx : x;
+      }
+      while (k < e) {
+        const int base = std::min(k / align * align, Mpad - 32);
+        const int hi = std::min(e, base + 32);
+        int dx = 0, mixed = 0;   // sign of xi of the window's ordinates
+        for (int q = k; q < hi; ++q) {
+          const int x = sgn(quad->xi[q]);
+          if (x && dx && x != dx) mixed = 1;
+          dx = dx ? dx : x;
+        }
+        for (int q = base; mixed && q < base + 32; q += 4) {
+          int lx = 0;
+          for (int j = std::max(q, k); j < std::min(q + 4, hi); ++j) {
+            const int x = sgn(quad->xi[j]);
+            if (x && lx && x != lx) return std::vector<int4>();
+            lx = lx ? lx : x;
+          }
+        }
+        const bool whole = k == base && hi == base + 32;
+        out.push_back(make_int4(base, (k - base) | (hi - base) << 8, sy < 0 ? -1 : 1,
+                                mixed || !whole ? 0 : (dx < 0 ? -1 : 1)));
+        k = hi;
+      }
+    }
+    return out;
+  };
+  std::vector<int4> a = cover(false), b = cover(true);
+  if (a.empty() || b.size() <= a.size()) a.swap(b);
+  if ((int64_t)a.size() * 2 > (int64_t)Mpad / 32 * 3) a.clear();
+  return a;
+}
+
+// Resident CTAs per SM of the general Cartesian kernel at segment length ly: the
 // kernel's launch bound (2 with 8 values per thread and row, else 3) and its shared
 // memory (the Heun stage 2 ring is the largest).
 static int cart_ctas_per_sm(const Instance& I, int ly) {
@@ -454,9 +506,8 @@ static bool regroup_quadrature(const rt_quadrature* quad, std::vector<double>& x
                                std::vector<double>& w, std::vector<int32_t>& kmap, std::vector<int32_t>& inv) {
   const int M = (int)quad->M;
   const int Mpad = (M + 31) / 32 * 32;
-  int8_t dx[kMaxUniChunks], dy[kMaxUniChunks];
   for (int V = 4; V >= 2; V /= 2)
-    if (Mpad % (32 * V) == 0 && chunks_uniform(quad, Mpad, V, dx, dy)) return false;   // already uniform
+    if (Mpad % (32 * V) == 0 && chunks_uniform(quad, Mpad, V)) return false;   // already uniform
   auto quadrant = [&](int k) {
     const bool xp = quad->xi[k] >= 0.0, yp = quad->eta[k] >= 0.0;
     return xp ? (yp ? 0 : 3) : (yp ? 1 : 2);
@@ -491,10 +542,50 @@ static bool regroup_quadrature(const rt_quadrature* quad, std::vector<double>& x
   return false;
 }
 
+// Segment length of the streaming kernel for a tile of I.run, by a model of a launch in
+// units of one row of a warp that shares its SM with one CTA. A CTA costs a fixed part
+// (start, tile constants, QoI sums, about 10 rows) and chunks x rows, 1.28 times that
+// with two CTAs on the SM (the most that are resident); with more items than fit at
+// once the fixed parts overlap other CTAs' rows, and the last round adds about 0.4 of
+// an item. Against timings of 13 problems at 3 to 64 rows (70^2 x 64 to 1400^2 x 512)
+// its choice is within 4 % of the best. *cost receives the model's time.
+static int stream_segment(const Instance& I, int run, double* cost) {
+  const int sms = device_sm_count();
+  const int tx = cart_tile_width(run), groups = cart_stream_chunk_groups(tx);
+  const int64_t strips = (I.nx + tx - 1) / tx;
+  const int chunks = ((int)I.str_chunks.size() + groups - 1) / groups;
+  const int stage_hi = I.integrator == RT_HEUN ? STAGE_HEUN2 : STAGE_EULER;
+  int best = 8;
+  *cost = INFINITY;
+  for (int ly = 3; ly <= 64; ++ly) {
+    // two CTAs per SM by shared memory (228 KB, 1 KB of it per CTA reserved)
+    if (cart_smem_bytes(I.order, I.storage, run, I.cvec, ly, stage_hi, 1) > 113 * 1024) break;
+    const int64_t items = strips * ((I.ny + ly - 1) / ly);
+    const int rows = (std::min(ly, I.ny) + (I.order == 2 ? 3 : 1) + 1) / 2 * 2;
+    double t;
+    if (items <= sms) {
+      t = 9.6 + (double)chunks * rows;
+    } else if (items <= 2 * sms) {
+      t = 12.0 + 1.28 * chunks * rows;
+    } else {
+      t = (5.8 + 1.28 * chunks * rows) * ((double)items / (2.0 * sms) + 0.4);
+    }
+    if (t < *cost) {
+      *cost = t;
+      best = ly;
+    }
+  }
+  return best;
+}
+
 static void choose_cart_tiles(Instance& I, int tile_y) {
+  int ly = tile_y;
+  if (ly <= 0 && I.uni) {
+    double cost;
+    ly = stream_segment(I, I.run, &cost);
+  }
   I.tx = cart_tile_width(I.run);
   I.n_strips = (I.nx + I.tx - 1) / I.tx;
-  int ly = tile_y;
   if (ly <= 0) {
     // Segment length by a throughput model: a CTA pulls n_chunks * (ly + H + 1)
     // rows per work item plus a fixed cost of about 4 rows (tile set-up,
@@ -667,7 +758,6 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
   I.source_rate = aq * wsum;
 
   // --- tiles and work items
-  int8_t cdx[kMaxUniChunks] = {0}, cdy[kMaxUniChunks] = {0};
   if (I.kind == RT_MESH_CARTESIAN) {
     if (variant < 0 || variant > 2) { set_error("variant must be 0, 1 or 2"); return RT_EINVAL; }
     // per-lane width first; the chunk-uniform variant is taken (automatically) when
@@ -681,21 +771,14 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
     }
     if (tile_x != 0 && tile_x != 16 && tile_x != 32) { set_error("tile_x must be 0, 16 or 32"); return RT_EINVAL; }
     I.run = 2;
-    // 32-cell strips (runs of 4 cells per warp) with chunk-uniform directions and
-    // 2 ordinates per lane: fewer face evaluations and shared-memory reads per
-    // cell, but twice the chunks of 4 ordinates per lane. Chosen automatically
-    // only when 4 ordinates per lane do not give uniform chunks (the 16-cell
-    // strips with 4 per lane measured faster where both apply), and only on
-    // grids of more than kWideMinCells cells: with 256 ordinates (quadrants of
-    // 64) the per-lane kernel measured faster on 70^2..280^2 grids (0.16 against
-    // 0.21 ms per step at 70^2, 0.31 against 0.34 at 280^2), the 32-cell strips
-    // on 560^2 (0.64 against 0.68) and 1400^2 (2.31 against 2.89).
+    // 32-cell tiles: asked for, or taken when whole chunks of 128 ordinates mix signs but
+    // chunks of 64 do not (256 ordinates), on grids of more than kWideMinCells cells.
     constexpr int64_t kWideMinCells = 100000;
     bool wide = false;
     if (variant != 1 && (vec == 0 || vec == 2) && tile_x != 16) {
-      const bool narrow4 = tile_x == 0 && vec == 0 && I.cvec >= 4 && chunks_uniform(quad, I.Mpad, 4, cdx, cdy);
+      const bool narrow4 = tile_x == 0 && vec == 0 && I.cvec >= 4 && chunks_uniform(quad, I.Mpad, 4);
       const bool small = tile_x == 0 && variant == 0 && vec == 0 && n_cells <= kWideMinCells;
-      wide = !narrow4 && !small && chunks_uniform(quad, I.Mpad, 2, cdx, cdy);
+      wide = !narrow4 && !small && chunks_uniform(quad, I.Mpad, 2);
     }
     if (wide) {
       I.uni = 1;
@@ -706,7 +789,7 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
       return RT_EINVAL;
     } else if (variant != 1) {
       for (int V = (variant == 2 && vec == 0 ? 4 : I.cvec); V >= 2; V /= 2) {
-        if (chunks_uniform(quad, I.Mpad, V, cdx, cdy)) {
+        if (chunks_uniform(quad, I.Mpad, V)) {
           I.uni = 1;
           I.cvec = V;
           break;
@@ -718,6 +801,33 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
         return RT_EINVAL;
       }
     }
+    // What the caller sees of the choice: chunk-uniform (2) or per-lane (1) directions.
+    // The streaming kernel runs both: always for chunk-uniform ones, and for per-lane
+    // ones unless a number of ordinates per lane was asked for (that is the general
+    // kernel's option; the streaming kernel always takes four, and vec reads 0). The
+    // general kernel is left for quadratures whose signs change too often for windows
+    // of 32: at 1000^2 x 128, where both run, it takes 0.84 ms per Heun step against
+    // 0.59, at 531^2 x 100 0.52 against 0.24, at 140^2 x 128 0.076 against 0.055.
+    I.info_variant = I.uni ? 2 : 1;
+    I.info_vec = I.cvec;
+    if (I.uni || vec == 0) I.str_chunks = plan_stream_chunks(quad, I.Mpad, storage);
+    if (!I.str_chunks.empty()) {
+      if (!I.uni) I.info_vec = 0;
+      I.uni = 1;
+      I.cvec = 4;
+      // one or two chunks (64 ordinates): a tile of 16 cells leaves half of a CTA's warps
+      // without a chunk, which costs less than larger tiles only on small grids
+      // (70^2 x 64 Heun: 35.4 us per step with 16, 38.5 with 32)
+      if (tile_x == 0 && I.run == 2 && I.str_chunks.size() <= 2) {
+        double narrow, wider;
+        stream_segment(I, 2, &narrow);
+        stream_segment(I, 4, &wider);
+        if (wider < narrow) I.run = 4;
+      }
+    } else {
+      I.uni = 0;
+      I.run = 2;
+    }
     choose_cart_tiles(I, tile_y);
     I.stage_items.clear();
     const int n = I.n_strips * I.n_segs;
@@ -728,7 +838,7 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
         I.stage_items.push_back(w);
       }
     const int stage_hi = integrator == RT_HEUN ? STAGE_HEUN2 : STAGE_EULER;
-    I.cart_smem = cart_smem_bytes(order, storage, I.run, I.cvec, I.ly, stage_hi);
+    I.cart_smem = cart_smem_bytes(order, storage, I.run, I.cvec, I.ly, stage_hi, I.uni);
     if (I.cart_smem > 227 * 1024) { set_error("tile %dx%d needs %zu bytes of shared memory", I.tx, I.ly, I.cart_smem); return RT_EINVAL; }
   } else {
     // persistent work items: item g processes 64-cell chunks g, g + G, ...; the
@@ -836,6 +946,14 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
     RT_CUDA_TRY(cudaMemcpyAsync(I.kmap, hm, ((size_t)I.M + I.Mpad) * sizeof(int32_t), cudaMemcpyHostToDevice, stream));
   }
 
+  int4* d_str_chunks = nullptr;
+  if (I.kind == RT_MESH_CARTESIAN && I.uni) {
+    const size_t bytes = I.str_chunks.size() * sizeof(int4);
+    if ((s = arena.get(bytes, &p)) != RT_OK) return s;
+    d_str_chunks = (int4*)p;
+    RT_CUDA_TRY(cudaMemcpyAsync(d_str_chunks, I.str_chunks.data(), bytes, cudaMemcpyHostToDevice, stream));
+  }
+
   uint8_t* d_mat = nullptr;
   uint8_t* d_reg = nullptr;
   int4* d_nbr = nullptr;
@@ -912,10 +1030,11 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
   InstDesc& D = I.desc;
   std::memset(&D, 0, sizeof(D));
   if (I.kind == RT_MESH_CARTESIAN) {
-    for (int b = 0; b < 2; ++b)
+    for (int b = 0; b < 2 && !I.uni; ++b)   // (the streaming kernel loads without tensor maps)
       if ((s = encode_psi_map(&D.tm_psi_halo[b], I.psi[b], storage, I.Mpad, I.nx, I.ny, 32 * I.cvec,
                               I.tx + 2 * order)) != RT_OK) return s;
-    if ((s = encode_psi_map(&D.tm_psi_center, I.psi[0], storage, I.Mpad, I.nx, I.ny, 32 * I.cvec, I.tx)) != RT_OK)
+    if (!I.uni &&
+        (s = encode_psi_map(&D.tm_psi_center, I.psi[0], storage, I.Mpad, I.nx, I.ny, 32 * I.cvec, I.tx)) != RT_OK)
       return s;
   }
   for (int b = 0; b < 2; ++b) { D.psi[b] = I.psi[b]; D.phi[b] = I.phi[b]; }
@@ -928,7 +1047,10 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
   D.st = I.st; D.partials = I.partials;
   D.kind = I.kind; D.order = order; D.integrator = integrator; D.storage = storage;
   D.nx = I.nx; D.ny = I.ny; D.M = I.M; D.Mpad = I.Mpad;
-  D.n_chunks = (I.kind == RT_MESH_CARTESIAN) ? I.Mpad / (32 * I.cvec) : I.Mpad / kChunk; D.tx = I.tx; D.ly = I.ly; D.n_strips = I.n_strips;
+  D.n_chunks = I.kind != RT_MESH_CARTESIAN ? I.Mpad / kChunk
+               : I.uni ? (int32_t)I.str_chunks.size() : I.Mpad / (32 * I.cvec);
+  D.str_chunks = d_str_chunks;
+  D.tx = I.tx; D.ly = I.ly; D.n_strips = I.n_strips;
   D.n_segs = I.n_segs; D.n_items = (int32_t)I.stage_items.size(); D.n_regions = I.n_regions;
   D.n_cells = n_cells; D.n_steps = I.n_steps;
   D.wait_limit = 4000000000LL;   // about two seconds of SM clock
@@ -941,11 +1063,6 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
   for (int sd = 0; sd < 4; ++sd) D.ghost[sd] = bc->side_kind[sd] == RT_BC_INFLOW ? (float)bc->inflow[sd] : 0.f;
   D.periodic_x = bc->side_kind[0] == RT_BC_PERIODIC ? 1 : 0;
   D.periodic_y = bc->side_kind[2] == RT_BC_PERIODIC ? 1 : 0;
-  D.uni = I.uni;
-  for (int c = 0; c < kMaxUniChunks; ++c) {
-    D.cdir_x[c] = cdx[c];
-    D.cdir_y[c] = cdy[c];
-  }
   for (int m = 0; m < kMaxMat; ++m) {
     const bool in = m < mat->n_mat;
     const double sa = in ? mat->sigma_a[m] : 0.0, ss = in ? mat->sigma_s[m] : 0.0, q = in ? mat->Q[m] : 0.0;

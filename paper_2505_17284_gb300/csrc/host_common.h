@@ -48,8 +48,10 @@ struct Instance {
   double dt = 0, t_end = 0;
   int64_t n_steps = 0;
   int32_t tx = 16, ly = 32, n_strips = 0, n_segs = 0;
-  int32_t run = 2, cvec = 1;        // Cartesian kernel: cells per thread, ordinates per lane
-  int32_t uni = 0;                  // Cartesian kernel: chunk-uniform flow directions; triangles (first
+  int32_t run = 2, cvec = 1;        // Cartesian kernels: tile width / 8, ordinates per lane
+  int32_t info_variant = 0, info_vec = 0;   // Cartesian: rt_info_t.variant and vec
+  std::vector<int4> str_chunks;     // streaming Cartesian kernel: its ordinate chunks
+  int32_t uni = 0;                  // Cartesian: 1 = streaming kernel (tile width 8 run); triangles (first
                                     // order): 1 = staged kernel (ly then holds the largest chunk halo)
   int32_t staged_ok = 0;            // triangles: the staged kernel's metadata exists (test hook switches)
   // ordinate layout: 0 the caller's order; 1 regrouped by direction quadrant,

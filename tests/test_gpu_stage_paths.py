@@ -50,3 +50,111 @@ def test_qoi_sums_of_many_regions(rt, kind, M, regions):
     assert abs(q["mass"] - S["mass"]) <= QOI_TOL * S["mass"]
     assert abs(q["outflow_now"] - S["outflow"]) <= QOI_TOL * max(abs(S["outflow"]), 1e-3 * S["mass"])
     assert abs(q["outflow_int"] - acc.outflow_int) <= QOI_TOL * max(abs(acc.outflow_int), 1e-3 * S["mass"])
+
+
+def cart_problem(nx, ny, seed, periodic=(False, False)):
+    """Random materials and regions on an nx x ny grid, inflow on every side (or periodic axes)."""
+    rng = np.random.default_rng(seed)
+    mesh = si.CartesianMesh(nx=nx, ny=ny, x0=0.0, y0=0.0, dx=0.1, dy=0.07)
+    mats = si.Materials(sigma_a=rng.uniform(0, 5, 4), sigma_s=rng.uniform(0, 3, 4), Q=rng.uniform(0, 1, 4),
+                        cell_mat=rng.integers(0, 4, nx * ny).astype(np.int32),
+                        cell_region=rng.integers(0, 3, nx * ny).astype(np.int32), region_names=("a", "b", "c"))
+    kind, inflow = [si.INFLOW] * 4, rng.uniform(0.2, 1.5, 4)
+    for axis in range(2):
+        if periodic[axis]:
+            kind[2 * axis] = kind[2 * axis + 1] = si.PERIODIC
+            inflow[2 * axis:2 * axis + 2] = 0.0
+    return si.Problem(mesh=mesh, materials=mats, boundary=si.Boundary(tuple(kind), tuple(inflow)), t_end=1.0)
+
+
+def quadratures(rt, name):
+    """Quadratures by how their directions change along the ordinates."""
+    kind, a = name.split("-")
+    if kind == "prod":
+        return rt.rt_quad_product(*[int(v) for v in a.split("x")])
+    if kind == "tess":
+        return rt.rt_quad_tessellation(int(a))
+    xi, eta, mu, w = rt.rt_quad_product(4, 16)
+    if kind == "axes":      # components that are exactly 0, at the runs' ends and inside them
+        xi, eta = xi.copy(), eta.copy()
+        xi[[0, 15, 20, 33]] = 0.0
+        eta[[3, 31, 32, 40]] = 0.0
+        xi[50], eta[50] = 0.0, 0.0
+    if kind == "shuffled":  # signs change from ordinate to ordinate
+        k = np.random.default_rng(int(a)).permutation(64)
+        xi, eta, mu, w = xi[k], eta[k], mu[k], w[k]
+    if kind == "first":     # a few ordinates only
+        xi, eta, mu, w = (v[:int(a)] for v in (xi, eta, mu, w))
+    return xi, eta, mu, w
+
+
+@pytest.mark.parametrize("quad", ["prod-4x16", "prod-8x16", "prod-2x16", "prod-3x12", "prod-8x32", "tess-3", "tess-5",
+                                  "tess-7", "tess-9", "axes-0", "shuffled-1", "first-1", "first-33"])
+@pytest.mark.parametrize("order,heun", [(1, False), (2, True), (1, True), (2, False)])
+def test_cartesian_stage_over_quadratures_and_ragged_tiles(rt, quad, order, heun):
+    """Every way the ordinates fall into windows (whole, partial, mixed signs of xi, or
+    none: the general kernel), on grids smaller than a tile, ragged in x and y, with
+    segments from one row up, inflow on all sides."""
+    q = quadratures(rt, quad)
+    for i, (nx, ny, ty) in enumerate([(1, 1, 0), (3, 2, 1), (9, 7, 2), (17, 11, 3), (37, 21, 0), (40, 33, 16)]):
+        p = cart_problem(nx, ny, seed=17 * i + order)
+        psi0 = si.random_psi(p.mesh.n_cells, len(q[0]), seed=i)
+        s = rt.Solver(p, q, order=order, integrator=rt.RT_HEUN if heun else rt.RT_EULER, dt=0.02, tile_y=ty)
+        s.set_psi(psi0)
+        s.step(3)
+        psi, qoi, dt = s.psi(), s.qoi(), s.info.dt
+        s.close()
+        op = oracle.CartesianOracle(p, q, order=order)
+        ref, acc, S = oracle.run(op, psi0, dt, 3, "heun" if heun else "euler")
+        assert rel_l2(psi, ref) <= PSI_TOL, (nx, ny)
+        assert abs(qoi["mass"] - S["mass"]) <= QOI_TOL * S["mass"], (nx, ny)
+        assert abs(qoi["outflow_int"] - acc.outflow_int) <= QOI_TOL * max(abs(acc.outflow_int), 1e-3 * S["mass"]), (nx, ny)
+
+
+@pytest.mark.parametrize("periodic", [(True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("quad", ["prod-4x16", "tess-5"])
+def test_cartesian_stage_partial_windows_on_periodic_sides(rt, quad, periodic):
+    q = quadratures(rt, quad)
+    for nx, ny, ty in ((5, 4, 1), (18, 13, 4)):
+        p = cart_problem(nx, ny, seed=5, periodic=periodic)
+        psi0 = si.random_psi(p.mesh.n_cells, len(q[0]), seed=2)
+        s = rt.Solver(p, q, order=2, integrator=rt.RT_HEUN, dt=0.02, tile_y=ty)
+        s.set_psi(psi0)
+        s.step(3)
+        psi, dt = s.psi(), s.info.dt
+        s.close()
+        ref, _, _ = oracle.run(oracle.CartesianOracle(p, q, order=2), psi0, dt, 3, "heun")
+        assert rel_l2(psi, ref) <= PSI_TOL, (nx, ny)
+
+
+@pytest.mark.parametrize("quad", ["prod-4x16", "prod-8x16", "tess-5"])
+def test_cartesian_stage_bf16_agrees_with_the_general_kernel(rt, quad):
+    """BF16 storage: the streaming kernel and the general one (an explicit number of
+    ordinates per lane) round with the same bits per (cell, ordinate, step, stage), so
+    after one Euler step nearly all stored values agree exactly, and both are within
+    BF16's unit roundoff (2^-8, stochastic rounding) of the oracle."""
+    q = quadratures(rt, quad)
+    p = cart_problem(37, 21, seed=3)
+    psi0 = si.random_psi(p.mesh.n_cells, len(q[0]), seed=4)
+    out = []
+    for vec in (0, 1):
+        s = rt.Solver(p, q, order=2, integrator=rt.RT_EULER, storage=rt.RT_BF16, dt=0.02, vec=vec)
+        s.set_psi(psi0)
+        start, dt = s.psi(), s.info.dt
+        s.step(1)
+        out.append(s.psi())
+        s.close()
+    ref, _, _ = oracle.run(oracle.CartesianOracle(p, q, order=2), start, dt, 1, "euler")
+    assert np.mean(out[0] == out[1]) >= 0.995
+    assert rel_l2(out[0], ref) <= 2.0 ** -8 and rel_l2(out[1], ref) <= 2.0 ** -8
+
+
+def test_dropped_load_of_the_streaming_kernel_is_reported(rt):
+    p = si.lattice_problem(35)
+    s = rt.Solver(p, rt.rt_quad_product(4, 16), order=2, integrator=rt.RT_HEUN, dt=0.1)
+    rt.rt_debug_set(s.h, "drop_load", 1)
+    s.step(1)
+    with pytest.raises(rt.RTError) as e:
+        s.qoi()
+    assert e.value.code == rt.RT_ETIMEOUT
+    s.close()
