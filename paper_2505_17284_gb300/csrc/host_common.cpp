@@ -166,7 +166,7 @@ static int64_t steps_for(double t_end, double dt_target) {
 struct TriMeta {
   std::vector<int4> nbr;
   std::vector<float4> geo;
-  std::vector<float4> geo2;   // second order: centroid-to-midpoint and centroid-to-neighbour vectors
+  std::vector<float4> geo2;   // second order: vectors to the edge midpoints from the centroid and from the neighbours'
   std::vector<double> area;
   double min_2a_over_p = 0;
 };
@@ -232,7 +232,7 @@ static rt_status triangle_metadata(const rt_mesh* m, const int32_t* cell_mat, co
     const int32_t a[3] = {T[3 * t], T[3 * t + 1], T[3 * t + 2]};
     const double A = out.area[t];
     int32_t nb[3];
-    float ax[3], ay[3], rx[3], ry[3], dx[3] = {0, 0, 0}, dy[3] = {0, 0, 0};
+    float ax[3], ay[3], rx[3], ry[3], sx[3] = {0, 0, 0}, sy[3] = {0, 0, 0};
     for (int e = 0; e < 3; ++e) {
       const int32_t p = a[e], q = a[(e + 1) % 3];
       const double px = V[2 * p], py = V[2 * p + 1], qx = V[2 * q], qy = V[2 * q + 1];
@@ -244,8 +244,8 @@ static rt_status triangle_metadata(const rt_mesh* m, const int32_t* cell_mat, co
       ry[e] = (float)(0.5 * (py + qy) - cen[2 * t + 1]);
       if (link[3 * t + e] >= 0) {
         nb[e] = link[3 * t + e];
-        dx[e] = (float)(cen[2 * (int64_t)nb[e]] - cen[2 * t]);
-        dy[e] = (float)(cen[2 * (int64_t)nb[e] + 1] - cen[2 * t + 1]);
+        sx[e] = (float)(0.5 * (px + qx) - cen[2 * (int64_t)nb[e]]);
+        sy[e] = (float)(0.5 * (py + qy) - cen[2 * (int64_t)nb[e] + 1]);
       } else {
         const double mx = 0.5 * (px + qx), my = 0.5 * (py + qy);
         const double dist[4] = {std::fabs(mx - xmin), std::fabs(mx - xmax), std::fabs(my - ymin), std::fabs(my - ymax)};
@@ -260,8 +260,8 @@ static rt_status triangle_metadata(const rt_mesh* m, const int32_t* cell_mat, co
     const double eps = A * A * A;   // the limiter's epsilon = K A^3 with K = 1
     out.geo[2 * t + 1] = float4{ax[2], ay[2], (float)A, (float)(eps * eps)};
     out.geo2[3 * t] = float4{rx[0], ry[0], rx[1], ry[1]};
-    out.geo2[3 * t + 1] = float4{rx[2], ry[2], dx[0], dy[0]};
-    out.geo2[3 * t + 2] = float4{dx[1], dy[1], dx[2], dy[2]};
+    out.geo2[3 * t + 1] = float4{rx[2], ry[2], sx[0], sy[0]};
+    out.geo2[3 * t + 2] = float4{sx[1], sy[1], sx[2], sy[2]};
   }
   return RT_OK;
 }
@@ -841,8 +841,8 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
     I.cart_smem = cart_smem_bytes(order, storage, I.run, I.cvec, I.ly, stage_hi, I.uni);
     if (I.cart_smem > 227 * 1024) { set_error("tile %dx%d needs %zu bytes of shared memory", I.tx, I.ly, I.cart_smem); return RT_EINVAL; }
   } else {
-    // persistent work items: item g processes 64-cell chunks g, g + G, ...; the
-    // staged first-order kernel runs two CTAs per SM, the others three
+    // persistent work items: item g processes chunks g, g + G, ..., with as many items
+    // as the kernel has CTAs resident
     const int64_t n_chunks = (n_cells + 63) / 64;
     if (order == 1) {
       build_chunk_halos(tm, n_cells, I, stg_halo_oc, stg_halo, stg_lidx);
@@ -854,7 +854,8 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
         stg_halo_oc.clear(); stg_halo.clear(); stg_lidx.clear();
       }
     }
-    const int G = (int)std::min<int64_t>(n_chunks, (I.uni ? 2LL : 3LL) * device_sm_count());
+    const int per_sm = I.uni ? 2 : (order == 2 ? tri2_ctas_per_sm(I.vec) : 3);
+    const int G = (int)std::min<int64_t>(n_chunks, (int64_t)per_sm * device_sm_count());
     I.stage_items.clear();
     for (int g = 0; g < G; ++g) {
       WorkItem w{};
@@ -1090,7 +1091,7 @@ rt_status launch_step(const InstDesc* d_desc, const WorkItem* d_items, int n_ite
     if (kind == RT_MESH_CARTESIAN)
       e = launch_cart_stage(d_desc, d_items, n_items, stages[i], order, storage, run, cvec, ly_max, stream, uni);
     else if (order == 2)
-      e = launch_tri2_stage(d_desc, d_items, n_items, stages[i], storage, std::min(vec, 2), vec, stream);
+      e = launch_tri2_stage(d_desc, d_items, n_items, stages[i], storage, vec, stream);
     else if (uni)
       e = launch_tri_staged(d_desc, d_items, n_items, stages[i], storage, vec, ly_max, stream);
     else

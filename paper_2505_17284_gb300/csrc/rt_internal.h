@@ -97,10 +97,11 @@ struct alignas(128) InstDesc {
   // normal)
   const int4* box_tasks;
   double* box_partials;         // [n_box_items][2 * kMaxBox]
-  int32_t n_boxes, n_box_tasks;  // triangles, second order: per cell {r0x, r0y, r1x, r1y}, {r2x, r2y, d0x, d0y},
-  // {d1x, d1y, d2x, d2y} (r_e: centroid to edge midpoint; d_e: centroid to the
-  // neighbour's centroid, 0 on the boundary), and the limited gradient L g,
-  // FP32 [cell][2][Mpad] (x row, then y row)
+  int32_t n_boxes, n_box_tasks;
+  // triangles, second order: per cell {r0x, r0y, r1x, r1y}, {r2x, r2y, s0x, s0y},
+  // {s1x, s1y, s2x, s2y} (r_e: centroid to edge midpoint; s_e: the neighbour's
+  // centroid to the same midpoint, 0 on the boundary), and the limited gradient
+  // L g, FP32 [cell][2][Mpad] (x row, then y row)
   const float4* tri_geo2;
   float* tri_lg;
   int32_t periodic_x;           // Cartesian: 1 if the x- and x+ sides are periodic (no boundary faces in x)
@@ -147,10 +148,11 @@ cudaError_t prepare_tri_staged(int stage, int storage, int vec, int hmax);
 size_t tri_staged_smem_bytes(int vec, int storage, int hmax, int stage);
 cudaError_t launch_init(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int vec,
                         int storage, cudaStream_t stream);
-// Second-order triangle stage: the limited-gradient kernel (grad_vec ordinates
-// per lane: 1, 2 or 4), then the stage kernel (vec 1 or 2).
-cudaError_t launch_tri2_stage(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage,
-                              int storage, int vec, int grad_vec, cudaStream_t stream);
+// Second-order triangle stage: the limited-gradient kernel, then the stage kernel, both
+// persistent with tri2_ctas_per_sm(vec) CTAs per SM (vec ordinates per lane: 1, 2 or 4).
+cudaError_t launch_tri2_stage(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage, int storage,
+                              int vec, cudaStream_t s);
+int tri2_ctas_per_sm(int vec);
 // Outflow through the QoI boxes after a time step (stage = STAGE_EULER, or
 // STAGE_HEUN2 after a whole Heun step) with the step's time-integration
 // update, or of the current state (STAGE_INIT). Work items: a = first face,

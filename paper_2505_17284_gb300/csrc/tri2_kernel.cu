@@ -10,15 +10,25 @@
 //
 // Two kernels per stage, both persistent over 64-cell chunks like the
 // first-order stage kernel (chunk metadata staged in shared memory by bulk
-// copies, one warp per cell, lanes over ordinates; 3 CTAs per SM, so the
-// 3-per-SM persistent grid is resident at once):
+// copies, one warp per cell, lanes over ordinates, FP32 pairs; the grid has
+// as many CTAs as are resident at once; a warp fetches the rows of its next
+// cell to L2 while it works on one, since only neighbours' rows are there
+// already):
 //   tri_grad_kernel    reads psi of a cell and its three neighbours and writes
 //                      the limited gradient L g (two FP32 rows per cell);
 //   tri_stage2_kernel  reads psi and L g of a cell and its neighbours, takes
 //                      the upwind reconstructed trace on each edge (the
-//                      neighbour's R at the shared midpoint, r_je = r_ie - d_ij
-//                      with d_ij = x_j - x_i) and writes the stage output, phi
+//                      neighbour's R at the shared midpoint) and writes the
+//                      stage output, phi
 //                      and the FP64 QoI partials as the first-order kernel does.
+//
+// Bound by the latency of the gathers (24 warps per SM in the gradient pass, 16 in
+// the stage pass; DRAM at 45 - 48 % of its peak, issue slots at 62 and 47 %). Differences
+// to the cell's value, not values, are summed over the edges: the sums of the normals
+// vanish, and the rounding error is smaller (650^2 x 256, one step against FP64: 4.22e-8
+// of psi, 4.33e-8 with values). At 400^2 x 256 (FP32), with IEEE divisions in divergent
+// branches and 2 ordinates per lane in the stage pass: gradient 0.82 ms, stage 0.45 ms;
+// now 0.27 and 0.35 ms. A Heun step at 650^2 x 256: 6.65 -> 3.29 ms.
 #include <cuda_bf16.h>
 
 #include "device_common.cuh"
@@ -29,6 +39,10 @@ namespace {
 
 constexpr int kT2Threads = 256;
 constexpr int kT2Warps = kT2Threads / 32;
+// With 4 ordinates per lane the stage pass needs 128 registers (two CTAs per SM); the
+// gradient pass needs 80, and takes 12 warps per CTA then, so that its two hold 24.
+constexpr int t2_ctas(int vec) { return vec == 4 ? 2 : 3; }
+constexpr int t2_grad_threads(int vec) { return vec == 4 ? 384 : 256; }
 constexpr int kT2Chunk = 64;
 constexpr uint32_t kT2MetaBytes = 16u + 32u + 48u;   // per cell: neighbours, geometry, second-order geometry
 
@@ -73,13 +87,78 @@ __device__ __forceinline__ float ghost_value(const InstDesc& d, int s, float xi,
 }
 
 // Venkatakrishnan value of one edge (Eq. V_limiter with the 1/Delta factor
-// cancelled): 1 for Delta = 0 (and for a vanishing denominator)
-__device__ __forceinline__ float venkat(float delta, float bmax, float bmin, float eps2) {
-  if (delta == 0.f) return 1.f;
-  const float b = delta > 0.f ? bmax : bmin;
-  const float num = b * b + eps2 + 2.f * delta * b;
-  const float den = b * b + 2.f * delta * delta + b * delta + eps2;
-  return den > 0.f ? num / den : 1.f;
+// cancelled), from x = |Delta| and y = |beta| on Delta's side: with p = x y and
+// c = y^2 + eps^2 + p it is (c + p) / (c + 2 x^2), and 1 where that is 0 / 0.
+__device__ __forceinline__ float venkat_exact(float x, float y, float eps2) {
+  const float p = x * y, c = fmaf(y, y, eps2) + p;
+  const float den = fmaf(x + x, x, c);
+  return den > 0.f ? (c + p) / den : 1.f;
+}
+
+__device__ __forceinline__ float fmin3f(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float fmax3f(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
+// L and L g of one value given its gradient and the spread of its neighbourhood. The
+// quotients are formed with __fdividef (2 ulp, where the denominators lie inside its
+// range; otherwise, for values below 1e-15 or above 1e18 of the state's unit, by IEEE
+// division): three IEEE divisions in divergent branches were 200 of 269 instructions
+// per cell and ordinate.
+__device__ __forceinline__ float limiter(const float (&x)[3], const float (&y)[3], const float (&num)[3],
+                                         const float (&den)[3], float eps2) {
+  const float lo = fmin3f(den[0], den[1], den[2]), hi = fmax3f(den[0], den[1], den[2]);
+  if (lo >= 1e-30f && hi <= 1e36f)
+    return fmin3f(__fdividef(num[0], den[0]), __fdividef(num[1], den[1]), __fdividef(num[2], den[2]));
+  return fminf(fminf(venkat_exact(x[0], y[0], eps2), venkat_exact(x[1], y[1], eps2)), venkat_exact(x[2], y[2], eps2));
+}
+
+// Limited gradient L g of a pair of ordinates from the cell's values c and its
+// neighbours' n0, n1, n2 (FP32 pairs: two values per instruction). The normals of a
+// triangle sum to zero, so the Green-Gauss sum of l n (c + n_e)/2 is that of
+// l n (n_e - c)/2, whose rounding error scales with the differences, not the values.
+__device__ __forceinline__ void limited_gradient2(float2 c, float2 n0, float2 n1, float2 n2, const float (&axh)[3],
+                                                  const float (&ayh)[3], const float (&rxh)[3], const float (&ryh)[3],
+                                                  float eps2, float2& lx, float2& ly) {
+  auto dup = [](float a) { return make_float2(a, a); };
+  const float2 mc = make_float2(-c.x, -c.y);
+  const float2 s0 = __fadd2_rn(n0, mc), s1 = __fadd2_rn(n1, mc), s2 = __fadd2_rn(n2, mc);
+  const float2 gx = __ffma2_rn(dup(axh[2]), s2, __ffma2_rn(dup(axh[1]), s1, __fmul2_rn(dup(axh[0]), s0)));
+  const float2 gy = __ffma2_rn(dup(ayh[2]), s2, __ffma2_rn(dup(ayh[1]), s1, __fmul2_rn(dup(ayh[0]), s0)));
+  // beta_max and -beta_min
+  const float2 up = make_float2(fmaxf(fmax3f(s0.x, s1.x, s2.x), 0.f), fmaxf(fmax3f(s0.y, s1.y, s2.y), 0.f));
+  const float2 dn = make_float2(-fminf(fmin3f(s0.x, s1.x, s2.x), 0.f), -fminf(fmin3f(s0.y, s1.y, s2.y), 0.f));
+  float xa[3], ya[3], na[3], da[3], xb[3], yb[3], nb[3], db[3];
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    const float2 D = __ffma2_rn(dup(ryh[e]), gy, __fmul2_rn(dup(rxh[e]), gx));
+    const float2 x = make_float2(fabsf(D.x), fabsf(D.y));
+    const float2 y = make_float2(D.x > 0.f ? up.x : dn.x, D.y > 0.f ? up.y : dn.y);
+    const float2 p = __fmul2_rn(x, y);
+    const float2 q = __fadd2_rn(__ffma2_rn(y, y, dup(eps2)), p);
+    const float2 n = __fadd2_rn(q, p), d = __ffma2_rn(__fadd2_rn(x, x), x, q);
+    xa[e] = x.x; ya[e] = y.x; na[e] = n.x; da[e] = d.x;
+    xb[e] = x.y; yb[e] = y.y; nb[e] = n.y; db[e] = d.y;
+  }
+  const float2 L = make_float2(limiter(xa, ya, na, da, eps2), limiter(xb, yb, nb, db, eps2));
+  lx = __fmul2_rn(L, gx);
+  ly = __fmul2_rn(L, gy);
+}
+
+// Fetch the rows of a cell to L2, a 128-byte line per lane at a time: na lines at a,
+// nb at b, and the rest at c.
+__device__ __forceinline__ void prefetch_lines(const void* a, int na, const void* b, int nb, const void* c, int nc) {
+  for (int o = threadIdx.x & 31; o < na + nb + nc; o += 32) {
+    const char* p = reinterpret_cast<const char*>(o < na ? a : (o < na + nb ? b : c));
+    const int q = o < na ? o : (o < na + nb ? o - na : o - na - nb);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 128 * q));
+  }
 }
 
 // Chunk metadata in shared memory, double-buffered.
@@ -101,8 +180,9 @@ __device__ __forceinline__ void t2_stage_meta(const InstDesc& d, T2Meta& m, int 
 
 // -------------------------------------------------------------------- gradient
 template <int VEC, typename T>
-__global__ void __launch_bounds__(kT2Threads, 3)
+__global__ void __launch_bounds__(t2_grad_threads(VEC), t2_ctas(VEC))
     tri_grad_kernel(const InstDesc* __restrict__ descs, const WorkItem* __restrict__ items, int stage) {
+  constexpr int kGradWarps = t2_grad_threads(VEC) / 32;
   __shared__ __align__(16) T2Meta meta;
   const WorkItem it = items[blockIdx.x];
   const InstDesc& d = descs[it.inst];
@@ -114,6 +194,7 @@ __global__ void __launch_bounds__(kT2Threads, 3)
   float* __restrict__ lg = d.tri_lg;
   const int Mpad = d.Mpad;
   const int nv = Mpad / (32 * VEC);
+  const int psi_lines = (Mpad * (int)sizeof(T) + 127) / 128;
   const int n_cells = (int)d.n_cells;
   const int n_chunks = (n_cells + kT2Chunk - 1) / kT2Chunk;
   const int G = it.b;
@@ -137,49 +218,65 @@ __global__ void __launch_bounds__(kT2Threads, 3)
     }
     const int c0 = k * kT2Chunk;
     const int c_end = min(n_cells, c0 + kT2Chunk);
-    for (int cell = c0 + warp; cell < c_end; cell += kT2Warps) {
+    for (int cell = c0 + warp; cell < c_end; cell += kGradWarps) {
       const int li = cell - c0;
       const int4 nb = meta.nbr[b][li];
       const float4 g0 = meta.geo[b][2 * li], g1 = meta.geo[b][2 * li + 1];
       const float4 h0 = meta.geo2[b][3 * li], h1 = meta.geo2[b][3 * li + 1];
-      const float ax[3] = {g0.x, g0.z, g1.x}, ay[3] = {g0.y, g0.w, g1.y};
-      const float rx[3] = {h0.x, h0.z, h1.x}, ry[3] = {h0.y, h0.w, h1.y};
+      // halves: of the face average in the gradient, and of Delta = (1/2) g . r
+      const float axh[3] = {0.5f * g0.x, 0.5f * g0.z, 0.5f * g1.x}, ayh[3] = {0.5f * g0.y, 0.5f * g0.w, 0.5f * g1.y};
+      const float rxh[3] = {0.5f * h0.x, 0.5f * h0.z, 0.5f * h1.x}, ryh[3] = {0.5f * h0.y, 0.5f * h0.w, 0.5f * h1.y};
       const float eps2 = g1.w;
       const int nbr[3] = {nb.x, nb.y, nb.z};
+      const bool has_bnd = (nbr[0] < 0) | (nbr[1] < 0) | (nbr[2] < 0);
+      {
+        const int64_t nc = cell + kGradWarps < c_end ? cell + kGradWarps : (int64_t)(k + G) * kT2Chunk + warp;
+        if (nc < n_cells) prefetch_lines(psi + (size_t)nc * Mpad, psi_lines, nullptr, 0, nullptr, 0);
+      }
+      const T* row_c = psi + (size_t)cell * Mpad + lane * VEC;
+      const T* row_n[3];
+#pragma unroll
+      for (int e = 0; e < 3; ++e) row_n[e] = psi + (size_t)(nbr[e] >= 0 ? nbr[e] : cell) * Mpad + lane * VEC;
+      float* row_g = lg + (size_t)cell * 2 * Mpad + lane * VEC;
       for (int v = 0; v < nv; ++v) {
-        const int kk = (v * 32 + lane) * VEC;
-        float c[VEC], nv3[3][VEC];
-        ld_vec<T, VEC>(psi + (size_t)cell * Mpad + kk, c);
+        float c[VEC], nb3[3][VEC], ox[VEC], oy[VEC];
+        ld_vec<T, VEC>(row_c, c);
 #pragma unroll
-        for (int e = 0; e < 3; ++e)
-          if (nbr[e] >= 0) ld_vec<T, VEC>(psi + (size_t)nbr[e] * Mpad + kk, nv3[e]);
-        float xi[VEC], eta[VEC];
-        ld_vec<float, VEC>(d.xi + kk, xi);
-        ld_vec<float, VEC>(d.eta + kk, eta);
-        float ox[VEC], oy[VEC];
+        for (int e = 0; e < 3; ++e) ld_vec<T, VEC>(row_n[e], nb3[e]);
+        if (has_bnd) {
+          const int kk = (v * 32 + lane) * VEC;
 #pragma unroll
-        for (int l = 0; l < VEC; ++l) {
-          float nbv[3];
+          for (int e = 0; e < 3; ++e)
+            if (nbr[e] < 0) {
 #pragma unroll
-          for (int e = 0; e < 3; ++e) nbv[e] = (nbr[e] >= 0) ? nv3[e][l] : ghost_value(d, -1 - nbr[e], xi[l], eta[l]);
-          float gx = 0.f, gy = 0.f;
-#pragma unroll
-          for (int e = 0; e < 3; ++e) {
-            const float avg = 0.5f * (c[l] + nbv[e]);
-            gx = fmaf(ax[e], avg, gx);
-            gy = fmaf(ay[e], avg, gy);
-          }
-          const float pmax = fmaxf(fmaxf(c[l], nbv[0]), fmaxf(nbv[1], nbv[2]));
-          const float pmin = fminf(fminf(c[l], nbv[0]), fminf(nbv[1], nbv[2]));
-          const float bmax = pmax - c[l], bmin = pmin - c[l];
-          float L = INFINITY;
-#pragma unroll
-          for (int e = 0; e < 3; ++e) L = fminf(L, venkat(0.5f * (gx * rx[e] + gy * ry[e]), bmax, bmin, eps2));
-          ox[l] = L * gx;
-          oy[l] = L * gy;
+              for (int l = 0; l < VEC; ++l) nb3[e][l] = ghost_value(d, -1 - nbr[e], d.xi[kk + l], d.eta[kk + l]);
+            }
         }
-        st_vec<float, VEC>(lg + (size_t)cell * 2 * Mpad + kk, ox);
-        st_vec<float, VEC>(lg + (size_t)cell * 2 * Mpad + Mpad + kk, oy);
+        if constexpr (VEC >= 2) {
+#pragma unroll
+          for (int l = 0; l < VEC; l += 2) {
+            float2 gx, gy;
+            limited_gradient2(make_float2(c[l], c[l + 1]), make_float2(nb3[0][l], nb3[0][l + 1]),
+                              make_float2(nb3[1][l], nb3[1][l + 1]), make_float2(nb3[2][l], nb3[2][l + 1]), axh, ayh, rxh,
+                              ryh, eps2, gx, gy);
+            ox[l] = gx.x;
+            ox[l + 1] = gx.y;
+            oy[l] = gy.x;
+            oy[l + 1] = gy.y;
+          }
+        } else {
+          float2 gx, gy;   // the pair's second value is not used
+          limited_gradient2(make_float2(c[0], c[0]), make_float2(nb3[0][0], nb3[0][0]), make_float2(nb3[1][0], nb3[1][0]),
+                            make_float2(nb3[2][0], nb3[2][0]), axh, ayh, rxh, ryh, eps2, gx, gy);
+          ox[0] = gx.x;
+          oy[0] = gy.x;
+        }
+        st_vec<float, VEC>(row_g, ox);
+        st_vec<float, VEC>(row_g + Mpad, oy);
+        row_c += 32 * VEC;
+        row_g += 32 * VEC;
+#pragma unroll
+        for (int e = 0; e < 3; ++e) row_n[e] += 32 * VEC;
       }
     }
     __syncthreads();
@@ -197,7 +294,7 @@ __global__ void __launch_bounds__(kT2Threads, 3)
 
 // -------------------------------------------------------------------- stage
 template <int VEC, int STAGE, typename T>
-__global__ void __launch_bounds__(kT2Threads, 3)
+__global__ void __launch_bounds__(kT2Threads, t2_ctas(VEC))
     tri_stage2_kernel(const InstDesc* __restrict__ descs, const WorkItem* __restrict__ items) {
   __shared__ __align__(16) T2Meta meta;
   __shared__ double red[(kT2Warps + 1) * NQ];
@@ -217,10 +314,14 @@ __global__ void __launch_bounds__(kT2Threads, 3)
   const T* __restrict__ psi_base = reinterpret_cast<const T*>(d.psi[0]);
   T* __restrict__ psi_out = reinterpret_cast<T*>(d.psi[out_buf]);
   const float* __restrict__ lg = d.tri_lg;
+  const float* __restrict__ d_xi = d.xi;
+  const float* __restrict__ d_eta = d.eta;
+  const float* __restrict__ d_w = d.w;
   const float* __restrict__ phi_in = d.phi[in_buf];
   float* __restrict__ phi_out = d.phi[out_buf];
   const int Mpad = d.Mpad;
   const int nv = Mpad / (32 * VEC);
+  const int psi_lines = (Mpad * (int)sizeof(T) + 127) / 128;
   const float dt = d.dt;
   const int nreg = d.n_regions, nq = nreg + 2;
   const int n_cells = (int)d.n_cells;
@@ -258,88 +359,119 @@ __global__ void __launch_bounds__(kT2Threads, 3)
       const float4 g0 = meta.geo[b][2 * li], g1 = meta.geo[b][2 * li + 1];
       const float4 h0 = meta.geo2[b][3 * li], h1 = meta.geo2[b][3 * li + 1], h2 = meta.geo2[b][3 * li + 2];
       const float ax[3] = {g0.x, g0.z, g1.x}, ay[3] = {g0.y, g0.w, g1.y};
-      const float rx[3] = {h0.x, h0.z, h1.x}, ry[3] = {h0.y, h0.w, h1.y};
-      // r_je = r_ie - d_ij: the neighbour's centroid-to-midpoint vector of the shared edge
-      const float sx[3] = {rx[0] - h1.z, rx[1] - h2.x, rx[2] - h2.z};
-      const float sy[3] = {ry[0] - h1.w, ry[1] - h2.y, ry[2] - h2.w};
+      float rx[3] = {h0.x, h0.z, h1.x}, ry[3] = {h0.y, h0.w, h1.y};
+      // the neighbour's centroid-to-midpoint vector of the shared edge
+      float sx[3] = {h1.z, h2.x, h2.z}, sy[3] = {h1.w, h2.y, h2.w};
       const int nbr[3] = {nb.x, nb.y, nb.z};
       const int m = nb.w & 255, reg = (nb.w >> 8) & 255;
       const float area = g1.z;
       const float sig_t = d.sig_t[m];
-      const float phin = phi_in[cell];
-      const float src = d.sig_s2pi[m] * phin + d.q_src[m];
+      const float src = d.sig_s2pi[m] * phi_in[cell] + d.q_src[m];
       const bool has_bnd = (nbr[0] < 0) | (nbr[1] < 0) | (nbr[2] < 0);
+      {
+        // the rows of the warp's next cell: their first use goes to DRAM, the neighbours' mostly to L2
+        const int64_t nc = cell + kT2Warps < c_end ? cell + kT2Warps : (int64_t)(k + G) * kT2Chunk + warp;
+        if (nc < n_cells)
+          prefetch_lines(psi_in + (size_t)nc * Mpad, psi_lines, lg + (size_t)nc * 2 * Mpad, Mpad / 16,
+                         psi_base + (size_t)nc * Mpad, STAGE == STAGE_HEUN2 ? psi_lines : 0);
+      }
+      // the lane's pieces of the rows: its own, and per edge the neighbour's (psi, then L g in x and y)
+      const T* row_c = psi_in + (size_t)cell * Mpad + lane * VEC;
+      const float* row_g = lg + (size_t)cell * 2 * Mpad + lane * VEC;
+      const T* nrow[3];
+      const float* ngrow[3];
       float gh[3];
 #pragma unroll
-      for (int e = 0; e < 3; ++e) gh[e] = (nbr[e] < 0) ? d.ghost[-1 - nbr[e]] : 0.f;
+      for (int e = 0; e < 3; ++e) {
+        const size_t j = nbr[e] >= 0 ? nbr[e] : cell;   // (a boundary edge reads its own cell's, unused)
+        nrow[e] = psi_in + j * Mpad + lane * VEC;
+        ngrow[e] = lg + j * 2 * Mpad + lane * VEC;
+        gh[e] = 0.f;
+        if (nbr[e] < 0) {   // first order on the boundary: the traces are the cell value and psi^-
+          gh[e] = d.ghost[-1 - nbr[e]];
+          rx[e] = ry[e] = sx[e] = sy[e] = 0.f;
+        }
+      }
 
       float phi_part = 0.f, bpart = 0.f;
       for (int v = 0; v < nv; ++v) {
         const int kk = (v * 32 + lane) * VEC;
-        float c[VEC], cx[VEC], cy[VEC], base[VEC];
-        float nbv[3][VEC], nx[3][VEC], ny[3][VEC];
-        ld_vec<T, VEC>(psi_in + (size_t)cell * Mpad + kk, c);
-        ld_vec<float, VEC>(lg + (size_t)cell * 2 * Mpad + kk, cx);
-        ld_vec<float, VEC>(lg + (size_t)cell * 2 * Mpad + Mpad + kk, cy);
+        float c[VEC], cx[VEC], cy[VEC], nbv[3][VEC], nx[3][VEC], ny[3][VEC];
+        [[maybe_unused]] float base[VEC];
+        ld_vec<T, VEC>(row_c, c);
+        ld_vec<float, VEC>(row_g, cx);
+        ld_vec<float, VEC>(row_g + Mpad, cy);
 #pragma unroll
         for (int e = 0; e < 3; ++e) {
-          if (nbr[e] >= 0) {
-            ld_vec<T, VEC>(psi_in + (size_t)nbr[e] * Mpad + kk, nbv[e]);
-            ld_vec<float, VEC>(lg + (size_t)nbr[e] * 2 * Mpad + kk, nx[e]);
-            ld_vec<float, VEC>(lg + (size_t)nbr[e] * 2 * Mpad + Mpad + kk, ny[e]);
-          } else {
-#pragma unroll
-            for (int l = 0; l < VEC; ++l) nbv[e][l] = nx[e][l] = ny[e][l] = 0.f;
-          }
+          ld_vec<T, VEC>(nrow[e], nbv[e]);
+          ld_vec<float, VEC>(ngrow[e], nx[e]);
+          ld_vec<float, VEC>(ngrow[e] + Mpad, ny[e]);
+          nrow[e] += 32 * VEC;
+          ngrow[e] += 32 * VEC;
         }
-        if constexpr (STAGE == STAGE_HEUN2) ld_vec<T, VEC>(psi_base + (size_t)cell * Mpad + kk, base);
+        if constexpr (STAGE == STAGE_HEUN2) ld_vec<T, VEC>(psi_base + (row_c - psi_in), base);
+        row_c += 32 * VEC;
+        row_g += 32 * VEC;
+        if (has_bnd) {
+#pragma unroll
+          for (int e = 0; e < 3; ++e)
+            if (nbr[e] < 0) {
+#pragma unroll
+              for (int l = 0; l < VEC; ++l) nbv[e][l] = gh[e];
+            }
+        }
         float xi[VEC], eta[VEC], w[VEC], out[VEC];
-        ld_vec<float, VEC>(d.xi + kk, xi);
-        ld_vec<float, VEC>(d.eta + kk, eta);
-        ld_vec<float, VEC>(d.w + kk, w);
+        ld_vec<float, VEC>(d_xi + kk, xi);
+        ld_vec<float, VEC>(d_eta + kk, eta);
+        ld_vec<float, VEC>(d_w + kk, w);
         // BF16 rounding bits of the lane's ordinates kk .. kk+VEC-1 (one group of four)
         [[maybe_unused]] uint2 rb4;
         if constexpr (sizeof(T) == 2) rb4 = sr_bits4((uint32_t)cell, sr_gkey(kk >> 2, salt));
+        // ordinate pairs (two FP32 values per instruction); a single ordinate is a pair of itself
 #pragma unroll
-        for (int l = 0; l < VEC; ++l) {
-          float div = 0.f;
+        for (int l = 0; l < VEC; l += 2) {
+          const int l1 = VEC > 1 ? l + 1 : l;
+          auto pair = [&](const float (&a)[VEC]) { return make_float2(a[l], a[l1]); };
+          auto dup = [](float a) { return make_float2(a, a); };
+          const float2 c2 = pair(c), xi2 = pair(xi), eta2 = pair(eta), cx2 = pair(cx), cy2 = pair(cy);
+          // traces less the cell's value: omega . n l / A sums to zero over the edges
+          const float2 mc2 = make_float2(-c2.x, -c2.y);
+          float2 div = make_float2(0.f, 0.f);
 #pragma unroll
           for (int e = 0; e < 3; ++e) {
-            const float on = xi[l] * ax[e] + eta[l] * ay[e];
-            float tr;
-            if (nbr[e] < 0) {
-              tr = (on > 0.f) ? c[l] : gh[e];   // first order on the boundary
-            } else if (on > 0.f) {
-              tr = fmaf(cx[l], rx[e], fmaf(cy[l], ry[e], c[l]));
-            } else {
-              tr = fmaf(nx[e][l], sx[e], fmaf(ny[e][l], sy[e], nbv[e][l]));
-            }
-            div = fmaf(on, tr, div);
+            const float2 on = __ffma2_rn(eta2, dup(ay[e]), __fmul2_rn(xi2, dup(ax[e])));
+            const float2 mine = __ffma2_rn(cx2, dup(rx[e]), __fmul2_rn(cy2, dup(ry[e])));
+            const float2 other = __ffma2_rn(pair(nx[e]), dup(sx[e]),
+                                            __ffma2_rn(pair(ny[e]), dup(sy[e]), __fadd2_rn(pair(nbv[e]), mc2)));
+            div = __ffma2_rn(on, make_float2(on.x > 0.f ? mine.x : other.x, on.y > 0.f ? mine.y : other.y), div);
           }
-          const float F = -div - sig_t * c[l] + src;
-          float o;
+          const float2 F = __fadd2_rn(__ffma2_rn(dup(-sig_t), c2, make_float2(-div.x, -div.y)), dup(src));
+          float2 o;
           if constexpr (STAGE == STAGE_HEUN2) {
-            o = 0.5f * (base[l] + c[l] + dt * F);
+            o = __fmul2_rn(dup(0.5f), __ffma2_rn(dup(dt), F, __fadd2_rn(pair(base), c2)));
           } else {
-            o = c[l] + dt * F;
+            o = __ffma2_rn(dup(dt), F, c2);
           }
           if constexpr (sizeof(T) == 2) {
-            const int ko = kk + l;
-            o = Store<T>::round_sr(o, sr_elem(rb4, ko & 3));
+            o.x = Store<T>::round_sr(o.x, sr_elem(rb4, (kk + l) & 3));
+            o.y = Store<T>::round_sr(o.y, sr_elem(rb4, (kk + l1) & 3));
           }
-          out[l] = o;
-          phi_part += w[l] * o;
-          if (has_bnd) {
-#pragma unroll
-            for (int e = 0; e < 3; ++e) {
-              if (nbr[e] < 0) {
-                const float on = xi[l] * ax[e] + eta[l] * ay[e];
-                bpart += w[l] * on * ((on > 0.f) ? o : gh[e]);
-              }
-            }
-          }
+          out[l] = o.x;
+          if constexpr (VEC > 1) out[l1] = o.y;
         }
         st_vec<T, VEC>(psi_out + (size_t)cell * Mpad + kk, out);
+#pragma unroll
+        for (int l = 0; l < VEC; ++l) {
+          phi_part = fmaf(w[l], out[l], phi_part);
+          if (has_bnd) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e)
+              if (nbr[e] < 0) {
+                const float on = xi[l] * ax[e] + eta[l] * ay[e];
+                bpart += w[l] * on * ((on > 0.f) ? out[l] : gh[e]);
+              }
+          }
+        }
       }
       const float ph = warp_sum(phi_part);
       float bsum = 0.f;
@@ -384,15 +516,14 @@ __global__ void __launch_bounds__(kT2Threads, 3)
 
 }  // namespace
 
+int tri2_ctas_per_sm(int vec) { return t2_ctas(vec); }
+
 cudaError_t launch_tri2_stage(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage, int storage,
-                              int vec, int grad_vec, cudaStream_t s) {
+                              int vec, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
-  // the gradient pass takes 4 ordinates per lane where the quadrature allows
-  // (fewer, wider loads); the stage pass at most 2 (its registers)
 #define RTK_T2(V, ST, TT)                                                                       \
   if (vec == V && stage == ST) {                                                                \
-    if (grad_vec == 4) tri_grad_kernel<4, TT><<<n_items, kT2Threads, 0, s>>>(d_desc, d_items, ST); \
-    else tri_grad_kernel<V, TT><<<n_items, kT2Threads, 0, s>>>(d_desc, d_items, ST);            \
+    tri_grad_kernel<V, TT><<<n_items, t2_grad_threads(V), 0, s>>>(d_desc, d_items, ST);         \
     cudaError_t e = cudaGetLastError();                                                         \
     if (e != cudaSuccess) return e;                                                             \
     tri_stage2_kernel<V, ST, TT><<<n_items, kT2Threads, 0, s>>>(d_desc, d_items);               \
@@ -400,7 +531,8 @@ cudaError_t launch_tri2_stage(const InstDesc* d_desc, const WorkItem* d_items, i
   }
 #define RTK_T2_ALL(TT)                                                                          \
   RTK_T2(1, STAGE_EULER, TT) RTK_T2(1, STAGE_HEUN1, TT) RTK_T2(1, STAGE_HEUN2, TT)              \
-  RTK_T2(2, STAGE_EULER, TT) RTK_T2(2, STAGE_HEUN1, TT) RTK_T2(2, STAGE_HEUN2, TT)
+  RTK_T2(2, STAGE_EULER, TT) RTK_T2(2, STAGE_HEUN1, TT) RTK_T2(2, STAGE_HEUN2, TT)              \
+  RTK_T2(4, STAGE_EULER, TT) RTK_T2(4, STAGE_HEUN1, TT) RTK_T2(4, STAGE_HEUN2, TT)
   if (storage == 0) { RTK_T2_ALL(float) } else { RTK_T2_ALL(__nv_bfloat16) }
 #undef RTK_T2_ALL
 #undef RTK_T2

@@ -158,3 +158,26 @@ def test_dropped_load_of_the_streaming_kernel_is_reported(rt):
         s.qoi()
     assert e.value.code == rt.RT_ETIMEOUT
     s.close()
+
+
+@pytest.mark.parametrize("M", [(2, 16), (4, 16), (6, 16), (8, 16)])   # 1, 2, 1 and 4 ordinates per lane
+@pytest.mark.parametrize("scale", [1e-16, 1e-9, 1.0, 1e18])
+def test_second_order_triangles_over_scales_of_the_state(rt, M, scale):
+    """The limiter divides with a fast quotient inside its range and by IEEE division
+    outside it (states below 1e-15 or above 1e18): the scheme is homogeneous in the
+    state and source, so every scale must match the oracle alike."""
+    mesh = si.split_grid_mesh(13, 0.01, jitter=0.2, seed=4)   # cells so small that epsilon^2 is far below beta^2
+    n = mesh.n_cells
+    mats = si.Materials(sigma_a=np.array([1.0, 40.0]), sigma_s=np.array([20.0, 3.0]), Q=np.array([0.5, 30.0]) * scale,
+                        cell_mat=(np.arange(n) // 5 % 2).astype(np.int32), cell_region=np.zeros(n, np.int32),
+                        region_names=("all",))
+    p = si.Problem(mesh=mesh, materials=mats, boundary=si.Boundary(), t_end=1.0)
+    psi0 = (si.smooth_psi(mesh, M[0] * M[1], seed=2) + 0.2 * si.random_psi(n, M[0] * M[1], seed=3)) * scale
+    s = rt.Solver(p, rt.rt_quad_product(*M), order=2, integrator=rt.RT_HEUN)
+    s.set_psi(psi0)
+    s.step(2)
+    psi, dt = s.psi(), s.info.dt
+    s.close()
+    op = oracle.TriangleOracle(p, oracle.product_quadrature(*M), order=2)
+    ref, _, _ = oracle.run(op, psi0, dt, 2, "heun")
+    assert rel_l2(psi, ref) <= PSI_TOL
