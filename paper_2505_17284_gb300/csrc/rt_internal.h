@@ -141,7 +141,7 @@ int cart_tile_width(int run);
 cudaError_t launch_tri_stage(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage,
                              int storage, int vec, cudaStream_t stream);
 // Staged first-order triangle stage (rows of a chunk's cells and halo in shared
-// memory, one 512-thread CTA per SM): hmax = the instances' largest halo.
+// memory, two 256-thread CTAs per SM): hmax = the instances' largest halo.
 cudaError_t launch_tri_staged(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage, int storage,
                               int vec, int hmax, cudaStream_t stream);
 cudaError_t prepare_tri_staged(int stage, int storage, int vec, int hmax);

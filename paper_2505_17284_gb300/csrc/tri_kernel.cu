@@ -2,15 +2,16 @@
 // the cell-range kernels shared by both mesh kinds: initial phi/QoIs of a state
 // and the FP64 <-> storage conversions.
 //
-// Stage kernel: one warp per cell, lanes over ordinates (VEC consecutive
-// ordinates per lane per access, so a row of M_pad values is read with 16-byte
-// vector loads). For each ordinate k the three edges of cell i contribute
-// (omega_k . n_e) l_e / A_i * psi_hat with psi_hat = psi_i if omega_k . n_e > 0 else
-// the neighbour's psi (or psi^- of the boundary side) (Eq. upwind1stOrder);
-// F = -sum_e(...) - sigma_t psi + sigma_s/(2 pi) phi + Q (Eq. sn_2d_eqn_fv).
-// The warp sums w_k out_k over all ordinates to phi_out of the cell directly.
-// Cells are ordered by grid row, so the neighbours one row up/down (2n cells
-// away) stay in L2 while a band of rows is processed.
+// Stage kernel (where a chunk's halo is too wide for the staged kernel's buffers): one
+// warp per cell, lanes over ordinates (VEC consecutive ordinates per lane per access, so
+// a row of M_pad values is read with 16-byte vector loads). For each ordinate k the three
+// edges of cell i contribute (omega_k . n_e) l_e / A_i * psi_hat with psi_hat = psi_i if
+// omega_k . n_e > 0 else the neighbour's psi (or psi^- of the boundary side) (Eq.
+// upwind1stOrder); F = -sum_e(...) - sigma_t psi + sigma_s/(2 pi) phi + Q (Eq.
+// sn_2d_eqn_fv). The warp sums w_k out_k over all ordinates to phi_out of the cell.
+// Bound by the latency of the gathers: 1300^2 x 256 first-order Euler 2.36 -> 2.00 ms
+// with differences instead of selected traces, cell tables and the next cell's row
+// fetched to L2 (the staged kernel takes 1.66).
 #include <cuda_bf16.h>
 
 #include "device_common.cuh"
@@ -73,15 +74,20 @@ struct LaneQoI {
 
 // Persistent stage kernel: work item g of G processes the 64-cell chunks
 // g, g + G, g + 2G, ... in increasing order, so all SMs sweep the mesh together
-// and the rows of the neighbouring grid row (2n cells away on the split grid)
-// are still in L2 when they are gathered. The neighbour lists and edge
-// geometry of a chunk (contiguous arrays) are staged in shared memory by two
-// TMA bulk copies, double-buffered one chunk ahead, so a warp starts a cell
-// with its metadata at hand and goes straight to the row loads. Warp w takes
-// cells w, w + 8, ... of a chunk (neighbours one cell apart are fetched by
-// adjacent warps at the same time, L1), and loads the rows of two ordinate
-// blocks before computing either. QoI terms are summed per warp in shared
-// memory (FP32 over 32 cells, then FP64).
+// and the rows of neighbouring cells (close in the Morton order) are still in L1
+// or L2 when they are gathered. The neighbour lists and edge geometry of a chunk
+// (contiguous arrays) are staged in shared memory by two TMA bulk copies,
+// double-buffered one chunk ahead; a thread per cell turns them into a table of
+// the cell's constants, and the warps, which take cells w, w + 8, ... of the
+// chunk, then go straight to the row loads of two ordinate blocks at a time.
+//
+// With the edge normals of a cell summing to zero, the upwind flux sum is
+//   sum_e (omega . n_e) l_e / A psi_hat_e = sum_e min((omega . n_e) l_e / A, 0) (psi_e - psi_i)
+// (an edge that the ordinate leaves through contributes nothing), so an edge costs
+// a dot product, a min, a difference and a multiply-add, without a select, and the
+// rounding error scales with the differences. Arithmetic runs on FP32 pairs.
+// A cell's phi and boundary flow go to shared memory; at the chunk's end a thread
+// per cell stores phi and adds the QoI terms (FP32 over 32 chunks, then FP64).
 constexpr int kTriChunk = 64;
 
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -90,21 +96,31 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                : "memory");
 }
 
+// Constants of a chunk's cells: {dt ax0, dt ax1, dt ax2, dt ay0}, {dt ay1, dt ay2,
+// -dt sigma_t, dt (sigma_s/(2 pi) phi + Q)} with a_e = n_e l_e / A, the neighbours
+// {cell ids; own id on the boundary}, flag bit e of w set for a boundary edge.
+struct TriTable {
+  float4 g[kTriChunk], h[kTriChunk];
+  int4 nbr[kTriChunk];
+  float phi[kTriChunk], out[kTriChunk];   // results: scalar flux, boundary flow / area
+};
+
 template <int VEC, int STAGE, typename T>
 __global__ void __launch_bounds__(kTriThreads, 3)
     tri_stage_kernel(const InstDesc* __restrict__ descs, const WorkItem* __restrict__ items) {
-  __shared__ double red[(kTriWarps + 1) * NQ];
-  __shared__ float wacc[kTriWarps][NQ];
-  __shared__ double wdacc[kTriWarps][NQ];
+  __shared__ double red[2 * NQ];
+  __shared__ float facc[NQ][kTriChunk];
+  __shared__ double dacc[NQ][kTriChunk];
   __shared__ __align__(16) int4 s_nbr[2][kTriChunk];
   __shared__ __align__(16) float4 s_geo[2][2 * kTriChunk];
+  __shared__ __align__(16) TriTable tab;
   __shared__ __align__(8) uint64_t s_bar[2];
   const WorkItem it = items[blockIdx.x];
   const InstDesc& d = descs[it.inst];
   InstState* st = d.st;
   if (st->step >= d.n_steps || st->status != DEV_OK) return;
 
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int parity = (STAGE == STAGE_EULER) ? st->parity : 0;
   [[maybe_unused]] const uint32_t salt = sr_salt(st->step, STAGE);   // BF16 stochastic rounding
   const int in_buf = (STAGE == STAGE_EULER) ? parity : (STAGE == STAGE_HEUN1 ? 0 : 1);
@@ -114,9 +130,12 @@ __global__ void __launch_bounds__(kTriThreads, 3)
   T* __restrict__ psi_out = reinterpret_cast<T*>(d.psi[out_buf]);
   const float* __restrict__ phi_in = d.phi[in_buf];
   float* __restrict__ phi_out = d.phi[out_buf];
+  const float* __restrict__ q_xi = d.xi;
+  const float* __restrict__ q_eta = d.eta;
+  const float* __restrict__ q_w = d.w;
   const int Mpad = d.Mpad;
   const int nv = Mpad / (32 * VEC);
-  const float dt = d.dt;
+  const int psi_lines = (Mpad * (int)sizeof(T) + 127) / 128;
   const int nreg = d.n_regions, nq = nreg + 2;
   const int n_cells = (int)d.n_cells;
   const int n_chunks = (n_cells + kTriChunk - 1) / kTriChunk;
@@ -131,11 +150,13 @@ __global__ void __launch_bounds__(kTriThreads, 3)
     bulk_load(s_nbr[b], d.tri_nbr + c0, (uint32_t)cells * 16u, &s_bar[b]);
     bulk_load(s_geo[b], d.tri_geo + 2 * (size_t)c0, (uint32_t)cells * 32u, &s_bar[b]);
   };
-  if (lane < NQ) {
-    wacc[warp][lane] = 0.f;
-    wdacc[warp][lane] = 0.0;
+  if (tid < kTriChunk) {
+    for (int q = 0; q < nq; ++q) {
+      facc[q][tid] = 0.f;
+      dacc[q][tid] = 0.0;
+    }
   }
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     mbar_init(&s_bar[0], 1);
     mbar_init(&s_bar[1], 1);
     fence_barrier_init();
@@ -144,7 +165,6 @@ __global__ void __launch_bounds__(kTriThreads, 3)
   }
   __syncthreads();
   bool ok = true;
-  int ncell = 0;
   int i = 0;   // chunks done by this CTA
   for (int k = it.a; k < n_chunks; k += G, ++i) {
     const int b = i & 1;
@@ -154,114 +174,143 @@ __global__ void __launch_bounds__(kTriThreads, 3)
       break;
     }
     const int c0 = k * kTriChunk;
-    const int c_end = min(n_cells, c0 + kTriChunk);
-    for (int cell = c0 + warp; cell < c_end; cell += kTriWarps) {
-      const int li = cell - c0;
-      const int4 nb = s_nbr[b][li];
-      const float4 g0 = s_geo[b][2 * li], g1 = s_geo[b][2 * li + 1];
-      const float ax[3] = {g0.x, g0.z, g1.x};
-      const float ay[3] = {g0.y, g0.w, g1.y};
-      const int nbr[3] = {nb.x, nb.y, nb.z};
-      const int m = nb.w & 255, reg = (nb.w >> 8) & 255;
-      const float area = g1.z;
-      const float sig_t = d.sig_t[m];
-      const float phin = phi_in[cell];
-      const bool has_bnd = (nbr[0] < 0) | (nbr[1] < 0) | (nbr[2] < 0);
-      float gh[3];
-#pragma unroll
-      for (int e = 0; e < 3; ++e) gh[e] = (nbr[e] < 0) ? d.ghost[-1 - nbr[e]] : 0.f;
-
+    const int cells = min(kTriChunk, n_cells - c0);
+    if (tid < cells) {
+      const int4 nb = s_nbr[b][tid];
+      const float4 g0 = s_geo[b][2 * tid], g1 = s_geo[b][2 * tid + 1];
+      const int m = nb.w & 255;
+      const float dt = d.dt;
+      tab.g[tid] = make_float4(dt * g0.x, dt * g0.z, dt * g1.x, dt * g0.y);
+      tab.h[tid] = make_float4(dt * g0.w, dt * g1.y, -dt * d.sig_t[m], dt * (d.sig_s2pi[m] * phi_in[c0 + tid] + d.q_src[m]));
+      tab.nbr[tid] = make_int4(nb.x < 0 ? c0 + tid : nb.x, nb.y < 0 ? c0 + tid : nb.y, nb.z < 0 ? c0 + tid : nb.z,
+                               (nb.x < 0) | (nb.y < 0) << 1 | (nb.z < 0) << 2);
+    }
+    __syncthreads();
+    for (int li = warp; li < cells; li += kTriWarps) {
+      const int cell = c0 + li;
+      const float4 g = tab.g[li], h = tab.h[li];
+      const int4 nb = tab.nbr[li];
+      const float ax[3] = {g.x, g.y, g.z}, ay[3] = {g.w, h.x, h.y};
+      {
+        // the warp's next cell: its own row comes from DRAM, its neighbours' mostly from L2
+        const int64_t nc = li + kTriWarps < cells ? cell + kTriWarps : (int64_t)(k + G) * kTriChunk + warp;
+        for (int o = lane; nc < n_cells && o < psi_lines; o += 32)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(psi_in + (size_t)nc * Mpad) + 128 * o));
+      }
+      const T* row_c = psi_in + (size_t)cell * Mpad + lane * VEC;
+      const T* row_n[3] = {psi_in + (size_t)nb.x * Mpad + lane * VEC, psi_in + (size_t)nb.y * Mpad + lane * VEC,
+                           psi_in + (size_t)nb.z * Mpad + lane * VEC};
+      const int64_t to_base = psi_base - psi_in;
+      T* row_o = psi_out + (size_t)cell * Mpad + lane * VEC;
       float phi_part = 0.f, bpart = 0.f;
       for (int v0 = 0; v0 < nv; v0 += 2) {
         // the rows of two ordinate blocks are loaded before either is computed
-        float c2[2][VEC], nbv2[2][3][VEC], base2[2][VEC];
+        float c2[2][VEC], n2[2][3][VEC], b2[2][VEC];
         const bool two = v0 + 1 < nv;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (h == 1 && !two) break;
-          const int kk = ((v0 + h) * 32 + lane) * VEC;
-          load_vec<T, VEC>(psi_in + (size_t)cell * Mpad + kk, c2[h]);
+        for (int s = 0; s < 2; ++s) {
+          if (s == 1 && !two) break;
+          load_vec<T, VEC>(row_c + s * 32 * VEC, c2[s]);
 #pragma unroll
-          for (int e = 0; e < 3; ++e) {
-            if (nbr[e] >= 0) {
-              load_vec<T, VEC>(psi_in + (size_t)nbr[e] * Mpad + kk, nbv2[h][e]);
-            } else {
-#pragma unroll
-              for (int l = 0; l < VEC; ++l) nbv2[h][e][l] = gh[e];
-            }
-          }
-          if constexpr (STAGE == STAGE_HEUN2) load_vec<T, VEC>(psi_base + (size_t)cell * Mpad + kk, base2[h]);
+          for (int e = 0; e < 3; ++e) load_vec<T, VEC>(row_n[e] + s * 32 * VEC, n2[s][e]);
+          if constexpr (STAGE == STAGE_HEUN2) load_vec<T, VEC>(row_c + to_base + s * 32 * VEC, b2[s]);
         }
-        const float src = d.sig_s2pi[m] * phin + d.q_src[m];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (h == 1 && !two) break;
-          const int kk = ((v0 + h) * 32 + lane) * VEC;
+        for (int s = 0; s < 2; ++s) {
+          if (s == 1 && !two) break;
+          const int kk = ((v0 + s) * 32 + lane) * VEC;
           float xi[VEC], eta[VEC], w[VEC], out[VEC];
-          load_vec<float, VEC>(d.xi + kk, xi);
-          load_vec<float, VEC>(d.eta + kk, eta);
-          load_vec<float, VEC>(d.w + kk, w);
+          load_vec<float, VEC>(q_xi + kk, xi);
+          load_vec<float, VEC>(q_eta + kk, eta);
+          load_vec<float, VEC>(q_w + kk, w);
+          if (nb.w) {
+            // boundary edges: psi^- of the side
+#pragma unroll
+            for (int e = 0; e < 3; ++e)
+              if (nb.w >> e & 1) {
+                const int4 r = s_nbr[b][li];
+                const float gh = d.ghost[-1 - (e == 0 ? r.x : e == 1 ? r.y : r.z)];
+#pragma unroll
+                for (int l = 0; l < VEC; ++l) n2[s][e][l] = gh;
+              }
+          }
           // BF16 rounding bits of the lane's ordinates kk .. kk+VEC-1 (one group of four)
           [[maybe_unused]] uint2 rb4;
           if constexpr (sizeof(T) == 2) rb4 = sr_bits4((uint32_t)cell, sr_gkey(kk >> 2, salt));
+          // ordinate pairs (a single ordinate is a pair of itself)
 #pragma unroll
-          for (int l = 0; l < VEC; ++l) {
-            const float c = c2[h][l];
-            float div = 0.f;
+          for (int l = 0; l < VEC; l += 2) {
+            const int l1 = VEC > 1 ? l + 1 : l;
+            auto pair = [&](const float (&a)[VEC]) { return make_float2(a[l], a[l1]); };
+            auto dup = [](float a) { return make_float2(a, a); };
+            const float2 c = pair(c2[s]), x = pair(xi), y = pair(eta);
+            float2 inc = __ffma2_rn(dup(h.z), c, dup(h.w));   // dt F
 #pragma unroll
             for (int e = 0; e < 3; ++e) {
-              const float on = xi[l] * ax[e] + eta[l] * ay[e];
-              div += on * ((on > 0.f) ? c : nbv2[h][e][l]);
+              const float2 on = __ffma2_rn(y, dup(ay[e]), __fmul2_rn(x, dup(ax[e])));
+              const float2 n = pair(n2[s][e]);
+              inc = __ffma2_rn(make_float2(fminf(on.x, 0.f), fminf(on.y, 0.f)),
+                               __fadd2_rn(c, make_float2(-n.x, -n.y)), inc);
             }
-            const float F = -div - sig_t * c + src;
-            float o;
-            if constexpr (STAGE == STAGE_HEUN2) {
-              o = 0.5f * (base2[h][l] + c + dt * F);
-            } else {
-              o = c + dt * F;
-            }
+            float2 o = __fadd2_rn(c, inc);
+            if constexpr (STAGE == STAGE_HEUN2) o = __fmul2_rn(dup(0.5f), __fadd2_rn(pair(b2[s]), o));
             if constexpr (sizeof(T) == 2) {
-              const int ko = kk + l;
-              o = Store<T>::round_sr(o, sr_elem(rb4, ko & 3));
+              o.x = Store<T>::round_sr(o.x, sr_elem(rb4, (kk + l) & 3));
+              o.y = Store<T>::round_sr(o.y, sr_elem(rb4, (kk + l1) & 3));
             }
-            out[l] = o;
-            phi_part += w[l] * o;
-            if (has_bnd) {
+            out[l] = o.x;
+            if constexpr (VEC > 1) out[l1] = o.y;
+          }
+          store_vec<T, VEC>(row_o + s * 32 * VEC, out);
 #pragma unroll
-              for (int e = 0; e < 3; ++e) {
-                if (nbr[e] < 0) {
-                  const float on = xi[l] * ax[e] + eta[l] * ay[e];
-                  bpart += w[l] * on * ((on > 0.f) ? o : gh[e]);
+          for (int l = 0; l < VEC; ++l) phi_part = fmaf(w[l], out[l], phi_part);
+          if (nb.w) {
+            const float4 g0 = s_geo[b][2 * li], g1 = s_geo[b][2 * li + 1];
+#pragma unroll
+            for (int e = 0; e < 3; ++e)
+              if (nb.w >> e & 1) {
+                const float bx = e == 0 ? g0.x : e == 1 ? g0.z : g1.x, by = e == 0 ? g0.y : e == 1 ? g0.w : g1.y;
+#pragma unroll
+                for (int l = 0; l < VEC; ++l) {
+                  const float on = xi[l] * bx + eta[l] * by;
+                  bpart += w[l] * on * ((on > 0.f) ? out[l] : n2[s][e][l]);
                 }
               }
-            }
           }
-          store_vec<T, VEC>(psi_out + (size_t)cell * Mpad + kk, out);
         }
+        row_c += 64 * VEC;
+        row_o += 64 * VEC;
+#pragma unroll
+        for (int e = 0; e < 3; ++e) row_n[e] += 64 * VEC;
       }
       const float ph = warp_sum(phi_part);
       float bsum = 0.f;
-      if (has_bnd) bsum = warp_sum(bpart);
+      if (nb.w) bsum = warp_sum(bpart);
       if (lane == 0) {
-        phi_out[cell] = ph;
-        wacc[warp][reg] += d.sig_a_f[m] * area * ph;
-        wacc[warp][nreg] += area * ph;
-        wacc[warp][nreg + 1] += bsum * area;
-      }
-      if ((++ncell & 31) == 0) {
-        __syncwarp();
-        if (lane < nq) {
-          wdacc[warp][lane] += (double)wacc[warp][lane];
-          wacc[warp][lane] = 0.f;
-        }
-        __syncwarp();
+        tab.phi[li] = ph;
+        tab.out[li] = bsum;
       }
     }
-    // every warp is done with buffer b: it takes the chunk two ahead
+    // every warp is done with the chunk: its cells' results, then buffer b takes the chunk two ahead
     __syncthreads();
-    if (threadIdx.x == 0 && k + 2 * G < n_chunks) stage_meta(k + 2 * G, b);
+    if (tid < cells) {
+      const int w4 = s_nbr[b][tid].w;
+      const int m = w4 & 255, reg = (w4 >> 8) & 255;
+      const float area = s_geo[b][2 * tid + 1].z, ph = tab.phi[tid];
+      phi_out[c0 + tid] = ph;
+      facc[reg][tid] += d.sig_a_f[m] * area * ph;
+      facc[nreg][tid] += area * ph;
+      facc[nreg + 1][tid] += tab.out[tid] * area;
+      if ((i & 31) == 31)
+        for (int q = 0; q < nq; ++q) {
+          dacc[q][tid] += (double)facc[q][tid];
+          facc[q][tid] = 0.f;
+        }
+    }
+    __syncthreads();
+    if (tid == 0 && k + 2 * G < n_chunks) stage_meta(k + 2 * G, b);
   }
-  if (!ok && threadIdx.x == 0) {
+  if (!ok && tid == 0) {
     // drain: the metadata copies issued and not consumed (chunks i and i + 1)
     for (int j = i; j < i + 2; ++j) {
       const int kj = it.a + j * G;
@@ -270,13 +319,10 @@ __global__ void __launch_bounds__(kTriThreads, 3)
     atomicCAS(&st->status, DEV_OK, DEV_TIMEOUT);
     st->timeout_where = ((int64_t)blockIdx.x << 32) | (int64_t)i;
   }
-  __syncwarp();
-  if (lane < nq) wdacc[warp][lane] += (double)wacc[warp][lane];
   __syncthreads();
-  if (threadIdx.x < nq) {
-    double s = 0.0;
-    for (int w2 = 0; w2 < kTriWarps; ++w2) s += wdacc[w2][threadIdx.x];
-    red[threadIdx.x] = s;
+  for (int q = warp; q < nq; q += kTriWarps) {
+    const double s = warp_sum_d((dacc[q][lane] + (double)facc[q][lane]) + (dacc[q][lane + 32] + (double)facc[q][lane + 32]));
+    if (lane == 0) red[q] = s;
   }
   __syncthreads();
   finalize_item<kTriThreads>(d, it, red, STAGE, red + NQ);

@@ -181,3 +181,32 @@ def test_second_order_triangles_over_scales_of_the_state(rt, M, scale):
     op = oracle.TriangleOracle(p, oracle.product_quadrature(*M), order=2)
     ref, _, _ = oracle.run(op, psi0, dt, 2, "heun")
     assert rel_l2(psi, ref) <= PSI_TOL
+
+
+@pytest.mark.parametrize("integrator", ["euler", "heun"])
+def test_first_order_triangle_quantities_over_many_chunks_per_block(rt, integrator):
+    """11,025 chunks of 32 cells, about 36 per resident block: the FP32 sums of 32
+    chunks that each warp records before it adds them in FP64, against the sums of the
+    state itself in FP64. A recorded float has at most 32 additions of non-negative
+    terms and each term 32 ordinates' worth: 64 * 2^-24 = 3.8e-6 at most."""
+    p = si.enclosure_problem(420, jitter=0.2, seed=9)
+    quad = rt.rt_quad_product(2, 16)
+    op = oracle.TriangleOracle(p, oracle.product_quadrature(2, 16), order=1)
+    w, area, sa = oracle.product_quadrature(2, 16)[3], op.area, p.materials.sigma_a[p.materials.cell_mat]
+    psi0 = si.random_psi(p.mesh.n_cells, 32, seed=12)
+    got = []
+    for staged in (1, 0):
+        s = rt.Solver(p, quad, order=1, integrator=rt.RT_HEUN if integrator == "heun" else rt.RT_EULER)
+        rt.rt_debug_set(s.h, "tri_staged", staged)
+        s.set_psi(psi0)
+        s.step(2)
+        phi = s.psi().astype(np.float64) @ w
+        q = s.qoi()
+        s.close()
+        assert abs(q["mass"] - np.sum(area * phi)) <= 4e-6 * q["mass"]
+        per = np.bincount(p.materials.cell_region, weights=area * sa * phi, minlength=p.materials.n_regions)
+        assert np.max(np.abs(np.asarray(q["abs_now"]) - per)) <= 4e-6 * np.max(per)
+        got.append(q)
+    for k in ("mass", "abs_int", "outflow_int"):
+        a, b = (np.asarray(g[k], float) for g in got)
+        assert np.max(np.abs(a - b)) <= 8e-6 * np.max(np.abs(b)), k
