@@ -42,7 +42,7 @@ rt_status launch_steps_direct(rt_solver* s, int64_t n, cudaStream_t stream) {
   for (int64_t i = 0; i < n; ++i) {
     rt_status st = launch_step(s->d_desc, s->d_stage_items, (int)I.stage_items.size(), I.kind, I.integrator,
                                I.storage, I.order, I.run, I.cvec, I.ly, I.vec, stream, I.uni, s->d_box_items,
-                               (int)I.box_items.size());
+                               (int)I.box_items.size(), i > 0);
     if (st != RT_OK) return st;
   }
   return RT_OK;

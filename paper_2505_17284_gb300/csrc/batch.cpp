@@ -300,7 +300,7 @@ rt_status enqueue_steps(rt_batch* b, int64_t n, cudaStream_t stream, int64_t* la
   for (int64_t i = 0; i < n; ++i) {
     for (const Group& g : b->groups) {
       rt_status st = launch_step(b->d_desc, b->d_items + g.offset, g.count, g.kind, g.integrator, b->storage, g.order,
-                                 g.run, g.cvec, g.ly_max, g.vec, stream, g.uni, nullptr, 0);
+                                 g.run, g.cvec, g.ly_max, g.vec, stream, g.uni, nullptr, 0, i > 0 || &g != &b->groups[0]);
       if (st != RT_OK) return st;
       *launched += g.integrator == RT_HEUN ? 2 : 1;
     }

@@ -14,7 +14,7 @@ RTK_UNIT_DECL(bf16_lane)
 #define RTK_STR_DECL(NAME)                                                                                  \
   cudaError_t str_prepare_##NAME(int stage, int tx, int ly);                                                \
   cudaError_t str_launch_##NAME(const InstDesc*, const WorkItem*, int n_items, int stage, int tx, int ly,    \
-                                cudaStream_t);                                                              \
+                                cudaStream_t, bool chained);                                                \
   size_t str_smem_##NAME(int stage, int tx, int ly);
 RTK_STR_DECL(f32_o1)
 RTK_STR_DECL(f32_o2)
@@ -42,10 +42,12 @@ cudaError_t prepare_cart_stage(int stage, int order, int storage, int run, int v
 }
 
 cudaError_t launch_cart_stage(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage, int order,
-                              int storage, int run, int vec, int ly_max, cudaStream_t stream, int uni) {
+                              int storage, int run, int vec, int ly_max, cudaStream_t stream, int uni,
+                              bool chained) {
   if (n_items <= 0) return cudaSuccess;
   if (!variant_exists(order, run, vec, uni)) return cudaErrorInvalidValue;
-  if (uni) return RTK_STR_PICK(str_launch)(d_desc, d_items, n_items, stage, cart_tile_width(run), ly_max, stream);
+  if (uni) return RTK_STR_PICK(str_launch)(d_desc, d_items, n_items, stage, cart_tile_width(run), ly_max, stream,
+                                         chained);
   return (storage == 0 ? cart_launch_f32_lane : cart_launch_bf16_lane)(d_desc, d_items, n_items, stage, order, vec,
                                                                        ly_max, stream);
 }

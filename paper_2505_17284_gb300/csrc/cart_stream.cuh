@@ -484,8 +484,10 @@ __global__ void __launch_bounds__(kStrThreads, 2)
   const WorkItem it = items[blockIdx.x];
   const InstDesc& d = descs[it.inst];
   InstState* st = d.st;
+  grid_wait();
+  const StepHead head = step_head(st);
   // finished or failed instances are masked
-  if (st->step >= d.n_steps || st->status != DEV_OK) return;
+  if (head.step >= d.n_steps || head.status != DEV_OK) return;
   if (d.drop_load >= 0) {
     // test hook: a load that never arrives. Nothing here waits on a barrier that a load
     // completes, so the launch gives up at once instead of after the wait limit.
@@ -498,8 +500,8 @@ __global__ void __launch_bounds__(kStrThreads, 2)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int TX = d.tx, tx_shift = 31 - __clz(TX), WX = TX / kStrCells, WC = kStrWarps / WX;
   const int wx = warp & (WX - 1), wc = warp / WX;
-  const int parity = (STAGE == STAGE_EULER) ? st->parity : 0;
-  const uint32_t salt = sr_salt(st->step, STAGE);   // BF16 stochastic rounding
+  const int parity = (STAGE == STAGE_EULER) ? head.parity : 0;
+  const uint32_t salt = sr_salt(head.step, STAGE);   // BF16 stochastic rounding
   const int in_buf = (STAGE == STAGE_EULER) ? parity : (STAGE == STAGE_HEUN1 ? 0 : 1);
   const int out_buf = (STAGE == STAGE_EULER) ? (1 - parity) : (STAGE == STAGE_HEUN1 ? 1 : 0);
   const float* __restrict__ phi_in = d.phi[in_buf];
@@ -622,14 +624,14 @@ static cudaError_t str_prepare_one(int tx, int ly) {
                                 : str_smem_for<ORDER, STAGE_EULER, TT>(tx, ly);                               \
   }                                                                                                           \
   cudaError_t str_launch_##NAME(const InstDesc* d, const WorkItem* items, int n, int stage, int tx, int ly,   \
-                                cudaStream_t s) {                                                             \
+                                cudaStream_t s, bool chained) {                                               \
     cudaError_t e = str_prepare_##NAME(stage, tx, ly);                                                        \
     if (e != cudaSuccess) return e;                                                                           \
     const size_t smem = str_smem_##NAME(stage, tx, ly);                                                       \
-    if (stage == STAGE_EULER) cart_stream_kernel<ORDER, STAGE_EULER, TT><<<n, kStrThreads, smem, s>>>(d, items); \
-    else if (stage == STAGE_HEUN1) cart_stream_kernel<ORDER, STAGE_HEUN1, TT><<<n, kStrThreads, smem, s>>>(d, items); \
-    else cart_stream_kernel<ORDER, STAGE_HEUN2, TT><<<n, kStrThreads, smem, s>>>(d, items);                   \
-    return cudaGetLastError();                                                                                \
+    return launch_stage_kernel(stage == STAGE_EULER   ? cart_stream_kernel<ORDER, STAGE_EULER, TT>            \
+                               : stage == STAGE_HEUN1 ? cart_stream_kernel<ORDER, STAGE_HEUN1, TT>            \
+                                                      : cart_stream_kernel<ORDER, STAGE_HEUN2, TT>,           \
+                               n, kStrThreads, smem, s, chained, d, items);                                   \
   }
 
 }  // namespace rtk

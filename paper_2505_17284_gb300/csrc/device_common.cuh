@@ -128,6 +128,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+constexpr int64_t kDrainCycles = 4000000000LL;   // bound of a wait for copies in flight (about two seconds)
+
 // Wait for phase `parity` of `bar` to complete, for at most `limit` SM clock
 // cycles. Returns false if the limit ran out.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, int64_t limit) {
@@ -137,6 +139,28 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     if (mbar_try_wait(bar, parity)) return true;
     if (clock64() - t0 > limit) return false;
   }
+}
+
+// Stage kernels of a run of steps are launched with programmatic serialisation: a grid's
+// blocks become resident when those of the stage before have left, before its writes are
+// flushed and its end is reported, and run what depends on set-up data alone (descriptors,
+// work items, mesh data) until grid_wait() returns: the stage before has then completed and
+// its writes are visible (at once in a launch without the attribute). Every thread calls it,
+// in every block and before any return: a grid that completed without waiting would let the
+// one after it start too early. No grid lets the next one in before its own blocks leave
+// (griddepcontrol.launch_dependents): that cost 2 us a launch, and the next stage's blocks
+// then filled whichever SMs emptied first, two to an SM on grids below one wave (140^2 x 128
+// Heun 52 -> 59 us). Without it 60^2 x 64 triangles 14.6 -> 12.3 us a first-order step and
+// 55.7 -> 45.8 a second-order one, 130^2 x 64 20.7 -> 18.4 and 100.8 -> 97.7.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The instance's position in time, read past L1.
+struct StepHead {
+  int64_t step;
+  int32_t parity, status;
+};
+__device__ __forceinline__ StepHead step_head(const InstState* st) {
+  return {__ldcg(&st->step), __ldcg(&st->parity), __ldcg(&st->status)};
 }
 
 // 3-D tiled TMA load of one box into shared memory, completing on `bar`.
@@ -355,6 +379,23 @@ __device__ void finalize_item(const InstDesc& d, const WorkItem& it, const doubl
     }
     st->ticket = 0u;
   }
+}
+
+// Launch of a stage kernel; `chained`: it follows another kernel of the same run of steps.
+template <typename... P, typename... A>
+inline cudaError_t launch_stage_kernel(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t stream,
+                                       bool chained, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 }  // namespace rtk

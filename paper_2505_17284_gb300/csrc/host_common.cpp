@@ -1083,17 +1083,18 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
 
 rt_status launch_step(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int kind, int integrator,
                       int storage, int order, int run, int cvec, int ly_max, int vec, cudaStream_t stream,
-                      int uni, const WorkItem* d_box_items, int n_box_items) {
+                      int uni, const WorkItem* d_box_items, int n_box_items, bool chained) {
   const int stages[2] = {integrator == RT_HEUN ? STAGE_HEUN1 : STAGE_EULER, STAGE_HEUN2};
   const int n_st = integrator == RT_HEUN ? 2 : 1;
   for (int i = 0; i < n_st; ++i) {
     cudaError_t e;
     if (kind == RT_MESH_CARTESIAN)
-      e = launch_cart_stage(d_desc, d_items, n_items, stages[i], order, storage, run, cvec, ly_max, stream, uni);
+      e = launch_cart_stage(d_desc, d_items, n_items, stages[i], order, storage, run, cvec, ly_max, stream, uni,
+                            chained || i > 0);
     else if (order == 2)
-      e = launch_tri2_stage(d_desc, d_items, n_items, stages[i], storage, vec, stream);
+      e = launch_tri2_stage(d_desc, d_items, n_items, stages[i], storage, vec, stream, chained || i > 0);
     else if (uni)
-      e = launch_tri_staged(d_desc, d_items, n_items, stages[i], storage, vec, ly_max, stream);
+      e = launch_tri_staged(d_desc, d_items, n_items, stages[i], storage, vec, ly_max, stream, chained || i > 0);
     else
       e = launch_tri_stage(d_desc, d_items, n_items, stages[i], storage, vec, stream);
     if (e != cudaSuccess) {

@@ -92,10 +92,11 @@ int device_sm_count();
 // Launch the stage(s) of one time step for the given instances' work items.
 // `run`/`cvec` select the Cartesian variant, `vec` the triangle vector width.
 // d_box_items/n_box_items: the QoI-box work items of the same instances (one
-// launch after the step's last stage).
+// launch after the step's last stage). chained: not the first step of a run of steps.
 rt_status launch_step(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int kind, int integrator,
                       int storage, int order, int run, int cvec, int ly_max, int vec, cudaStream_t stream,
-                      int uni = 0, const WorkItem* d_box_items = nullptr, int n_box_items = 0);
+                      int uni = 0, const WorkItem* d_box_items = nullptr, int n_box_items = 0,
+                      bool chained = false);
 // Initial-state launches: phi and QoI integrands, then the box outflow.
 rt_status launch_init_all(const InstDesc* d_desc, const WorkItem* d_init_items, int n_init_items,
                           const WorkItem* d_box_items, int n_box_items, int vec, int storage, cudaStream_t stream);

@@ -128,12 +128,14 @@ struct WorkItem {
   int32_t pad;
 };
 
-// Launchers (defined in the .cu files). All enqueue on `stream`.
+// Launchers (defined in the .cu files). All enqueue on `stream`. chained: the launch
+// follows a kernel of the same run of steps, and nothing else, on its stream, so its blocks
+// may start before that one ends.
 // Cartesian stage kernels. uni != 0: the streaming kernel (InstDesc::str_chunks; tile
 // width 8 * run, run 2 or 4); uni = 0: the general kernel (run 2, vec ordinates per lane).
 cudaError_t launch_cart_stage(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage,
                               int order, int storage, int run, int vec, int ly_max, cudaStream_t stream,
-                              int uni = 0);
+                              int uni = 0, bool chained = false);
 size_t cart_smem_bytes(int order, int storage, int run, int vec, int ly, int stage, int uni = 0);
 int cart_stream_chunk_groups(int tx);   // warps that share a column of a tile of tx cells
 cudaError_t prepare_cart_stage(int stage, int order, int storage, int run, int vec, int ly_max, int uni = 0);
@@ -143,7 +145,7 @@ cudaError_t launch_tri_stage(const InstDesc* d_desc, const WorkItem* d_items, in
 // Staged first-order triangle stage (rows of a chunk's cells and halo in shared
 // memory, two 256-thread CTAs per SM): hmax = the instances' largest halo.
 cudaError_t launch_tri_staged(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage, int storage,
-                              int vec, int hmax, cudaStream_t stream);
+                              int vec, int hmax, cudaStream_t stream, bool chained = false);
 cudaError_t prepare_tri_staged(int stage, int storage, int vec, int hmax);
 size_t tri_staged_smem_bytes(int vec, int storage, int hmax, int stage);
 cudaError_t launch_init(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int vec,
@@ -151,7 +153,7 @@ cudaError_t launch_init(const InstDesc* d_desc, const WorkItem* d_items, int n_i
 // Second-order triangle stage: the limited-gradient kernel, then the stage kernel, both
 // persistent with tri2_ctas_per_sm(vec) CTAs per SM (vec ordinates per lane: 1, 2 or 4).
 cudaError_t launch_tri2_stage(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage, int storage,
-                              int vec, cudaStream_t s);
+                              int vec, cudaStream_t s, bool chained = false);
 int tri2_ctas_per_sm(int vec);
 // Outflow through the QoI boxes after a time step (stage = STAGE_EULER, or
 // STAGE_HEUN2 after a whole Heun step) with the step's time-integration

@@ -187,11 +187,7 @@ __global__ void __launch_bounds__(t2_grad_threads(VEC), t2_ctas(VEC))
   const WorkItem it = items[blockIdx.x];
   const InstDesc& d = descs[it.inst];
   InstState* st = d.st;
-  if (st->step >= d.n_steps || st->status != DEV_OK) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int in_buf = (stage == STAGE_EULER) ? st->parity : (stage == STAGE_HEUN1 ? 0 : 1);
-  const T* __restrict__ psi = reinterpret_cast<const T*>(d.psi[in_buf]);
-  float* __restrict__ lg = d.tri_lg;
   const int Mpad = d.Mpad;
   const int nv = Mpad / (32 * VEC);
   const int psi_lines = (Mpad * (int)sizeof(T) + 127) / 128;
@@ -206,6 +202,18 @@ __global__ void __launch_bounds__(t2_grad_threads(VEC), t2_ctas(VEC))
     if (it.a < n_chunks) t2_stage_meta(d, meta, it.a, 0, n_cells);
     if (it.a + G < n_chunks) t2_stage_meta(d, meta, it.a + G, 1, n_cells);
   }
+  grid_wait();
+  const StepHead head = step_head(st);
+  if (head.step >= d.n_steps || head.status != DEV_OK) {
+    // finished or failed instances are masked; no copy may be in flight when the block leaves
+    if (threadIdx.x == 0)
+      for (int j = 0; j < 2; ++j)
+        if (it.a + j * G < n_chunks) mbar_wait_bounded(&meta.bar[j], 0u, kDrainCycles);
+    return;
+  }
+  const int in_buf = (stage == STAGE_EULER) ? head.parity : (stage == STAGE_HEUN1 ? 0 : 1);
+  const T* __restrict__ psi = reinterpret_cast<const T*>(d.psi[in_buf]);
+  float* __restrict__ lg = d.tri_lg;
   __syncthreads();
   bool ok = true;
   int i = 0;
@@ -303,22 +311,11 @@ __global__ void __launch_bounds__(kT2Threads, t2_ctas(VEC))
   const WorkItem it = items[blockIdx.x];
   const InstDesc& d = descs[it.inst];
   InstState* st = d.st;
-  if (st->step >= d.n_steps || st->status != DEV_OK) return;
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int parity = (STAGE == STAGE_EULER) ? st->parity : 0;
-  [[maybe_unused]] const uint32_t salt = sr_salt(st->step, STAGE);   // BF16 stochastic rounding
-  const int in_buf = (STAGE == STAGE_EULER) ? parity : (STAGE == STAGE_HEUN1 ? 0 : 1);
-  const int out_buf = (STAGE == STAGE_EULER) ? (1 - parity) : (STAGE == STAGE_HEUN1 ? 1 : 0);
-  const T* __restrict__ psi_in = reinterpret_cast<const T*>(d.psi[in_buf]);
-  const T* __restrict__ psi_base = reinterpret_cast<const T*>(d.psi[0]);
-  T* __restrict__ psi_out = reinterpret_cast<T*>(d.psi[out_buf]);
-  const float* __restrict__ lg = d.tri_lg;
   const float* __restrict__ d_xi = d.xi;
   const float* __restrict__ d_eta = d.eta;
   const float* __restrict__ d_w = d.w;
-  const float* __restrict__ phi_in = d.phi[in_buf];
-  float* __restrict__ phi_out = d.phi[out_buf];
   const int Mpad = d.Mpad;
   const int nv = Mpad / (32 * VEC);
   const int psi_lines = (Mpad * (int)sizeof(T) + 127) / 128;
@@ -340,6 +337,25 @@ __global__ void __launch_bounds__(kT2Threads, t2_ctas(VEC))
     if (it.a < n_chunks) t2_stage_meta(d, meta, it.a, 0, n_cells);
     if (it.a + G < n_chunks) t2_stage_meta(d, meta, it.a + G, 1, n_cells);
   }
+  grid_wait();
+  const StepHead head = step_head(st);
+  if (head.step >= d.n_steps || head.status != DEV_OK) {
+    // finished or failed instances are masked; no copy may be in flight when the block leaves
+    if (threadIdx.x == 0)
+      for (int j = 0; j < 2; ++j)
+        if (it.a + j * G < n_chunks) mbar_wait_bounded(&meta.bar[j], 0u, kDrainCycles);
+    return;
+  }
+  const int parity = (STAGE == STAGE_EULER) ? head.parity : 0;
+  [[maybe_unused]] const uint32_t salt = sr_salt(head.step, STAGE);   // BF16 stochastic rounding
+  const int in_buf = (STAGE == STAGE_EULER) ? parity : (STAGE == STAGE_HEUN1 ? 0 : 1);
+  const int out_buf = (STAGE == STAGE_EULER) ? (1 - parity) : (STAGE == STAGE_HEUN1 ? 1 : 0);
+  const T* __restrict__ psi_in = reinterpret_cast<const T*>(d.psi[in_buf]);
+  const T* __restrict__ psi_base = reinterpret_cast<const T*>(d.psi[0]);
+  T* __restrict__ psi_out = reinterpret_cast<T*>(d.psi[out_buf]);
+  const float* __restrict__ lg = d.tri_lg;
+  const float* __restrict__ phi_in = d.phi[in_buf];
+  float* __restrict__ phi_out = d.phi[out_buf];
   __syncthreads();
   bool ok = true;
   int ncell = 0;
@@ -519,15 +535,14 @@ __global__ void __launch_bounds__(kT2Threads, t2_ctas(VEC))
 int tri2_ctas_per_sm(int vec) { return t2_ctas(vec); }
 
 cudaError_t launch_tri2_stage(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage, int storage,
-                              int vec, cudaStream_t s) {
+                              int vec, cudaStream_t s, bool chained) {
   if (n_items <= 0) return cudaSuccess;
 #define RTK_T2(V, ST, TT)                                                                       \
   if (vec == V && stage == ST) {                                                                \
-    tri_grad_kernel<V, TT><<<n_items, t2_grad_threads(V), 0, s>>>(d_desc, d_items, ST);         \
-    cudaError_t e = cudaGetLastError();                                                         \
+    cudaError_t e = launch_stage_kernel(tri_grad_kernel<V, TT>, n_items, t2_grad_threads(V), 0, s, chained, \
+                                        d_desc, d_items, ST);                                   \
     if (e != cudaSuccess) return e;                                                             \
-    tri_stage2_kernel<V, ST, TT><<<n_items, kT2Threads, 0, s>>>(d_desc, d_items);               \
-    return cudaGetLastError();                                                                  \
+    return launch_stage_kernel(tri_stage2_kernel<V, ST, TT>, n_items, kT2Threads, 0, s, true, d_desc, d_items); \
   }
 #define RTK_T2_ALL(TT)                                                                          \
   RTK_T2(1, STAGE_EULER, TT) RTK_T2(1, STAGE_HEUN1, TT) RTK_T2(1, STAGE_HEUN2, TT)              \

@@ -149,20 +149,10 @@ __global__ void __launch_bounds__(kStgThreads, 2)
   const WorkItem it = items[blockIdx.x];
   const InstDesc& d = descs[it.inst];
   InstState* st = d.st;
-  if (st->step >= d.n_steps || st->status != DEV_OK) return;
 
   constexpr int W = 32 * VEC;
   constexpr bool kBase = STAGE == STAGE_HEUN2;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int parity = (STAGE == STAGE_EULER) ? st->parity : 0;
-  [[maybe_unused]] const uint32_t salt = sr_salt(st->step, STAGE);   // BF16 stochastic rounding
-  const int in_buf = (STAGE == STAGE_EULER) ? parity : (STAGE == STAGE_HEUN1 ? 0 : 1);
-  const int out_buf = (STAGE == STAGE_EULER) ? (1 - parity) : (STAGE == STAGE_HEUN1 ? 1 : 0);
-  const T* __restrict__ psi_in = reinterpret_cast<const T*>(d.psi[in_buf]);
-  const T* __restrict__ psi_base = reinterpret_cast<const T*>(d.psi[0]);
-  T* __restrict__ psi_out = reinterpret_cast<T*>(d.psi[out_buf]);
-  const float* __restrict__ phi_in = d.phi[in_buf];
-  float* __restrict__ phi_out = d.phi[out_buf];
   const float* __restrict__ d_xi = d.xi;
   const float* __restrict__ d_eta = d.eta;
   const float* __restrict__ d_w = d.w;
@@ -176,7 +166,6 @@ __global__ void __launch_bounds__(kStgThreads, 2)
   const int64_t limit = d.wait_limit;
   const StgLayout L = stg_layout(VEC, (int)sizeof(T), d.tri_hmax, kBase);
   const int base_row = kStgChunk + L.hmax;
-  const int64_t to_base = psi_base - psi_in;
 
   uint8_t* smem = stg_raw + ((128u - (smem_u32(stg_raw) & 127u)) & 127u);
   uint8_t* rowbuf[2] = {smem, smem + L.buf_bytes};
@@ -214,6 +203,38 @@ __global__ void __launch_bounds__(kStgThreads, 2)
     bulk_copy(m + 3 * kStgChunk * 16, d.tri_lidx + (size_t)k * kStgChunk, kStgChunk * 4u, &meta_bar[mb]);
     if (hpad > 0) bulk_copy(m + 3 * kStgChunk * 16 + kStgChunk * 4, d.tri_halo + oc.x, (uint32_t)hpad * 4u, &meta_bar[mb]);
   };
+
+  if (threadIdx.x < kStgChunk)
+    for (int q = 0; q < nq; ++q) facc[q][threadIdx.x] = 0.f;
+  if (lane < NQ) dacc[warp][lane] = 0.0;
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < kStgMeta; ++q) {
+      mbar_init(&meta_bar[q], 1);
+      s_meta_last[q] = -1;
+    }
+    fence_barrier_init();
+    for (int i = 0; i < min(n_my, kStgMeta - 1); ++i) issue_meta(i);
+  }
+  grid_wait();
+  const StepHead head = step_head(st);
+  if (head.step >= d.n_steps || head.status != DEV_OK) {
+    // finished or failed instances are masked; no copy may be in flight when the block leaves
+    if (threadIdx.x == 0)
+      for (int i = 0; i < min(n_my, kStgMeta - 1); ++i) mbar_wait_bounded(&meta_bar[i], 0u, kDrainCycles);
+    return;
+  }
+  const int parity = (STAGE == STAGE_EULER) ? head.parity : 0;
+  [[maybe_unused]] const uint32_t salt = sr_salt(head.step, STAGE);   // BF16 stochastic rounding
+  const int in_buf = (STAGE == STAGE_EULER) ? parity : (STAGE == STAGE_HEUN1 ? 0 : 1);
+  const int out_buf = (STAGE == STAGE_EULER) ? (1 - parity) : (STAGE == STAGE_HEUN1 ? 1 : 0);
+  const T* __restrict__ psi_in = reinterpret_cast<const T*>(d.psi[in_buf]);
+  const T* __restrict__ psi_base = reinterpret_cast<const T*>(d.psi[0]);
+  T* __restrict__ psi_out = reinterpret_cast<T*>(d.psi[out_buf]);
+  const float* __restrict__ phi_in = d.phi[in_buf];
+  float* __restrict__ phi_out = d.phi[out_buf];
+  const int64_t to_base = psi_base - psi_in;
+  __syncthreads();
+
   // Start the copies of block bb of chunk ordinal ii (whose metadata must have arrived: false
   // if waiting for it ran out) into row buffer rb, 16 bytes per lane: a warp takes rows
   // warp * RPI .. + RPI - 1 and every kStgWarps * RPI-th group after them.
@@ -241,9 +262,6 @@ __global__ void __launch_bounds__(kStgThreads, 2)
     return true;
   };
 
-  if (threadIdx.x < kStgChunk)
-    for (int q = 0; q < nq; ++q) facc[q][threadIdx.x] = 0.f;
-  if (lane < NQ) dacc[warp][lane] = 0.0;
   // add a warp's FP32 QoI sums (its cells of a chunk) to its FP64 ones
   auto flush = [&]() {
     __syncwarp();
@@ -257,15 +275,6 @@ __global__ void __launch_bounds__(kStgThreads, 2)
     }
     __syncwarp();
   };
-  if (threadIdx.x == 0) {
-    for (int q = 0; q < kStgMeta; ++q) {
-      mbar_init(&meta_bar[q], 1);
-      s_meta_last[q] = -1;
-    }
-    fence_barrier_init();
-    for (int i = 0; i < min(n_my, kStgMeta - 1); ++i) issue_meta(i);
-  }
-  __syncthreads();
   // Cell table of chunk ordinal i, lane l of the last warp for cell l: what a cell needs
   // besides its rows. Built while the chunk before it is computed, in two halves, so that
   // the load of phi has that long.
@@ -489,9 +498,8 @@ static cudaError_t stg_prepare_one(size_t smem) {
 
 template <int VEC, int STAGE, typename T>
 static cudaError_t stg_launch_one(const InstDesc* d_desc, const WorkItem* d_items, int n_items, size_t smem,
-                                  cudaStream_t s) {
-  tri_staged_kernel<VEC, STAGE, T><<<n_items, kStgThreads, smem, s>>>(d_desc, d_items);
-  return cudaGetLastError();
+                                  cudaStream_t s, bool chained) {
+  return launch_stage_kernel(tri_staged_kernel<VEC, STAGE, T>, n_items, kStgThreads, smem, s, chained, d_desc, d_items);
 }
 
 #define RTK_STG_ALL(X, TT)                                                                          \
@@ -517,12 +525,12 @@ cudaError_t prepare_tri_staged(int stage, int storage, int vec, int hmax) {
 }
 
 cudaError_t launch_tri_staged(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage, int storage,
-                              int vec, int hmax, cudaStream_t s) {
+                              int vec, int hmax, cudaStream_t s, bool chained) {
   if (n_items <= 0) return cudaSuccess;
   const size_t smem = tri_staged_smem_bytes(vec, storage, hmax, stage);
   vec = stg_vec(storage, vec);
 #define RTK_L(V, ST, TT) \
-  if (vec == V && stage == ST) return stg_launch_one<V, ST, TT>(d_desc, d_items, n_items, smem, s);
+  if (vec == V && stage == ST) return stg_launch_one<V, ST, TT>(d_desc, d_items, n_items, smem, s, chained);
   if (storage == 0) { RTK_STG_ALL(RTK_L, float) } else { RTK_STG_ALL(RTK_L, __nv_bfloat16) }
 #undef RTK_L
   return cudaErrorInvalidValue;
