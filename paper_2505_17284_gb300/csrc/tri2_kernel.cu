@@ -106,16 +106,28 @@ __device__ __forceinline__ float fmax3f(float a, float b, float c) {
   return r;
 }
 
-// L and L g of one value given its gradient and the spread of its neighbourhood. The
-// quotients are formed with __fdividef (2 ulp, where the denominators lie inside its
-// range; otherwise, for values below 1e-15 or above 1e18 of the state's unit, by IEEE
-// division): three IEEE divisions in divergent branches were 200 of 269 instructions
-// per cell and ordinate.
+// Smallest of the three edges' limiter values. The quotients are formed with __fdividef
+// (2 ulp inside its range of denominators): three IEEE divisions in divergent branches were
+// 200 of 269 instructions per cell and ordinate. Denominators below that range, which a
+// state of zeros or a front's foot has where epsilon^2 = A^6 is small (10^-36 at 2 * 650^2
+// cells), are formed again from x and y times 2^63, the quotient being homogeneous; only
+// states above 10^18 divide by IEEE.
 __device__ __forceinline__ float limiter(const float (&x)[3], const float (&y)[3], const float (&num)[3],
                                          const float (&den)[3], float eps2) {
   const float lo = fmin3f(den[0], den[1], den[2]), hi = fmax3f(den[0], den[1], den[2]);
-  if (lo >= 1e-30f && hi <= 1e36f)
+  if (lo >= 0x1p-126f && hi <= 1e36f)
     return fmin3f(__fdividef(num[0], den[0]), __fdividef(num[1], den[1]), __fdividef(num[2], den[2]));
+  if (hi <= 1e36f) {
+    float L[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      const float s = den[e] < 0x1p-100f ? 0x1p63f : 1.f;
+      const float xs = x[e] * s, ys = y[e] * s, p = xs * ys, c = fmaf(ys, ys, eps2 * s * s) + p;
+      const float d = fmaf(xs + xs, xs, c);
+      L[e] = d > 0.f ? __fdividef(c + p, d) : 1.f;   // 0 / 0 without a spread
+    }
+    return fmin3f(L[0], L[1], L[2]);
+  }
   return fminf(fminf(venkat_exact(x[0], y[0], eps2), venkat_exact(x[1], y[1], eps2)), venkat_exact(x[2], y[2], eps2));
 }
 

@@ -210,3 +210,26 @@ def test_first_order_triangle_quantities_over_many_chunks_per_block(rt, integrat
     for k in ("mass", "abs_int", "outflow_int"):
         a, b = (np.asarray(g[k], float) for g in got)
         assert np.max(np.abs(a - b)) <= 8e-6 * np.max(np.abs(b)), k
+
+
+@pytest.mark.parametrize("M", [(2, 16), (4, 16), (8, 16)])   # 1, 2 and 4 ordinates per lane
+@pytest.mark.parametrize("scale", [0.0, 1e-18, 1e-19, 1e-20, 1e-25])
+def test_second_order_triangles_with_denominators_below_the_fast_range(rt, M, scale):
+    """States whose squared differences lie around epsilon^2 = A^6 (about 1e-39 here, below
+    the normal range) and a state of zeros: the limiter rescales its quotients there.
+    epsilon^2 itself is held to 2e-6 of its value, the limiter with it."""
+    mesh = si.split_grid_mesh(13, 0.01, jitter=0.2, seed=4)
+    n = mesh.n_cells
+    mats = si.Materials(sigma_a=np.array([1.0, 40.0]), sigma_s=np.array([20.0, 3.0]),
+                        Q=np.array([0.0, 30.0]) * (scale or 1.0), cell_mat=(np.arange(n) == 60).astype(np.int32),
+                        cell_region=np.zeros(n, np.int32), region_names=("all",))
+    p = si.Problem(mesh=mesh, materials=mats, boundary=si.Boundary(), t_end=1.0)
+    psi0 = (si.smooth_psi(mesh, M[0] * M[1], seed=2) + 0.2 * si.random_psi(n, M[0] * M[1], seed=3)) * scale
+    s = rt.Solver(p, rt.rt_quad_product(*M), order=2, integrator=rt.RT_HEUN)
+    s.set_psi(psi0)
+    s.step(3)
+    psi, dt = s.psi(), s.info.dt
+    s.close()
+    op = oracle.TriangleOracle(p, oracle.product_quadrature(*M), order=2)
+    ref, _, _ = oracle.run(op, psi0, dt, 3, "heun")
+    assert rel_l2(psi, ref) <= PSI_TOL
