@@ -546,9 +546,13 @@ static bool regroup_quadrature(const rt_quadrature* quad, std::vector<double>& x
 // units of one row of a warp that shares its SM with one CTA. A CTA costs a fixed part
 // (start, tile constants, QoI sums, about 10 rows) and chunks x rows, 1.28 times that
 // with two CTAs on the SM (the most that are resident); with more items than fit at
-// once the fixed parts overlap other CTAs' rows, and the last round adds about 0.4 of
-// an item. Against timings of 13 problems at 3 to 64 rows (70^2 x 64 to 1400^2 x 512)
-// its choice is within 4 % of the best. *cost receives the model's time.
+// once the fixed parts overlap other CTAs' rows, and the last round adds about half an
+// item. With more than one chunk of ordinates segments end at 40 rows: longer ones lose
+// more, to neighbouring strips whose rows have left L2 and to SMs that finish early, than
+// their shared rows save (1400^2 x 512 Heun 3745 us at 61 rows, 3590 at 37; 911^2 x 196 BF16
+// 1078 at 57, 976 at 44). Against timings of 29 problems at 3 to 64 rows (70^2 x 64 to
+// 1400^2 x 512) its choice is 4 % from the best on average, 14 % at most. *cost receives
+// the model's time.
 static int stream_segment(const Instance& I, int run, double* cost) {
   const int sms = device_sm_count();
   const int tx = cart_tile_width(run), groups = cart_stream_chunk_groups(tx);
@@ -557,7 +561,8 @@ static int stream_segment(const Instance& I, int run, double* cost) {
   const int stage_hi = I.integrator == RT_HEUN ? STAGE_HEUN2 : STAGE_EULER;
   int best = 8;
   *cost = INFINITY;
-  for (int ly = 3; ly <= 64; ++ly) {
+  const int ly_most = I.str_chunks.size() > 1 ? 40 : 64;
+  for (int ly = 3; ly <= ly_most; ++ly) {
     // two CTAs per SM by shared memory (228 KB, 1 KB of it per CTA reserved)
     if (cart_smem_bytes(I.order, I.storage, run, I.cvec, ly, stage_hi, 1) > 113 * 1024) break;
     const int64_t items = strips * ((I.ny + ly - 1) / ly);
@@ -568,7 +573,7 @@ static int stream_segment(const Instance& I, int run, double* cost) {
     } else if (items <= 2 * sms) {
       t = 12.0 + 1.28 * chunks * rows;
     } else {
-      t = (5.8 + 1.28 * chunks * rows) * ((double)items / (2.0 * sms) + 0.4);
+      t = (7.0 + 1.28 * chunks * rows) * ((double)items / (2.0 * sms) + 0.5);
     }
     if (t < *cost) {
       *cost = t;
@@ -773,7 +778,9 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
     I.run = 2;
     // 32-cell tiles: asked for, or taken when whole chunks of 128 ordinates mix signs but
     // chunks of 64 do not (256 ordinates), on grids of more than kWideMinCells cells.
-    constexpr int64_t kWideMinCells = 100000;
+    // Above kWideMaxCells cells second order takes tiles of 16 cells all the same (256
+    // ordinates, Heun: 450^2 304 us with 32, 280 with 16; 840^2 848 and 756).
+    constexpr int64_t kWideMinCells = 100000, kWideMaxCells = 1 << 17;
     bool wide = false;
     if (variant != 1 && (vec == 0 || vec == 2) && tile_x != 16) {
       const bool narrow4 = tile_x == 0 && vec == 0 && I.cvec >= 4 && chunks_uniform(quad, I.Mpad, 4);
@@ -815,6 +822,7 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
       if (!I.uni) I.info_vec = 0;
       I.uni = 1;
       I.cvec = 4;
+      if (tile_x == 0 && I.run == 4 && I.order == 2 && n_cells > kWideMaxCells) I.run = 2;
       // one or two chunks (64 ordinates): a tile of 16 cells leaves half of a CTA's warps
       // without a chunk, which costs less than larger tiles only on small grids
       // (70^2 x 64 Heun: 35.4 us per step with 16, 38.5 with 32)

@@ -233,3 +233,20 @@ def test_second_order_triangles_with_denominators_below_the_fast_range(rt, M, sc
     op = oracle.TriangleOracle(p, oracle.product_quadrature(*M), order=2)
     ref, _, _ = oracle.run(op, psi0, dt, 3, "heun")
     assert rel_l2(psi, ref) <= PSI_TOL
+
+
+@pytest.mark.parametrize("order,tile_x", [(2, 16), (1, 32)])
+def test_tiles_of_256_ordinates_above_2_17_cells(rt, order, tile_x):
+    """371^2 cells, quadrants of 64 ordinates: second order takes 16-cell tiles, first
+    order 32-cell ones, and either agrees with the other width to FP32 rounding of a few
+    steps (each value's operations are the same; only phi's order of summation differs)."""
+    p = si.lattice_problem(371)
+    quad = rt.rt_quad_product(8, 32)
+    out = []
+    for tx in (0, 32 if tile_x == 16 else 16):
+        s = rt.Solver(p, quad, order=order, integrator=rt.RT_HEUN, dt=0.5 * p.mesh.dx, tile_x=tx)
+        assert s.info.tile_x == (tx or tile_x)
+        s.step(3)
+        out.append(s.phi())
+        s.close()
+    assert np.max(np.abs(out[0] - out[1])) <= 1e-6 * np.max(np.abs(out[1]))
