@@ -67,7 +67,7 @@ def bytes_per_update(order, integrator, storage, mesh="lattice"):
     return base
 
 
-KERNEL_SOURCES = {"cart": ["cart_kernel.cuh", "device_common.cuh"],
+KERNEL_SOURCES = {"cart": ["cart_stream.cuh", "cart_common.cuh", "device_common.cuh"],
                   "tri": ["tri_staged_kernel.cu", "tri_kernel.cu", "device_common.cuh"],
                   "tri2": ["tri2_kernel.cu", "device_common.cuh"]}
 
@@ -357,7 +357,7 @@ def run_ours(args, spec):
                      "frac": achieved_gbs / peak, "traffic": traffic,
                      "traffic_per": "step (all stage launches), DRAM read + write bytes",
                      "traffic_source": traffic_src,
-                     "kernel": {"cart": "cart_stage_kernel",
+                     "kernel": {"cart": "cart_stream_kernel" if info.variant == 2 or info.vec == 0 else "cart_stage_kernel",
                                 "tri": "tri_staged_kernel" if info.variant == 3 else "tri_stage_kernel",
                                 "tri2": "tri_grad_kernel + tri_stage2_kernel"}[kind],
                      "bytes_per_update": bpu, "peak_source": f"{peak_src} hbm_gbs",
@@ -553,7 +553,7 @@ def run_sweep(args, w):
         "qoi_max_rel_diff_batched_vs_plain": diff,
         "updates_per_s_batched": updates / tb,
         "roofline": {"bound": "hbm", "achieved": nbytes / tb / 1e9, "peak": peak, "unit": "GB/s",
-                     "frac": nbytes / tb / 1e9 / peak, "traffic": None, "kernel": "cart_stage_kernel (batched)",
+                     "frac": nbytes / tb / 1e9 / peak, "traffic": None, "kernel": "cart_stream_kernel (batched)",
                      "peak_source": peak_src},
         "e2e": {"value": k / tb, "unit": "solves/s", "h2d_bytes_per_step": None, "d2h_bytes_per_step": k * QOI_BYTES,
                 "includes": "batch creation from host arrays, all steps, QoI read-back, destroy"},

@@ -29,8 +29,8 @@
 // wait on a barrier is bounded; one that runs out stops the whole CTA at the next
 // block's end, drains the copies in flight and reports RT_ETIMEOUT.
 //
-// Bound by issue slots and fixed latencies at 16 warps per SM (270 instructions per
-// cell of 256 ordinates, 41 % of the slots; DRAM 8.1 bytes per cell and ordinate at
+// Bound by issue slots and fixed latencies at 16 warps per SM (256 instructions per
+// cell of 256 ordinates, 44 % of the slots; DRAM 8.1 bytes per cell and ordinate at
 // half of its peak). 1300^2 x 256 first-order Euler, FP32: with selects between the
 // traces, two barriers per block, one thread's QoI sums per cell and per-row bulk copies
 // (which a warp issues lane by lane) 2.28 ms; now 1.66. 650^2 x 256 BF16 0.61 -> 0.42.
