@@ -37,6 +37,18 @@
 // in fixed order at the end. The boundary outflow is taken from the stored rows after
 // the walk; the epilogue writes phi_out and the FP64 QoI partials.
 //
+// Ordered form (second order, grids of at most 1e5 cells; kOrderedMaxCells has the reason).
+// The sums above add differences, and phi in another order than the kernels that read whole
+// chunks of 32 V ordinates do (V ordinates per lane). Where runs are long enough for the
+// scheme to amplify that, the operations of those kernels are kept, value for value: face
+// values F = u + m/2 and G, then div = ax (F_1 - F_0) + ay (G_1 - G_0) with the last product
+// fused (y for per-lane directions, x for chunk-uniform ones), out = (a c + b) - div; and the
+// lanes leave their terms of phi in shared memory (128 bytes per cell, no shuffles in the
+// walk), which are then added in the order of a warp's butterfly over the chunk. The face
+// values take 8 more registers (spilled, mostly at sides), the terms limit a segment to 13
+// rows with two CTAs per SM. Per Heun step, sums of differences and ordered: 140^2 x 128 52
+// and 55 us, 280^2 x 256 163 and 180; the general kernel 111 and 320.
+//
 // Bound by: HBM on large grids (1400^2 x 512 FP32 Heun: 20 bytes per cell and ordinate
 // at 5.4 TB/s; a pair of rows is about 500 instructions for 16 values a lane, issue
 // slots half used), by instruction latency and the fixed cost of a launch on small ones.
@@ -61,6 +73,7 @@ constexpr int kStrWarps = kStrThreads / 32;
 constexpr int kStrRun = 2;                   // consecutive cells of a lane
 constexpr int kStrCells = 4 * kStrRun;       // cells of a warp's strip
 constexpr int kStrOrds = 32;                 // ordinates of a chunk
+enum StrForm { STR_DIFF = 0, STR_LANE = 1, STR_UNI = 2 };   // order of the operations (str_chunk)
 
 template <int ORDER, int STAGE, typename T>
 struct StrCfg {
@@ -82,15 +95,18 @@ struct StrCfg {
   static constexpr int last_lanes = (row_cells - (copies - 1) * per_copy) * pieces;   // lanes of the last copy
 };
 
-// (a, b) of every cell, and one phi accumulator per cell and chunk group
-__host__ __device__ inline size_t str_tile_bytes(int tx, int ly) {
-  return (size_t)ly * tx * 8 + (size_t)ly * kStrWarps * kStrCells * 4;
+// Floats per cell that hold the lanes' terms of phi in the ordered form (form: CartForm).
+__host__ __device__ inline int str_parts(int form) { return form & (16 | 32 | 64); }
+// (a, b) of every cell, and one phi accumulator per cell and chunk group; in the ordered
+// form one per cell, and the lanes' terms
+__host__ __device__ inline size_t str_tile_bytes(int tx, int ly, int parts) {
+  return (size_t)ly * tx * 8 + (parts ? (size_t)ly * tx * 4 * (1 + parts) : (size_t)ly * kStrWarps * kStrCells * 4);
 }
 constexpr size_t kStrRedBytes = (kStrWarps + 1) * NQ * 8;
 
 template <int ORDER, int STAGE, typename T>
-size_t str_smem_for(int tx, int ly) {
-  return StrCfg<ORDER, STAGE, T>::ring_bytes + str_tile_bytes(tx, ly) + kStrRedBytes + 128;
+size_t str_smem_for(int tx, int ly, int form) {
+  return StrCfg<ORDER, STAGE, T>::ring_bytes + str_tile_bytes(tx, ly, str_parts(form)) + kStrRedBytes + 128;
 }
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
@@ -117,6 +133,8 @@ struct StrWarp {
   uint8_t* ring_p;
   const float2* ab;    // [ly][TX] of the tile
   float* acc;          // [ly][TX] of the warp's chunk group
+  float* part;         // ordered form: the lanes' terms of phi, [ly][TX][parts]
+  int parts, slots;    // ordered form: floats per cell, and windows that they hold
   const StrEdge* ed;
   const uint8_t* src;  // the lane's piece of the strip's row 0, ordinate 0: copy 0 of the halo row
   int64_t to_base;     // from there to its piece of the row of psi^n beside it, in bytes (Heun stage 2)
@@ -190,8 +208,9 @@ __device__ __forceinline__ void str_load(const StrWarp& w, uint32_t dst, int kb,
   }
 }
 
-// Window of one row: values, difference to the row before along the flow, and the
-// flux terms known when the row arrives (all of x, and of y the face below it).
+// Window of one row: values, difference to the row before along the flow, and the flux
+// terms known when the row arrives (all of x, and of y the face below it); in the ordered
+// form the differences of the face values in x.
 struct StrRow {
   float2 c[kStrRun][2], d[kStrRun][2], z[kStrRun][2];
 };
@@ -200,10 +219,13 @@ struct StrRow {
 // rows are loaded while this one ends. EDGE: the strip with its halo touches a side of
 // the domain. Strips away from the sides have a body of their own: testing for the sides
 // in the row cost 48 of 291 instructions and 17 % of the time at 560^2 x 512.
-template <int ORDER, int STAGE, typename T, bool EDGE>
-__device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, const int4 ch, const int c_next, int& slot,
-                                          const int in_buf, T* __restrict__ psi_out,
+// FORM: STR_DIFF, or the ordered form with the operations of per-lane (STR_LANE) or of
+// chunk-uniform directions (STR_UNI) and with V ordinates per term of phi.
+template <int ORDER, int STAGE, typename T, bool EDGE, int FORM, int V>
+__device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, const int4 ch, const int c, const int c_next,
+                                          int& slot, const int in_buf, T* __restrict__ psi_out,
                                           [[maybe_unused]] const uint32_t salt) {
+  constexpr bool ORD = FORM != STR_DIFF;
   using L = StrCfg<ORDER, STAGE, T>;
   constexpr int H = L::H, R = kStrRun, NS = L::NS;
   constexpr int NU = R + H + ORDER - 1;   // cells read per row: -H .. R + ORDER - 2 along the flow
@@ -219,13 +241,13 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
   const int dys = ch.z;
   const int n = w.yb - w.ya + L::EXTRA;                // rows of the chunk
   const int npair = (n + 1) / 2;
-  const bool part = ch.y != (32 << 8);                 // a partial window
+  const bool part = !ORD && ch.y != (32 << 8);         // a partial window
 
   float2 w2[2], ax2[2], ay2[2];
   float xsum = 0.f;
   {
     const float dt = d.dt;
-    const float half = STAGE == STAGE_HEUN2 ? -0.5f : -1.f;   // stage 2 averages psi^n and the update
+    const float half = ORD ? 1.f : STAGE == STAGE_HEUN2 ? -0.5f : -1.f;   // stage 2 averages psi^n and the update
     const int lo = ch.x + (ch.y & 255), hi = ch.x + (ch.y >> 8);
     float wv[4], ax[4], ay[4];
 #pragma unroll
@@ -257,6 +279,21 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
   const int mstep = dxs * d.Mpad;
   const float2* tab = w.ab + (start - w.ya) * w.TX - L::EXTRA * astep + w.xl + s0;
   float* tacc = w.acc + (start - w.ya) * w.TX - L::EXTRA * astep + w.xl + R * grp + (l8 >> 2) + ((l8 >> 1) & 1) * astep;
+  // ordered form: the lane's terms of the row's cells (a pair of cells has 2 parts floats in
+  // blocks of 32 / V, rotated by the pair so that the four of a row lie in different banks)
+  [[maybe_unused]] float* tpart = nullptr;
+  [[maybe_unused]] int poff[R], pstep = 0;
+  [[maybe_unused]] bool second = false;   // the term is added to that of the window 64 ordinates before
+  if constexpr (ORD) {
+    static_assert(R == 2, "pairs of cells");
+    const int wslot = c & (w.slots - 1);
+    tpart = w.part + ((start - w.ya) * w.TX - L::EXTRA * astep + w.xl + R * grp) * w.parts + l8 * (4 / V);
+    pstep = astep * w.parts;
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+      poff[r] = (((dxs > 0 ? r : 1 - r) * w.slots + wslot + grp) & (2 * w.slots - 1)) * (32 / V);
+    second = V == 4 && w.slots == 2 && (c & 2);
+  }
   const bool odd = part || w.xw + kStrCells > d.nx;    // a partial window, or the domain ends inside the strip
 
   // strips at an x side: which cells of a row lie outside (bits m), which of them upstream
@@ -275,6 +312,7 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
   // Row i of the chunk arrives in X; Y holds the row before it, which is completed
   // here (second order; first order completes the row itself). c: w-weighted sums of
   // the completed cells.
+  [[maybe_unused]] float2 G[R][2];   // ordered form: y face values before the row that is completed next
   auto row = [&](const int i, const int in_slot, const bool done, StrRow& X, const StrRow& Y, float (&c)[R]) {
     const uint8_t* cur = ring_l + in_slot;
     float2 u[NU][2];
@@ -316,41 +354,74 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
     }
     float2 out[R][2];
     const StrRow& C = ORDER == 2 ? Y : X;   // the row completed
+    if constexpr (ORD) {
 #pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      // x: the flux terms of the row
-      float2 D[NU];   // D[m] = u[m] - u[m-1]
-      [[maybe_unused]] float2 M[R + 1];
+      for (int v = 0; v < 2; ++v) {
+        float2 D[NU], RD[NU], F[R + 1];   // F: face before cell f
 #pragma unroll
-      for (int m = 1; m < NU; ++m) D[m] = sub2(u[m][v], u[m - 1][v]);
-      if constexpr (ORDER == 2) {
-        float2 RD[NU];
+        for (int m = 1; m < NU; ++m) {
+          D[m] = sub2(u[m][v], u[m - 1][v]);
+          RD[m] = relu2(D[m]);
+        }
 #pragma unroll
-        for (int m = 1; m < NU; ++m) RD[m] = relu2(D[m]);
+        for (int f = 0; f <= R; ++f) {
+          float2 M = minmod2r(D[f + 2], D[f + 1], RD[f + 2], RD[f + 1]);
+          if (EDGE && (xbits >> (16 + f) & 1)) M = make_float2(0.f, 0.f);   // domain faces are first order
+          F[f] = __ffma2_rn(make_float2(0.5f, 0.5f), M, u[f + 1][v]);
+        }
 #pragma unroll
-        for (int f = 0; f <= R; ++f) M[f] = minmod2r(D[f + 2], D[f + 1], RD[f + 2], RD[f + 1]);   // face before cell f
-        if constexpr (EDGE) {   // domain faces are first order
-#pragma unroll
-          for (int f = 0; f <= R; ++f)
-            if (xbits >> (16 + f) & 1) M[f] = make_float2(0.f, 0.f);
+        for (int r = 0; r < R; ++r) {
+          X.z[r][v] = sub2(F[r + 1], F[r]);
+          X.c[r][v] = u[r + H][v];
+          X.d[r][v] = sub2(X.c[r][v], Y.c[r][v]);
+          float2 M = minmod2r(X.d[r][v], Y.d[r][v], relu2(X.d[r][v]), relu2(Y.d[r][v]));
+          if (EDGE && !face2) M = make_float2(0.f, 0.f);
+          float2 up = Y.c[r][v];   // the face's upwind value; the general kernel walks +y whatever the flow
+          if (FORM == STR_LANE && dys < 0) up = sub2(X.c[r][v], X.d[r][v]);
+          const float2 g = __ffma2_rn(make_float2(0.5f, 0.5f), M, up);
+          const float2 dg = sub2(g, G[r][v]);
+          G[r][v] = g;
+          out[r][v] = FORM == STR_UNI ? __ffma2_rn(ax2[v], Y.z[r][v], __fmul2_rn(ay2[v], dg))
+                                      : __ffma2_rn(ay2[v], dg, __fmul2_rn(ax2[v], Y.z[r][v]));
         }
       }
+    } else {
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        float2 g = D[r + H];
-        if constexpr (ORDER == 2) g = __ffma2_rn(make_float2(0.5f, 0.5f), sub2(M[r + 1], M[r]), g);
-        float2 z = __fmul2_rn(ax2[v], g);
-        // y: difference to the row before, half the limited difference at the face between them
-        X.c[r][v] = u[r + H][v];
-        X.d[r][v] = sub2(X.c[r][v], Y.c[r][v]);
+      for (int v = 0; v < 2; ++v) {
+        // x: the flux terms of the row
+        float2 D[NU];   // D[m] = u[m] - u[m-1]
+        [[maybe_unused]] float2 M[R + 1];
+#pragma unroll
+        for (int m = 1; m < NU; ++m) D[m] = sub2(u[m][v], u[m - 1][v]);
         if constexpr (ORDER == 2) {
-          float2 h = __fmul2_rn(make_float2(0.5f, 0.5f),
-                                minmod2r(X.d[r][v], Y.d[r][v], relu2(X.d[r][v]), relu2(Y.d[r][v])));
-          if (EDGE && !face2) h = make_float2(0.f, 0.f);
-          out[r][v] = __ffma2_rn(ay2[v], h, Y.z[r][v]);
-          X.z[r][v] = __ffma2_rn(ay2[v], sub2(X.d[r][v], h), z);
-        } else {
-          out[r][v] = __ffma2_rn(ay2[v], X.d[r][v], z);
+          float2 RD[NU];
+#pragma unroll
+          for (int m = 1; m < NU; ++m) RD[m] = relu2(D[m]);
+#pragma unroll
+          for (int f = 0; f <= R; ++f) M[f] = minmod2r(D[f + 2], D[f + 1], RD[f + 2], RD[f + 1]);   // face before cell f
+          if constexpr (EDGE) {   // domain faces are first order
+#pragma unroll
+            for (int f = 0; f <= R; ++f)
+              if (xbits >> (16 + f) & 1) M[f] = make_float2(0.f, 0.f);
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          float2 g = D[r + H];
+          if constexpr (ORDER == 2) g = __ffma2_rn(make_float2(0.5f, 0.5f), sub2(M[r + 1], M[r]), g);
+          float2 z = __fmul2_rn(ax2[v], g);
+          // y: difference to the row before, half the limited difference at the face between them
+          X.c[r][v] = u[r + H][v];
+          X.d[r][v] = sub2(X.c[r][v], Y.c[r][v]);
+          if constexpr (ORDER == 2) {
+            float2 h = __fmul2_rn(make_float2(0.5f, 0.5f),
+                                  minmod2r(X.d[r][v], Y.d[r][v], relu2(X.d[r][v]), relu2(Y.d[r][v])));
+            if (EDGE && !face2) h = make_float2(0.f, 0.f);
+            out[r][v] = __ffma2_rn(ay2[v], h, Y.z[r][v]);
+            X.z[r][v] = __ffma2_rn(ay2[v], sub2(X.d[r][v], h), z);
+          } else {
+            out[r][v] = __ffma2_rn(ay2[v], X.d[r][v], z);
+          }
         }
       }
     }
@@ -364,7 +435,10 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
           float2 t = __ffma2_rn(make_float2(ab.x, ab.x), C.c[r][v], make_float2(ab.y, ab.y));
-          if constexpr (STAGE == STAGE_HEUN2) {
+          if constexpr (ORD) {
+            t = sub2(t, out[r][v]);
+            out[r][v] = STAGE == STAGE_HEUN2 ? __fmul2_rn(make_float2(0.5f, 0.5f), __fadd2_rn(base[v], t)) : t;
+          } else if constexpr (STAGE == STAGE_HEUN2) {
             out[r][v] = __ffma2_rn(make_float2(0.5f, 0.5f), __fadd2_rn(base[v], t), out[r][v]);
           } else {
             out[r][v] = __fadd2_rn(t, out[r][v]);
@@ -398,6 +472,32 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
     }
     op += ostep;
     tab += astep;
+    if constexpr (ORD) {
+      if (done) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          float* p = tpart + poff[r];
+          const float2 p0 = __fmul2_rn(w2[0], out[r][0]);
+          if constexpr (V == 4) {
+            float t;
+            if constexpr (FORM == STR_UNI) {
+              const float2 pw = __ffma2_rn(w2[1], out[r][1], p0);
+              t = pw.x + pw.y;
+            } else {
+              t = fmaf(w2[1].y, out[r][1].y, fmaf(w2[1].x, out[r][1].x, fmaf(w2[0].y, out[r][0].y, p0.x)));
+            }
+            *p = second ? *p + t : t;
+          } else {
+            const float2 p1 = __fmul2_rn(w2[1], out[r][1]);
+            *reinterpret_cast<float2*>(p) =
+                FORM == STR_UNI ? make_float2(p0.x + p0.y, p1.x + p1.y)
+                                : make_float2(fmaf(w2[0].y, out[r][0].y, p0.x), fmaf(w2[1].y, out[r][1].y, p1.x));
+          }
+        }
+      }
+      tpart += pstep;
+      return;
+    }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const float2 pw = __ffma2_rn(w2[1], out[r][1], __fmul2_rn(w2[0], out[r][0]));
@@ -409,7 +509,7 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
 #pragma unroll
   for (int r = 0; r < R; ++r)
 #pragma unroll
-    for (int v = 0; v < 2; ++v) B.c[r][v] = B.d[r][v] = B.z[r][v] = make_float2(0.f, 0.f);
+    for (int v = 0; v < 2; ++v) B.c[r][v] = B.d[r][v] = B.z[r][v] = G[r][v] = make_float2(0.f, 0.f);
 #pragma unroll 1
   for (int q = 0; q < npair; ++q) {
     if (NS > 2 && w.ahead == NS - 1) cp_async_wait<NS - 2>();
@@ -432,6 +532,7 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
     float c0[R], c1[R];
     row(i, in_slot, done0, A, B, c0);
     row(i + 1, in_slot + L::row_bytes, done1, B, A, c1);
+    if constexpr (ORD) continue;
     // phi of both completed rows, summed over the pair's 8 lanes: lanes 0, 1 end with the left cell of
     // the first row, 2, 3 with that of the second, 4 .. 7 with the right ones (a cell beyond a ragged
     // edge has an accumulator that nothing reads)
@@ -444,6 +545,76 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
     if ((lane & 1) == 0 && (h2 ? done1 : done0)) *tacc += s;
     tacc += 2 * astep;
   }
+}
+
+// Barrier of the WC warps of strip wx (at most four strips; the ids are constants, so that
+// a CTA reserves no more barriers than these).
+__device__ __forceinline__ void str_strip_barrier(int wx, int WC) {
+  const int threads = 32 * WC;
+  if (wx == 0) asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+  else if (wx == 1) asm volatile("bar.sync 2, %0;" ::"r"(threads) : "memory");
+  else if (wx == 2) asm volatile("bar.sync 3, %0;" ::"r"(threads) : "memory");
+  else asm volatile("bar.sync 4, %0;" ::"r"(threads) : "memory");
+}
+
+// Ordered form: phi of the strip's cells from the lanes' terms of `n` windows, added to acc.
+// A lane of the kernel whose order is kept holds V consecutive ordinates of a chunk of 32 V,
+// and a warp's butterfly adds lanes 16 apart, then 8, 4, 2 and 1: the same tree here, windows
+// first. The WC warps of the strip (this one is wc) share the cells.
+template <int V>
+__device__ __forceinline__ void str_phi_ordered(const StrWarp& w, int wc, int WC, int n) {
+  const int lane = threadIdx.x & 31, l8 = lane & 7, grp = lane >> 3;
+  const int mask = 2 * w.slots - 1;
+#pragma unroll 2
+  for (int i = wc; i < kStrRun * (w.yb - w.ya); i += WC) {
+    const int phys = i & 1, pair = (i >> 1) * w.TX + w.xl + kStrRun * grp;
+    const float* p = w.part + pair * w.parts + l8 * (4 / V);
+    auto at = [&](int slot) { return p + ((phys * w.slots + slot + grp) & mask) * (32 / V); };
+    float a = w.acc[pair + phys];
+    if constexpr (V == 4) {
+      float s = w.slots == 4 ? (*at(0) + *at(2)) + (*at(1) + *at(3)) : *at(0) + *at(1);
+      s += __shfl_xor_sync(0xffffffffu, s, 4);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      a += s;
+    } else {
+      for (int k = 0; k < n; k += 2) {
+        float2 s = __fadd2_rn(*reinterpret_cast<const float2*>(at(k)), *reinterpret_cast<const float2*>(at(k + 1)));
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+          s = __fadd2_rn(s, make_float2(__shfl_xor_sync(0xffffffffu, s.x, o), __shfl_xor_sync(0xffffffffu, s.y, o)));
+        a += s.x + s.y;
+      }
+    }
+    if (l8 == 0) w.acc[pair + phys] = a;
+  }
+}
+
+// Ordered form: the chunks of a warp. The warps of a strip meet where their windows complete
+// chunks of 32 V ordinates.
+template <int STAGE, typename T, int FORM, int V>
+__device__ __forceinline__ void str_chunks_ordered(const InstDesc& d, const StrWarp& w, int wx, int wc, int WC, bool active,
+                                                   bool edge, int in_buf, T* __restrict__ psi_out, uint32_t salt) {
+  const int per = max(V, WC), n_chunks = d.n_chunks;
+  if (active) {
+    int slot = 0;
+#pragma unroll 1
+    for (int c = wc; c < n_chunks; c += WC) {
+      const int4 ch = d.str_chunks[c];
+      if (edge) str_chunk<2, STAGE, T, true, FORM, V>(d, w, ch, c, c + WC, slot, in_buf, psi_out, salt);
+      else str_chunk<2, STAGE, T, false, FORM, V>(d, w, ch, c, c + WC, slot, in_buf, psi_out, salt);
+      const int next = c - wc + WC;   // first window of the strip's next round
+      if (next % per == 0 && next < n_chunks) {
+        str_strip_barrier(wx, WC);
+        str_phi_ordered<V>(w, wc, WC, per);
+        str_strip_barrier(wx, WC);
+      }
+    }
+    cp_async_wait<0>();
+  }
+  __syncthreads();
+  str_phi_ordered<V>(w, wc, WC, n_chunks - (n_chunks - 1) / per * per);
+  __syncthreads();
 }
 
 // Boundary outflow of a tile's output state (first-order traces: what leaves through a
@@ -477,10 +648,11 @@ __device__ __noinline__ float str_boundary(const InstDesc& d, const T* psi, int 
   return bacc;
 }
 
-template <int ORDER, int STAGE, typename T>
+template <int ORDER, int STAGE, typename T, int FORM>
 __global__ void __launch_bounds__(kStrThreads, 2)
     cart_stream_kernel(const InstDesc* __restrict__ descs, const WorkItem* __restrict__ items) {
   using L = StrCfg<ORDER, STAGE, T>;
+  constexpr bool ORD = FORM != STR_DIFF;
   const WorkItem it = items[blockIdx.x];
   const InstDesc& d = descs[it.inst];
   InstState* st = d.st;
@@ -510,14 +682,18 @@ __global__ void __launch_bounds__(kStrThreads, 2)
   const int x0 = it.a * TX, ya = it.b * d.ly, yb = min(ny, ya + d.ly), nrows = yb - ya;
 
   float2* tile_ab = reinterpret_cast<float2*>(smem + L::ring_bytes);
-  float* tile_acc = reinterpret_cast<float*>(tile_ab + d.ly * TX);   // [WC][ly][TX]
-  double* red = reinterpret_cast<double*>(smem + L::ring_bytes + str_tile_bytes(TX, d.ly));
+  float* tile_acc = reinterpret_cast<float*>(tile_ab + d.ly * TX);   // [WC][ly][TX]; ordered form [ly][TX]
+  const int parts = ORD ? d.ord_parts : 0;
+  double* red = reinterpret_cast<double*>(smem + L::ring_bytes + str_tile_bytes(TX, d.ly, parts));
 
   StrWarp w;
   w.ring_p = smem + warp * (L::NS * 2 * L::row_bytes);
   w.ring = smem_u32(w.ring_p);
   w.ab = tile_ab;
-  w.acc = tile_acc + wc * d.ly * TX;
+  w.acc = tile_acc + (ORD ? 0 : wc * d.ly * TX);
+  w.part = tile_acc + d.ly * TX;
+  w.parts = parts;
+  w.slots = ORD ? parts * d.ord_vec / 32 : 0;
   w.ed = &s_edge;
   w.xl = wx * kStrCells;
   w.xw = x0 + w.xl;
@@ -564,24 +740,31 @@ __global__ void __launch_bounds__(kStrThreads, 2)
     }
     tile_ab[i] = make_float2(a, b);
   }
-  for (int i = tid; i < WC * d.ly * TX; i += kStrThreads) tile_acc[i] = 0.f;
+  for (int i = tid; i < (ORD ? 1 : WC) * d.ly * TX; i += kStrThreads) tile_acc[i] = 0.f;
   __syncthreads();
 
-  if (active) {
-    int slot = 0;
+  const int n_chunks = d.n_chunks;
+  if constexpr (ORD) {
+    if (d.ord_vec == 4) str_chunks_ordered<STAGE, T, FORM, 4>(d, w, wx, wc, WC, active, edge, in_buf, psi_out, salt);
+    else str_chunks_ordered<STAGE, T, FORM, 2>(d, w, wx, wc, WC, active, edge, in_buf, psi_out, salt);
+  } else {
+    if (active) {
+      int slot = 0;
 #pragma unroll 1
-    for (int c = wc; c < d.n_chunks; c += WC) {
-      if (edge) str_chunk<ORDER, STAGE, T, true>(d, w, d.str_chunks[c], c + WC, slot, in_buf, psi_out, salt);
-      else str_chunk<ORDER, STAGE, T, false>(d, w, d.str_chunks[c], c + WC, slot, in_buf, psi_out, salt);
+      for (int c = wc; c < n_chunks; c += WC) {
+        const int4 ch = d.str_chunks[c];
+        if (edge) str_chunk<ORDER, STAGE, T, true, STR_DIFF, 4>(d, w, ch, c, c + WC, slot, in_buf, psi_out, salt);
+        else str_chunk<ORDER, STAGE, T, false, STR_DIFF, 4>(d, w, ch, c, c + WC, slot, in_buf, psi_out, salt);
+      }
+      cp_async_wait<0>();
     }
-    cp_async_wait<0>();
-  }
-  __syncthreads();
-  // phi of a cell: its chunk groups in order
-  for (int i = tid; i < nrows * TX; i += kStrThreads) {
-    float s = tile_acc[i];
-    for (int g = 1; g < WC; ++g) s += tile_acc[g * d.ly * TX + i];
-    tile_acc[i] = s;   // read back by the same thread only
+    __syncthreads();
+    // phi of a cell: its chunk groups in order
+    for (int i = tid; i < nrows * TX; i += kStrThreads) {
+      float s = tile_acc[i];
+      for (int g = 1; g < WC; ++g) s += tile_acc[g * d.ly * TX + i];
+      tile_acc[i] = s;   // read back by the same thread only
+    }
   }
   const int x1 = min(nx, x0 + TX);
   float bacc = 0.f;
@@ -590,19 +773,19 @@ __global__ void __launch_bounds__(kStrThreads, 2)
                                     L::ring_bytes / 4, x0, ya, nrows, TX, bacc);
 }
 
-template <int ORDER, int STAGE, typename T>
-static cudaError_t str_prepare_one(int tx, int ly) {
+template <int ORDER, int STAGE, typename T, int FORM>
+static cudaError_t str_prepare_one(int tx, int ly, int form) {
   // The dynamic shared-memory limit belongs to the current device and the kernel;
   // it is only ever raised (atomics: host threads may race here, harmlessly).
   constexpr int kDev = 64;
   static std::atomic<size_t> s_limit[kDev];
-  const size_t smem = str_smem_for<ORDER, STAGE, T>(tx, ly);
+  const size_t smem = str_smem_for<ORDER, STAGE, T>(tx, ly, form);
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const bool tracked = dev >= 0 && dev < kDev;
   if (tracked && smem <= s_limit[dev].load(std::memory_order_acquire)) return cudaSuccess;
-  e = cudaFuncSetAttribute(cart_stream_kernel<ORDER, STAGE, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = cudaFuncSetAttribute(cart_stream_kernel<ORDER, STAGE, T, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (tracked) {
     size_t cur = s_limit[dev].load(std::memory_order_relaxed);
@@ -612,26 +795,50 @@ static cudaError_t str_prepare_one(int tx, int ly) {
   return cudaSuccess;
 }
 
+template <int ORDER, int STAGE, typename T, int FORM>
+static cudaError_t str_launch_one(const InstDesc* d, const WorkItem* items, int n, int tx, int ly, int form, cudaStream_t s,
+                                  bool chained) {
+  cudaError_t e = str_prepare_one<ORDER, STAGE, T, FORM>(tx, ly, form);
+  if (e != cudaSuccess) return e;
+  return launch_stage_kernel(cart_stream_kernel<ORDER, STAGE, T, FORM>, n, kStrThreads,
+                             str_smem_for<ORDER, STAGE, T>(tx, ly, form), s, chained, d, items);
+}
+
+// Calls FN<..., FORM>(args) for the kernel of `form` (the ordered form: second order only).
+#define RTK_STR_FORM(FN, ...)                                                     \
+  if (form == STREAM_PLAIN) return FN<ORDER, STAGE, T, STR_DIFF>(__VA_ARGS__);    \
+  if constexpr (ORDER == 2) {                                                     \
+    if (form & STREAM_UNI) return FN<ORDER, STAGE, T, STR_UNI>(__VA_ARGS__);      \
+    return FN<ORDER, STAGE, T, STR_LANE>(__VA_ARGS__);                            \
+  }                                                                               \
+  return cudaErrorInvalidValue;
+template <int ORDER, int STAGE, typename T>
+static cudaError_t str_prepare(int tx, int ly, int form) {
+  RTK_STR_FORM(str_prepare_one, tx, ly, form)
+}
+template <int ORDER, int STAGE, typename T>
+static cudaError_t str_launch(const InstDesc* d, const WorkItem* items, int n, int tx, int ly, int form, cudaStream_t s,
+                              bool chained) {
+  RTK_STR_FORM(str_launch_one, d, items, n, tx, ly, form, s, chained)
+}
+#undef RTK_STR_FORM
+
 // One translation unit per (order, storage type): the three stages.
 #define RTK_STR_UNIT(NAME, ORDER, TT)                                                                         \
-  cudaError_t str_prepare_##NAME(int stage, int tx, int ly) {                                                 \
-    if (stage == STAGE_EULER) return str_prepare_one<ORDER, STAGE_EULER, TT>(tx, ly);                         \
-    if (stage == STAGE_HEUN1) return str_prepare_one<ORDER, STAGE_HEUN1, TT>(tx, ly);                         \
-    return str_prepare_one<ORDER, STAGE_HEUN2, TT>(tx, ly);                                                   \
+  cudaError_t str_prepare_##NAME(int stage, int tx, int ly, int form) {                                       \
+    if (stage == STAGE_EULER) return str_prepare<ORDER, STAGE_EULER, TT>(tx, ly, form);                       \
+    if (stage == STAGE_HEUN1) return str_prepare<ORDER, STAGE_HEUN1, TT>(tx, ly, form);                       \
+    return str_prepare<ORDER, STAGE_HEUN2, TT>(tx, ly, form);                                                 \
   }                                                                                                           \
-  size_t str_smem_##NAME(int stage, int tx, int ly) {                                                         \
-    return stage == STAGE_HEUN2 ? str_smem_for<ORDER, STAGE_HEUN2, TT>(tx, ly)                                \
-                                : str_smem_for<ORDER, STAGE_EULER, TT>(tx, ly);                               \
+  size_t str_smem_##NAME(int stage, int tx, int ly, int form) {                                               \
+    return stage == STAGE_HEUN2 ? str_smem_for<ORDER, STAGE_HEUN2, TT>(tx, ly, form)                          \
+                                : str_smem_for<ORDER, STAGE_EULER, TT>(tx, ly, form);                         \
   }                                                                                                           \
   cudaError_t str_launch_##NAME(const InstDesc* d, const WorkItem* items, int n, int stage, int tx, int ly,   \
-                                cudaStream_t s, bool chained) {                                               \
-    cudaError_t e = str_prepare_##NAME(stage, tx, ly);                                                        \
-    if (e != cudaSuccess) return e;                                                                           \
-    const size_t smem = str_smem_##NAME(stage, tx, ly);                                                       \
-    return launch_stage_kernel(stage == STAGE_EULER   ? cart_stream_kernel<ORDER, STAGE_EULER, TT>            \
-                               : stage == STAGE_HEUN1 ? cart_stream_kernel<ORDER, STAGE_HEUN1, TT>            \
-                                                      : cart_stream_kernel<ORDER, STAGE_HEUN2, TT>,           \
-                               n, kStrThreads, smem, s, chained, d, items);                                   \
+                                int form, cudaStream_t s, bool chained) {                                     \
+    if (stage == STAGE_EULER) return str_launch<ORDER, STAGE_EULER, TT>(d, items, n, tx, ly, form, s, chained); \
+    if (stage == STAGE_HEUN1) return str_launch<ORDER, STAGE_HEUN1, TT>(d, items, n, tx, ly, form, s, chained); \
+    return str_launch<ORDER, STAGE_HEUN2, TT>(d, items, n, tx, ly, form, s, chained);                         \
   }
 
 }  // namespace rtk

@@ -483,6 +483,14 @@ static std::vector<int4> plan_stream_chunks(const rt_quadrature* quad, int Mpad,
   return a;
 }
 
+// Whether the streaming kernel's windows are whole and aligned, in the order of the ordinates.
+static bool windows_whole(const std::vector<int4>& chunks, int Mpad) {
+  if ((int64_t)chunks.size() * 32 != Mpad) return false;
+  for (size_t c = 0; c < chunks.size(); ++c)
+    if (chunks[c].x != 32 * (int)c || chunks[c].y != (32 << 8)) return false;
+  return true;
+}
+
 // Resident CTAs per SM of the general Cartesian kernel at segment length ly: the
 // kernel's launch bound (2 with 8 values per thread and row, else 3) and its shared
 // memory (the Heun stage 2 ring is the largest).
@@ -551,9 +559,11 @@ static bool regroup_quadrature(const rt_quadrature* quad, std::vector<double>& x
 // more, to neighbouring strips whose rows have left L2 and to SMs that finish early, than
 // their shared rows save (1400^2 x 512 Heun 3745 us at 61 rows, 3590 at 37; 911^2 x 196 BF16
 // 1078 at 57, 976 at 44). Against timings of 29 problems at 3 to 64 rows (70^2 x 64 to
-// 1400^2 x 512) its choice is 4 % from the best on average, 14 % at most. *cost receives
-// the model's time.
-static int stream_segment(const Instance& I, int run, double* cost) {
+// 1400^2 x 512) its choice is 4 % from the best on average, 14 % at most. The ordered form's
+// few items come in whole rounds (280^2 x 256 Heun: 576 items of 9 rows 173 us, 504 of 10 rows
+// 192): 2 % from the best of 3 to 13 rows on average over 21 problems of 50^2 x 64 to
+// 280^2 x 512. *cost receives the model's time.
+static int stream_segment(const Instance& I, int run, int form, double* cost) {
   const int sms = device_sm_count();
   const int tx = cart_tile_width(run), groups = cart_stream_chunk_groups(tx);
   const int64_t strips = (I.nx + tx - 1) / tx;
@@ -564,7 +574,7 @@ static int stream_segment(const Instance& I, int run, double* cost) {
   const int ly_most = I.str_chunks.size() > 1 ? 40 : 64;
   for (int ly = 3; ly <= ly_most; ++ly) {
     // two CTAs per SM by shared memory (228 KB, 1 KB of it per CTA reserved)
-    if (cart_smem_bytes(I.order, I.storage, run, I.cvec, ly, stage_hi, 1) > 113 * 1024) break;
+    if (cart_smem_bytes(I.order, I.storage, run, I.cvec, ly, stage_hi, form) > 113 * 1024) break;
     const int64_t items = strips * ((I.ny + ly - 1) / ly);
     const int rows = (std::min(ly, I.ny) + (I.order == 2 ? 3 : 1) + 1) / 2 * 2;
     double t;
@@ -573,7 +583,8 @@ static int stream_segment(const Instance& I, int run, double* cost) {
     } else if (items <= 2 * sms) {
       t = 12.0 + 1.28 * chunks * rows;
     } else {
-      t = (7.0 + 1.28 * chunks * rows) * ((double)items / (2.0 * sms) + 0.5);
+      const double rounds = (double)items / (2.0 * sms);
+      t = (7.0 + 1.28 * chunks * rows) * (form == STREAM_PLAIN ? rounds + 0.5 : std::ceil(rounds));
     }
     if (t < *cost) {
       *cost = t;
@@ -583,11 +594,31 @@ static int stream_segment(const Instance& I, int run, double* cost) {
   return best;
 }
 
+// Whether a Cartesian problem's results keep the order of operations of the kernel that
+// reads whole chunks of 32 `vec` ordinates at once. Second order at the default time step is
+// not a contraction (a cell's weight reaches 0.75 (|xi| + |eta|) + dt sigma_t > 1), so the
+// limiters amplify rounding from step to step: with phi summed in another order single values
+// differ by 1e-5 after 32 Heun steps and by up to 2e-3 after 96 on lattices of 140^2 to 280^2
+// cells (relative L2 of psi 1e-7 and 3e-6; both are as far from FP64). Small grids are those
+// that run for hundreds of steps, so there the streaming kernel takes its ordered form where
+// the windows are whole, and per-lane directions that allow no such form (one ordinate per
+// lane) stay on the general kernel. First order contracts, and keeps to rounding anyway.
+constexpr int64_t kOrderedMaxCells = 100000;
+
+// Form of the streaming kernel (CartForm) for tiles of `run`: the ordered one if I.ord_vec is
+// set. A cell holds the terms of the windows that its column's warps compute at a time; two
+// warps (32-cell tiles) add the four windows of 4 ordinates per lane in place, in pairs.
+static int ordered_form(const Instance& I, int run) {
+  if (!I.ord_vec) return STREAM_PLAIN;
+  const int windows = std::min(cart_stream_chunk_groups(cart_tile_width(run)), (int)I.str_chunks.size());
+  return 32 / I.ord_vec * windows + (I.info_variant == 2 ? STREAM_UNI : 0);
+}
+
 static void choose_cart_tiles(Instance& I, int tile_y) {
   int ly = tile_y;
   if (ly <= 0 && I.uni) {
     double cost;
-    ly = stream_segment(I, I.run, &cost);
+    ly = stream_segment(I, I.run, I.uni, &cost);
   }
   I.tx = cart_tile_width(I.run);
   I.n_strips = (I.nx + I.tx - 1) / I.tx;
@@ -818,6 +849,18 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
     I.info_variant = I.uni ? 2 : 1;
     I.info_vec = I.cvec;
     if (I.uni || vec == 0) I.str_chunks = plan_stream_chunks(quad, I.Mpad, storage);
+    // whether as long a segment as asked for fits the shared memory of a CTA
+    auto fits = [&](int run) {
+      const int stage_hi = integrator == RT_HEUN ? STAGE_HEUN2 : STAGE_EULER;
+      return tile_y <= 0 || cart_smem_bytes(order, storage, run, 4, std::min(tile_y, 256), stage_hi,
+                                            ordered_form(I, run)) <= 227 * 1024;
+    };
+    I.ord_vec = 0;
+    if (order == 2 && n_cells <= kOrderedMaxCells && !I.str_chunks.empty()) {
+      if (I.cvec > 1 && windows_whole(I.str_chunks, I.Mpad)) I.ord_vec = I.cvec;
+      if (I.ord_vec && !fits(I.run)) I.ord_vec = 0;
+      if (!I.ord_vec && !I.uni) I.str_chunks.clear();
+    }
     if (!I.str_chunks.empty()) {
       if (!I.uni) I.info_vec = 0;
       I.uni = 1;
@@ -825,13 +868,15 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
       if (tile_x == 0 && I.run == 4 && I.order == 2 && n_cells > kWideMaxCells) I.run = 2;
       // one or two chunks (64 ordinates): a tile of 16 cells leaves half of a CTA's warps
       // without a chunk, which costs less than larger tiles only on small grids
-      // (70^2 x 64 Heun: 35.4 us per step with 16, 38.5 with 32)
-      if (tile_x == 0 && I.run == 2 && I.str_chunks.size() <= 2) {
+      // (70^2 x 64 Heun: 35.4 us per step with 16, 38.5 with 32); the ordered form gains up to
+      // four (280^2 x 128: 103 us with 16, 96 with 32), and no more beyond (280^2 x 512: 294, 342)
+      if (tile_x == 0 && I.run == 2 && I.str_chunks.size() <= (I.ord_vec ? 4u : 2u)) {
         double narrow, wider;
-        stream_segment(I, 2, &narrow);
-        stream_segment(I, 4, &wider);
-        if (wider < narrow) I.run = 4;
+        stream_segment(I, 2, ordered_form(I, 2), &narrow);
+        stream_segment(I, 4, ordered_form(I, 4), &wider);
+        if (wider < narrow && fits(4)) I.run = 4;
       }
+      I.uni = ordered_form(I, I.run);
     } else {
       I.uni = 0;
       I.run = 2;
@@ -1059,6 +1104,8 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
   D.n_chunks = I.kind != RT_MESH_CARTESIAN ? I.Mpad / kChunk
                : I.uni ? (int32_t)I.str_chunks.size() : I.Mpad / (32 * I.cvec);
   D.str_chunks = d_str_chunks;
+  D.ord_vec = I.uni >= 16 ? I.ord_vec : 0;
+  D.ord_parts = I.uni & ~STREAM_UNI;
   D.tx = I.tx; D.ly = I.ly; D.n_strips = I.n_strips;
   D.n_segs = I.n_segs; D.n_items = (int32_t)I.stage_items.size(); D.n_regions = I.n_regions;
   D.n_cells = n_cells; D.n_steps = I.n_steps;

@@ -51,7 +51,8 @@ struct Instance {
   int32_t run = 2, cvec = 1;        // Cartesian kernels: tile width / 8, ordinates per lane
   int32_t info_variant = 0, info_vec = 0;   // Cartesian: rt_info_t.variant and vec
   std::vector<int4> str_chunks;     // streaming Cartesian kernel: its ordinate chunks
-  int32_t uni = 0;                  // Cartesian: 1 = streaming kernel (tile width 8 run); triangles (first
+  int32_t ord_vec = 0;              // ... in its ordered form: ordinates per lane whose order of sums is kept
+  int32_t uni = 0;                  // Cartesian: CartForm (streaming: tile width 8 run); triangles (first
                                     // order): 1 = staged kernel (ly then holds the largest chunk halo)
   int32_t staged_ok = 0;            // triangles: the staged kernel's metadata exists (test hook switches)
   // ordinate layout: 0 the caller's order; 1 regrouped by direction quadrant,

@@ -30,6 +30,10 @@ constexpr int kMaxUniChunks = 64;      // chunk-uniform directions: at most this
 constexpr int kTriStgChunk = 32;       // cells per chunk of the staged first-order triangle kernel
 
 enum Stage : int32_t { STAGE_EULER = 0, STAGE_HEUN1 = 1, STAGE_HEUN2 = 2, STAGE_INIT = 3 };
+// Cartesian kernels (the launchers' `uni`): the general one, the streaming one, and the
+// latter in its ordered form: 16, 32 or 64 (floats per cell that hold the lanes' terms of
+// phi in shared memory), + STREAM_UNI with the operations of chunk-uniform directions.
+enum CartForm : int32_t { CART_GENERAL = 0, STREAM_PLAIN = 1, STREAM_UNI = 1 };
 enum Kind : int32_t { KIND_CART = 0, KIND_TRI = 1 };
 
 // Status codes written by kernels (same values as rt_status).
@@ -74,7 +78,10 @@ struct alignas(128) InstDesc {
   int32_t kind, order, integrator, storage;
   int32_t nx, ny, M, Mpad;
   int32_t n_chunks, tx, ly, n_strips;
-  int32_t n_segs, n_items, n_regions, pad1;
+  int32_t n_segs, n_items, n_regions;
+  // streaming Cartesian kernel, ordered form: ordinates per term of phi (2 or 4), floats per
+  // cell that hold the terms
+  int32_t ord_vec, ord_parts, pad1;
   int64_t n_cells;
   int64_t n_steps;
   int64_t wait_limit;           // device wait bound in clock64 cycles
@@ -131,8 +138,8 @@ struct WorkItem {
 // Launchers (defined in the .cu files). All enqueue on `stream`. chained: the launch
 // follows a kernel of the same run of steps, and nothing else, on its stream, so its blocks
 // may start before that one ends.
-// Cartesian stage kernels. uni != 0: the streaming kernel (InstDesc::str_chunks; tile
-// width 8 * run, run 2 or 4); uni = 0: the general kernel (run 2, vec ordinates per lane).
+// Cartesian stage kernels. uni (CartForm) != 0: the streaming kernel (InstDesc::str_chunks;
+// tile width 8 * run, run 2 or 4); 0: the general kernel (run 2, vec ordinates per lane).
 cudaError_t launch_cart_stage(const InstDesc* d_desc, const WorkItem* d_items, int n_items, int stage,
                               int order, int storage, int run, int vec, int ly_max, cudaStream_t stream,
                               int uni = 0, bool chained = false);
