@@ -96,8 +96,8 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
                : "memory");
 }
 
-// Constants of a chunk's cells: {dt ax0, dt ax1, dt ax2, dt ay0}, {dt ay1, dt ay2,
-// -dt sigma_t, dt (sigma_s/(2 pi) phi + Q)} with a_e = n_e l_e / A, the neighbours
+// Constants of a chunk's cells: {ax0, ax1, ax2, ay0}, {ay1, ay2, -sigma_t,
+// sigma_s/(2 pi) phi + Q} with a_e = n_e l_e / A, the neighbours
 // {cell ids; own id on the boundary}, flag bit e of w set for a boundary edge.
 struct TriTable {
   float4 g[kTriChunk], h[kTriChunk];
@@ -141,6 +141,7 @@ __global__ void __launch_bounds__(kTriThreads, 3)
   const int n_chunks = (n_cells + kTriChunk - 1) / kTriChunk;
   const int G = it.b;
   const int64_t limit = d.wait_limit;
+  const float dt = d.dt;
 
   // metadata of chunk k into buffer b (thread 0)
   auto stage_meta = [&](int k, int b) {
@@ -179,9 +180,8 @@ __global__ void __launch_bounds__(kTriThreads, 3)
       const int4 nb = s_nbr[b][tid];
       const float4 g0 = s_geo[b][2 * tid], g1 = s_geo[b][2 * tid + 1];
       const int m = nb.w & 255;
-      const float dt = d.dt;
-      tab.g[tid] = make_float4(dt * g0.x, dt * g0.z, dt * g1.x, dt * g0.y);
-      tab.h[tid] = make_float4(dt * g0.w, dt * g1.y, -dt * d.sig_t[m], dt * (d.sig_s2pi[m] * phi_in[c0 + tid] + d.q_src[m]));
+      tab.g[tid] = make_float4(g0.x, g0.z, g1.x, g0.y);
+      tab.h[tid] = make_float4(g0.w, g1.y, -d.sig_t[m], d.sig_s2pi[m] * phi_in[c0 + tid] + d.q_src[m]);
       tab.nbr[tid] = make_int4(nb.x < 0 ? c0 + tid : nb.x, nb.y < 0 ? c0 + tid : nb.y, nb.z < 0 ? c0 + tid : nb.z,
                                (nb.x < 0) | (nb.y < 0) << 1 | (nb.z < 0) << 2);
     }
@@ -244,15 +244,15 @@ __global__ void __launch_bounds__(kTriThreads, 3)
             auto pair = [&](const float (&a)[VEC]) { return make_float2(a[l], a[l1]); };
             auto dup = [](float a) { return make_float2(a, a); };
             const float2 c = pair(c2[s]), x = pair(xi), y = pair(eta);
-            float2 inc = __ffma2_rn(dup(h.z), c, dup(h.w));   // dt F
+            float2 F = __ffma2_rn(dup(h.z), c, dup(h.w));
 #pragma unroll
             for (int e = 0; e < 3; ++e) {
               const float2 on = __ffma2_rn(y, dup(ay[e]), __fmul2_rn(x, dup(ax[e])));
               const float2 n = pair(n2[s][e]);
-              inc = __ffma2_rn(make_float2(fminf(on.x, 0.f), fminf(on.y, 0.f)),
-                               __fadd2_rn(c, make_float2(-n.x, -n.y)), inc);
+              F = __ffma2_rn(make_float2(fminf(on.x, 0.f), fminf(on.y, 0.f)), __fadd2_rn(c, make_float2(-n.x, -n.y)), F);
             }
-            float2 o = __fadd2_rn(c, inc);
+            // dt enters last: rounded into the cell's constants, it would be off by the same amount in every step
+            float2 o = __ffma2_rn(dup(dt), F, c);
             if constexpr (STAGE == STAGE_HEUN2) o = __fmul2_rn(dup(0.5f), __fadd2_rn(pair(b2[s]), o));
             if constexpr (sizeof(T) == 2) {
               o.x = Store<T>::round_sr(o.x, sr_elem(rb4, (kk + l) & 3));

@@ -49,7 +49,7 @@ constexpr int kStgWarps = kStgThreads / 32;
 constexpr int kStgChunk = kTriStgChunk;   // cells per chunk (32)
 constexpr int kStgCellsPerWarp = kStgChunk / kStgWarps;
 constexpr int kStgMeta = 4;   // metadata buffers: chunks i .. i+3
-constexpr int kStgTab = 16;   // cell table entries: dt (n.l/A) x and y per edge, -dt sigma_t, dt source, offsets
+constexpr int kStgTab = 16;   // cell table entries: n.l/A x and y per edge, -sigma_t, source, offsets
                               // of the neighbours' staged rows, boundary flags, area, area sigma_a, QoI region
 
 __device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kStgThreads, 2)
     const int c0 = (it.a + i * G) * kStgChunk;
     if (c0 + lane < n_cells) {
       const int m = meta_nbr(i % kStgMeta)[lane].w & 255;
-      src_next = dt * (d.sig_s2pi[m] * phi_in[c0 + lane] + d.q_src[m]);
+      src_next = d.sig_s2pi[m] * phi_in[c0 + lane] + d.q_src[m];
     }
   };
   auto table_store = [&](int i) {
@@ -294,9 +294,9 @@ __global__ void __launch_bounds__(kStgThreads, 2)
       const float4 g0 = meta_geo(mb)[2 * lane], g1 = meta_geo(mb)[2 * lane + 1];
       const uint32_t lx = meta_lidx(mb)[lane];
       float* t = tabs + ((i & 1) * kStgChunk + lane) * kStgTab;
-      t[0] = dt * g0.x; t[1] = dt * g0.z; t[2] = dt * g1.x;   // x components of dt (n.l)/A for edges 0, 1, 2
-      t[3] = dt * g0.y; t[4] = dt * g0.w; t[5] = dt * g1.y;   // y components
-      t[6] = -dt * d.sig_t[nb4.w & 255];
+      t[0] = g0.x; t[1] = g0.z; t[2] = g1.x;   // x components of (n.l)/A for edges 0, 1, 2
+      t[3] = g0.y; t[4] = g0.w; t[5] = g1.y;   // y components
+      t[6] = -d.sig_t[nb4.w & 255];
       t[7] = src_next;
       flags = 0;
 #pragma unroll
@@ -398,14 +398,15 @@ __global__ void __launch_bounds__(kStgThreads, 2)
           auto pair = [&](const float (&a)[VEC]) { return make_float2(a[l], a[l1]); };
           auto dup = [](float a) { return make_float2(a, a); };
           const float2 c2 = pair(c), xi2 = pair(xi), eta2 = pair(eta);
-          float2 inc = __ffma2_rn(dup(t1.z), c2, dup(t1.w));   // dt F
+          float2 F = __ffma2_rn(dup(t1.z), c2, dup(t1.w));
 #pragma unroll
           for (int e = 0; e < 3; ++e) {
             const float2 on = __ffma2_rn(eta2, dup(ay[e]), __fmul2_rn(xi2, dup(ax[e])));
             const float2 n2 = pair(nbv[e]);
-            inc = __ffma2_rn(make_float2(fminf(on.x, 0.f), fminf(on.y, 0.f)), __fadd2_rn(c2, make_float2(-n2.x, -n2.y)), inc);
+            F = __ffma2_rn(make_float2(fminf(on.x, 0.f), fminf(on.y, 0.f)), __fadd2_rn(c2, make_float2(-n2.x, -n2.y)), F);
           }
-          float2 o = __fadd2_rn(c2, inc);
+          // dt enters last: rounded into the cell's constants, it would be off by the same amount in every step
+          float2 o = __ffma2_rn(dup(dt), F, c2);
           if constexpr (kBase) o = __fmul2_rn(dup(0.5f), __fadd2_rn(pair(base), o));
           if constexpr (sizeof(T) == 2) {
             o.x = Store<T>::round_sr(o.x, sr_elem(rb4, (kk + l) & 3));
