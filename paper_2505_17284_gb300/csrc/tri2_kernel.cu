@@ -28,7 +28,8 @@
 // vanish, and the rounding error is smaller (650^2 x 256, one step against FP64: 4.22e-8
 // of psi, 4.33e-8 with values). At 400^2 x 256 (FP32), with IEEE divisions in divergent
 // branches and 2 ordinates per lane in the stage pass: gradient 0.82 ms, stage 0.45 ms;
-// now 0.27 and 0.35 ms. A Heun step at 650^2 x 256: 6.65 -> 3.29 ms.
+// now 0.29 and 0.35 ms. A Heun step at 650^2 x 256: 6.65 -> 3.42 ms (3.29 with quotients that
+// were 2 ulp off).
 #include <cuda_bf16.h>
 
 #include "device_common.cuh"
@@ -106,29 +107,47 @@ __device__ __forceinline__ float fmax3f(float a, float b, float c) {
   return r;
 }
 
-// Smallest of the three edges' limiter values. The quotients are formed with __fdividef
-// (2 ulp inside its range of denominators): three IEEE divisions in divergent branches were
-// 200 of 269 instructions per cell and ordinate. Denominators below that range, which a
-// state of zeros or a front's foot has where epsilon^2 = A^6 is small (10^-36 at 2 * 650^2
-// cells), are formed again from x and y times 2^63, the quotient being homogeneous; only
-// states above 10^18 divide by IEEE.
-__device__ __forceinline__ float limiter(const float (&x)[3], const float (&y)[3], const float (&num)[3],
-                                         const float (&den)[3], float eps2) {
-  const float lo = fmin3f(den[0], den[1], den[2]), hi = fmax3f(den[0], den[1], den[2]);
-  if (lo >= 0x1p-126f && hi <= 1e36f)
-    return fmin3f(__fdividef(num[0], den[0]), __fdividef(num[1], den[1]), __fdividef(num[2], den[2]));
-  if (hi <= 1e36f) {
-    float L[3];
+// Quotients a / b of pairs of positive floats, b and 1 / b in the normal range: the product
+// with the approximate reciprocal, corrected once by its residual a - q b, which a fused
+// operation gives exactly (P. Markstein, Computation of elementary functions on the IBM RISC
+// System/6000 processor, 1990). Off from the rounded quotient only where a / b lies within
+// 2^-21 ulp of the middle of two floats.
+__device__ __forceinline__ float2 quotient2(float2 a, float2 b) {
+  float2 r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(b.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(b.y));
+  const float2 q = __fmul2_rn(a, r);
+  return __ffma2_rn(__ffma2_rn(make_float2(-q.x, -q.y), b, a), r, q);
+}
+
+// Smallest of the three edges' limiter values outside the range of quotient2 for the values as
+// they are. Numerators below 2^-117 (they are at most twice the denominators), whose residuals
+// leave the range of floats, are formed again from x and y times 2^63, the quotient being
+// homogeneous: a state of zeros or a front's foot has them where epsilon^2 = A^6 is small
+// (10^-36 at 2 * 650^2 cells). Only states above 10^18 divide by IEEE.
+__device__ __forceinline__ float limiter_rescaled(float gx, float gy, float up, float dn, const float (&rxh)[3],
+                                                  const float (&ryh)[3], float eps2) {
+  float x[3], y[3], den[3], L[3];
 #pragma unroll
-    for (int e = 0; e < 3; ++e) {
+  for (int e = 0; e < 3; ++e) {
+    const float D = fmaf(ryh[e], gy, rxh[e] * gx);
+    x[e] = fabsf(D);
+    y[e] = D > 0.f ? up : dn;
+    den[e] = fmaf(x[e] + x[e], x[e], fmaf(y[e], y[e], eps2) + x[e] * y[e]);
+  }
+  const bool ieee = !(fmax3f(den[0], den[1], den[2]) <= 1e36f);
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    if (ieee) {
+      L[e] = venkat_exact(x[e], y[e], eps2);
+    } else {
       const float s = den[e] < 0x1p-100f ? 0x1p63f : 1.f;
       const float xs = x[e] * s, ys = y[e] * s, p = xs * ys, c = fmaf(ys, ys, eps2 * s * s) + p;
       const float d = fmaf(xs + xs, xs, c);
-      L[e] = d > 0.f ? __fdividef(c + p, d) : 1.f;   // 0 / 0 without a spread
+      L[e] = d > 0.f ? quotient2(make_float2(c + p, 1.f), make_float2(d, 1.f)).x : 1.f;   // 0 / 0 without a spread
     }
-    return fmin3f(L[0], L[1], L[2]);
   }
-  return fminf(fminf(venkat_exact(x[0], y[0], eps2), venkat_exact(x[1], y[1], eps2)), venkat_exact(x[2], y[2], eps2));
+  return fminf(fminf(L[0], L[1]), L[2]);
 }
 
 // Limited gradient L g of a pair of ordinates from the cell's values c and its
@@ -146,7 +165,7 @@ __device__ __forceinline__ void limited_gradient2(float2 c, float2 n0, float2 n1
   // beta_max and -beta_min
   const float2 up = make_float2(fmaxf(fmax3f(s0.x, s1.x, s2.x), 0.f), fmaxf(fmax3f(s0.y, s1.y, s2.y), 0.f));
   const float2 dn = make_float2(-fminf(fmin3f(s0.x, s1.x, s2.x), 0.f), -fminf(fmin3f(s0.y, s1.y, s2.y), 0.f));
-  float xa[3], ya[3], na[3], da[3], xb[3], yb[3], nb[3], db[3];
+  float2 num[3], den[3];
 #pragma unroll
   for (int e = 0; e < 3; ++e) {
     const float2 D = __ffma2_rn(dup(ryh[e]), gy, __fmul2_rn(dup(rxh[e]), gx));
@@ -154,11 +173,20 @@ __device__ __forceinline__ void limited_gradient2(float2 c, float2 n0, float2 n1
     const float2 y = make_float2(D.x > 0.f ? up.x : dn.x, D.y > 0.f ? up.y : dn.y);
     const float2 p = __fmul2_rn(x, y);
     const float2 q = __fadd2_rn(__ffma2_rn(y, y, dup(eps2)), p);
-    const float2 n = __fadd2_rn(q, p), d = __ffma2_rn(__fadd2_rn(x, x), x, q);
-    xa[e] = x.x; ya[e] = y.x; na[e] = n.x; da[e] = d.x;
-    xb[e] = x.y; yb[e] = y.y; nb[e] = n.y; db[e] = d.y;
+    num[e] = __fadd2_rn(q, p);
+    den[e] = __ffma2_rn(__fadd2_rn(x, x), x, q);
   }
-  const float2 L = make_float2(limiter(xa, ya, na, da, eps2), limiter(xb, yb, nb, db, eps2));
+  // The smallest of the edges' values. Three IEEE divisions in divergent branches were 200 of
+  // 269 instructions per cell and ordinate.
+  float2 L;
+  const float lo = fminf(fmin3f(num[0].x, num[1].x, num[2].x), fmin3f(num[0].y, num[1].y, num[2].y));
+  const float hi = fmaxf(fmax3f(den[0].x, den[1].x, den[2].x), fmax3f(den[0].y, den[1].y, den[2].y));
+  if (lo >= 0x1p-117f && hi <= 1e36f) {
+    const float2 l0 = quotient2(num[0], den[0]), l1 = quotient2(num[1], den[1]), l2 = quotient2(num[2], den[2]);
+    L = make_float2(fmin3f(l0.x, l1.x, l2.x), fmin3f(l0.y, l1.y, l2.y));
+  } else {
+    L = make_float2(limiter_rescaled(gx.x, gy.x, up.x, dn.x, rxh, ryh, eps2), limiter_rescaled(gx.y, gy.y, up.y, dn.y, rxh, ryh, eps2));
+  }
   lx = __fmul2_rn(L, gx);
   ly = __fmul2_rn(L, gy);
 }

@@ -54,3 +54,91 @@ def test_decay_of_a_uniform_state(rt, order, staged, heun, n_p, n_phi):
             one = f32(0.5) * fma(f32(dt), -(f32(sigma) * one), c + one)
         c = one
     assert away.sum() > 40 and np.array_equal(psi[away], np.tile(c, (away.sum(), 1)))
+
+
+def second_order_euler(mesh, quad, psi, sigma, dt):
+    """One Euler step of the limited scheme in a pure absorber with vacuum sides, operation by operation as the
+    kernels compute it, with rounded quotients in the limiter."""
+    V, T = mesh.vertices, mesh.triangles
+    n, M = psi.shape
+    P = V[T]
+    Q = np.roll(P, -1, axis=1)
+    A = 0.5 * ((P[:, 1, 0] - P[:, 0, 0]) * (P[:, 2, 1] - P[:, 0, 1]) - (P[:, 1, 1] - P[:, 0, 1]) * (P[:, 2, 0] - P[:, 0, 0]))
+    cen = (P[:, 0] + P[:, 1] + P[:, 2]) / 3.0
+    side = {}
+    nbr = np.full((n, 3), -1)
+    for t in range(n):
+        for e in range(3):
+            key = frozenset((T[t, e], T[t, (e + 1) % 3]))
+            if key in side:
+                u, f = side[key]
+                nbr[t, e], nbr[u, f] = u, t
+            else:
+                side[key] = t, e
+    inside = (nbr >= 0)[:, :, None]
+    ax, ay = ((Q[..., 1] - P[..., 1]) / A[:, None]).astype(f32), (-(Q[..., 0] - P[..., 0]) / A[:, None]).astype(f32)
+    r = (0.5 * (P + Q) - cen[:, None]).astype(f32)
+    s = np.where(inside, 0.5 * (P + Q) - cen[nbr], 0.0).astype(f32)
+    eps2 = ((A * A * A) ** 2).astype(f32)[:, None]
+    c = psi
+    nb = [np.where(inside[:, e], psi[nbr[:, e]], f32(0)) for e in range(3)]
+    h = f32(0.5)
+    d3 = [v - c for v in nb]
+
+    def fm(a, b, x):
+        return (np.float64(1) * a * b.astype(np.float64) + x).astype(f32)
+
+    gx, gy = (fm(h * a[:, 2:3], d3[2], fm(h * a[:, 1:2], d3[1], h * a[:, 0:1] * d3[0])) for a in (ax, ay))
+    up, dn = np.maximum(np.maximum.reduce(d3), 0), -np.minimum(np.minimum.reduce(d3), 0)
+    def limiter(scale):
+        """(smallest of the three edges' values, smallest numerator); x and y times 2^63 where den < 2^-100 if asked for."""
+        L = lo = None
+        for e in range(3):
+            D = fm(h * r[:, e, 1:2], gy, h * r[:, e, 0:1] * gx)
+            x, y = np.abs(D), np.where(D > 0, up, dn)
+            den = fm(x + x, x, fm(y, y, eps2) + x * y)
+            k = np.where(scale & (den < f32(2.0 ** -100)), f32(2.0 ** 63), f32(1))
+            x, y = x * k, y * k
+            p = x * y
+            q = fm(y, y, eps2 * k * k) + p
+            one, num = (q + p) / fm(x + x, x, q), q + p
+            L, lo = (one, num) if L is None else (np.minimum(L, one), np.minimum(lo, num))
+        return L, lo
+
+    L, lo = limiter(False)
+    if lo.min() < 2.0 ** -117:   # the kernels rescale where residuals would leave the range of floats
+        pair = M > 32            # (both values of a lane's pair together)
+        low = lo < f32(2.0 ** -117)
+        low = (low | np.stack([low[:, 1::2], low[:, ::2]], 2).reshape(low.shape)) if pair else low
+        L = np.where(low, limiter(True)[0], L)
+    lx, ly = L * gx, L * gy
+    div = np.zeros_like(c)
+    xi, eta = (np.asarray(v, f32)[None] for v in quad[:2])
+    for e in range(3):
+        on = fm(eta, np.broadcast_to(ay[:, e:e + 1], c.shape), xi * ax[:, e:e + 1])
+        mine = fm(lx, r[:, e, 0:1], ly * r[:, e, 1:2])
+        other = fm(lx[nbr[:, e]], s[:, e, 0:1], fm(ly[nbr[:, e]], s[:, e, 1:2], d3[e]))
+        mine = np.where(inside[:, e], mine, f32(0))
+        other = np.where(inside[:, e], other, d3[e])
+        div = fm(on, np.where(on > 0, mine, other), div)
+    return fm(f32(dt), fm(np.full_like(c, -f32(sigma)), c, -div), c)
+
+
+@pytest.mark.parametrize("n_p,n_phi", [(2, 16), (4, 16), (8, 16)])   # 1, 2 and 4 ordinates per lane
+@pytest.mark.parametrize("L,scale", [(1.0, 1.0), (0.01, 1.0), (1.0, 1e-17), (0.01, 1e-18)])
+def test_limiter_divides_to_the_last_bit(rt, n_p, n_phi, L, scale):
+    """Every other cell is empty, so that a step leaves dt F there and the limiter's last bits show: equal but for
+    values that the 64-bit stand-in of a fused operation rounds twice, or a quotient within 2^-21 ulp of the middle
+    between two floats (1e-4 of the values: 36 quotients reach a value, with its neighbours')."""
+    mesh = si.split_grid_mesh(21, L, jitter=0.2, seed=4)
+    n, M, sigma = mesh.n_cells, n_p * n_phi, 3.0
+    mats = si.Materials(sigma_a=np.array([sigma]), sigma_s=np.array([0.0]), Q=np.array([0.0]), cell_mat=np.zeros(n, np.int32),
+                        cell_region=np.zeros(n, np.int32), region_names=("all",))
+    quad = rt.rt_quad_product(n_p, n_phi)
+    s = rt.Solver(si.Problem(mesh=mesh, materials=mats, boundary=si.Boundary(), t_end=1.0), quad, order=2, integrator=rt.RT_EULER)
+    psi0 = (si.random_psi(n, M, seed=6) * (np.arange(n) % 2)[:, None] * scale).astype(f32)
+    s.set_psi(psi0)
+    s.step(1)
+    psi, dt = s.psi(), s.info.dt
+    s.close()
+    assert np.mean(psi != second_order_euler(mesh, quad, psi0, sigma, dt)) <= 1e-4
