@@ -283,22 +283,27 @@ __device__ __forceinline__ void block_reduce_q(const double (&acc)[NQ], int nq, 
 
 // Sum over a block of one FP32 value per thread (v[0 .. NT) in shared memory), in
 // FP64, by one warp; every lane returns it. A lane first adds its NT / 32 values
-// with Knuth's two-sum (the rounding errors of an FP32 sum, kept beside it), so
-// that a conversion and 6 additions run on the FP64 pipe instead of 5 additions
-// in each of the block's warps: that pipe adds about 2 lanes per cycle and SM
-// here, and the block sums were most of a small launch's tail.
+// with Knuth's two-sum, twice: the rounding errors of the FP32 sum are kept beside
+// it, and those of their sum beside them, which together hold more bits than an
+// FP64 sum (s + e alone holds about 48). So three conversions and 7 additions run
+// on the FP64 pipe instead of 5 additions in each of the block's warps: that pipe
+// adds about 2 lanes per cycle and SM here, and the block sums were most of a small
+// launch's tail.
 template <int NT>
 __device__ __forceinline__ double warp_block_sum(const float* v) {
   const int lane = threadIdx.x & 31;
-  float s = 0.f, e = 0.f;
+  float s = 0.f, e = 0.f, f = 0.f;
 #pragma unroll
   for (int j = 0; j < NT / 32; ++j) {
     const float x = v[lane + 32 * j];
     const float t = s + x, z = t - s;
-    e += (s - (t - z)) + (x - z);
+    const float y = (s - (t - z)) + (x - z);   // t + y = s + x
+    const float u = e + y, w = u - e;
+    f += (e - (u - w)) + (y - w);
     s = t;
+    e = u;
   }
-  double r = (double)s + (double)e;
+  double r = (double)s + ((double)e + (double)f);
   if (!isfinite(r)) {   // a value, or the FP32 sum of finite ones, is not finite
     r = 0.0;
     for (int j = 0; j < NT / 32; ++j) r += (double)v[lane + 32 * j];

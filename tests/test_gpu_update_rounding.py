@@ -142,3 +142,28 @@ def test_limiter_divides_to_the_last_bit(rt, n_p, n_phi, L, scale):
     psi, dt = s.psi(), s.info.dt
     s.close()
     assert np.mean(psi != second_order_euler(mesh, quad, psi0, sigma, dt)) <= 1e-4
+
+
+@pytest.mark.parametrize("vec", [0, 1])   # the streaming and the general kernel
+@pytest.mark.parametrize("lane", [0, 13, 31])
+def test_quantities_are_summed_in_64_bits(rt, vec, lane):
+    """Scalar fluxes that any FP64 sum adds exactly (they span 53 bits) and an FP32 sum with one term for its errors
+    does not, in the eight cells that one lane adds. One ordinate without a direction and with weight 1, so that
+    phi = psi, unit cells of nothing, one cell per thread of a block."""
+    n = 48
+    mesh = si.CartesianMesh(nx=n, ny=n, x0=0.0, y0=0.0, dx=1.0, dy=1.0)
+    mats = si.Materials(sigma_a=np.zeros(1), sigma_s=np.zeros(1), Q=np.zeros(1), cell_mat=np.zeros(n * n, np.int32),
+                        cell_region=np.zeros(n * n, np.int32), region_names=("all",))
+    p = si.Problem(mesh=mesh, materials=mats, boundary=si.Boundary(), t_end=10.0)
+    psi = np.zeros((n, n))
+    for j, v in enumerate([2.0 ** 26, 1.0, 2.0 ** -25, 2.0 ** -25, -2.0 ** 26, -1.0, 2.0 ** -24, 0.0]):
+        t = lane + 32 * j
+        psi[16 + t // 16, 32 + t % 16] = v
+    one = (np.zeros(1), np.zeros(1), np.ones(1), np.ones(1))
+    s = rt.Solver(p, one, order=1, integrator=rt.RT_EULER, dt=1.0, tile_x=16, tile_y=16, vec=vec)
+    s.set_psi(psi.reshape(-1, 1))
+    s.step(2)
+    q, got = s.qoi(), s.psi()
+    s.close()
+    assert np.array_equal(got[:, 0], psi.ravel())
+    assert q["mass"] == 2.0 ** -23
