@@ -140,9 +140,10 @@ typedef void (*rt_free_fn)(void* ptr, void* ctx);
  *     arithmetic is FP32 either way, QoI accumulation FP64).
  *   dt > 0: target step; N_t = ceil(t_end/dt - 1e-9) and dt = t_end/N_t.
  *   dt <= 0: Cartesian 0.5*min(dx,dy); triangles 0.9*min_i 2 A_i / P_i.
- *   tile_x, tile_y: Cartesian tile: cells per work item in x (16, or 32, which needs
- *     chunk-uniform directions in chunks of 64 ordinates when asked for) and rows per
- *     segment (at most 256); 0 = chosen by the library.
+ *   tile_x, tile_y: Cartesian tile: cells per work item in x (16; or 32, which can be
+ *     asked for with chunk-uniform directions in chunks of 64 ordinates, and where the
+ *     library would choose it) and rows per segment (at most 256); 0 = chosen by the
+ *     library. What rt_info and rt_autotune report can be passed back.
  *   variant: directions of the Cartesian kernel. 0 = chosen by the library; 1 = per-lane
  *     flow directions (any quadrature); 2 = chunk-uniform directions, usable when
  *     every chunk of 128 or 64 ordinates has one sign of xi and one of eta (the product
@@ -331,10 +332,10 @@ const char* rt_last_error(void);
 /* ---------------------------------------------------------------------------
  * Autotuner (Cartesian meshes). The paper has no counterpart: it chooses among
  * the library's own kernel configurations. For the problem and options given,
- * each candidate (strip width 16 or 32 cells, segment length in {auto, 4, 6, 8, 12,
- * 16, 24, ..., 64} rows, per-lane or chunk-uniform directions; only those the
- * quadrature and shared memory allow, and opts->variant/vec if set) is built
- * as a full solver with rt_create, advanced one step, then timed with CUDA
+ * each candidate (the library's own choice; then strip width 16 or 32 cells, segment
+ * length in {auto, 4, 6, 8, 12, 16, 24, ..., 64} rows, per-lane or chunk-uniform
+ * directions; only those the quadrature and shared memory allow, and opts->variant/vec
+ * if set) is built as a full solver with rt_create, advanced one step, then timed with CUDA
  * events over `steps` further steps (at most N_t - 1) on opts->stream, and
  * destroyed. *best receives opts with tile_x, tile_y, variant and vec of the
  * fastest candidate (so rt_create(..., best, ...) builds it), and

@@ -23,12 +23,12 @@ extern "C" rt_status rt_autotune(const rt_mesh* mesh, const rt_materials* mat, c
   if (steps < 1 || steps > 1000) { set_error("steps must be in 1..1000"); return RT_EINVAL; }
   const cudaStream_t stream = (cudaStream_t)opts->stream;
 
+  // the library's own choice first
   struct Cand { int tile_x, tile_y, variant; };
-  std::vector<Cand> cands;
+  std::vector<Cand> cands{{0, 0, opts->variant}};
   const int lys[] = {0, 4, 6, 8, 12, 16, 24, 32, 40, 48, 56, 64};
   for (int tx : {16, 32})
     for (int var : {0, 1}) {
-      if (tx == 32 && var == 1) continue;   // 32-cell strips exist for chunk-uniform directions only
       if (opts->variant != 0 && var != 0 && var != opts->variant) continue;
       for (int ly : lys) cands.push_back({tx, ly, var != 0 ? var : opts->variant});
     }

@@ -705,6 +705,112 @@ static rt_status build_box_faces(const rt_mesh* mesh, const rt_materials* mat, s
   return RT_OK;
 }
 
+// ---------------------------------------------------------------- plan
+// Kernel, tile and segment of a Cartesian problem (I: grid, scheme, storage, Mpad) for the
+// options given; quad is the internal layout. Allocates nothing on the device.
+static rt_status plan_cart(Instance& I, const rt_quadrature* quad, int tile_x, int tile_y, int variant, int vec) {
+  if (variant < 0 || variant > 2) { set_error("variant must be 0, 1 or 2"); return RT_EINVAL; }
+  // per-lane width first; the chunk-uniform variant is taken (automatically) when
+  // the same width also gives sign-uniform chunks, or when asked for
+  if (vec != 0 && vec != 1 && vec != 2 && vec != 4) { set_error("vec must be 0, 1, 2 or 4"); return RT_EINVAL; }
+  I.uni = 0;
+  I.str_chunks.clear();
+  I.cvec = choose_cart_vec(quad, I.Mpad);
+  if (vec != 0) {
+    if (vec > I.cvec) { set_error("vec %d: the quadrature allows at most %d ordinates per lane", vec, I.cvec); return RT_EINVAL; }
+    I.cvec = vec;
+  }
+  if (tile_x != 0 && tile_x != 16 && tile_x != 32) { set_error("tile_x must be 0, 16 or 32"); return RT_EINVAL; }
+  I.run = 2;
+  // 32-cell tiles: asked for, or taken when whole chunks of 128 ordinates mix signs but
+  // chunks of 64 do not (256 ordinates), on grids of more than kWideMinCells cells.
+  // Above kWideMaxCells cells second order takes tiles of 16 cells all the same (256
+  // ordinates, Heun: 400^2 257 us with 32, 246 with 16; 840^2 848 and 756). Between the
+  // limits the two are 1 to 5 % apart (320^2 176 and 170, 350^2 218 and 213); 32 cells stay
+  // the library's documented choice there.
+  constexpr int64_t kWideMinCells = 100000, kWideMaxCells = 1 << 17;
+  bool wide = false;
+  if (variant != 1 && (vec == 0 || vec == 2) && tile_x != 16) {
+    const bool narrow4 = tile_x == 0 && vec == 0 && I.cvec >= 4 && chunks_uniform(quad, I.Mpad, 4);
+    const bool small = tile_x == 0 && variant == 0 && vec == 0 && I.n_cells <= kWideMinCells;
+    wide = !narrow4 && !small && chunks_uniform(quad, I.Mpad, 2);
+  }
+  if (wide) {
+    I.uni = 1;
+    I.cvec = 2;
+    I.run = 4;
+  } else if (tile_x == 32) {
+    // otherwise only where the library takes them itself (few windows, below), so that what
+    // rt_info and the tuner report can be asked for
+    const rt_status st = plan_cart(I, quad, 0, tile_y, variant, vec);
+    if (st == RT_OK && I.run != 4) {
+      set_error("tile_x 32 needs chunk-uniform directions with 2 ordinates per lane");
+      return RT_EINVAL;
+    }
+    return st;
+  } else if (variant != 1) {
+    for (int V = (variant == 2 && vec == 0 ? 4 : I.cvec); V >= 2; V /= 2) {
+      if (chunks_uniform(quad, I.Mpad, V)) {
+        I.uni = 1;
+        I.cvec = V;
+        break;
+      }
+      if (variant == 0 || vec != 0) break;
+    }
+    if (variant == 2 && !I.uni) {
+      set_error("variant 2 needs every ordinate chunk to have one sign of xi and one of eta");
+      return RT_EINVAL;
+    }
+  }
+  // What the caller sees of the choice: chunk-uniform (2) or per-lane (1) directions.
+  // The streaming kernel runs both: always for chunk-uniform ones, and for per-lane
+  // ones unless a number of ordinates per lane was asked for (that is the general
+  // kernel's option; the streaming kernel always takes four, and vec reads 0). The
+  // general kernel is left for quadratures whose signs change too often for windows
+  // of 32: at 1000^2 x 128, where both run, it takes 0.84 ms per Heun step against
+  // 0.59, at 531^2 x 100 0.52 against 0.24, at 140^2 x 128 0.076 against 0.055.
+  I.info_variant = I.uni ? 2 : 1;
+  I.info_vec = I.cvec;
+  if (I.uni || vec == 0) I.str_chunks = plan_stream_chunks(quad, I.Mpad, I.storage);
+  // whether as long a segment as asked for fits the shared memory of a CTA
+  auto fits = [&](int run) {
+    const int stage_hi = I.integrator == RT_HEUN ? STAGE_HEUN2 : STAGE_EULER;
+    return tile_y <= 0 || cart_smem_bytes(I.order, I.storage, run, 4, std::min(tile_y, 256), stage_hi,
+                                          ordered_form(I, run)) <= 227 * 1024;
+  };
+  I.ord_vec = 0;
+  if (I.order == 2 && I.n_cells <= kOrderedMaxCells && !I.str_chunks.empty()) {
+    if (I.cvec > 1 && windows_whole(I.str_chunks, I.Mpad)) I.ord_vec = I.cvec;
+    if (I.ord_vec && !fits(I.run)) I.ord_vec = 0;
+    if (!I.ord_vec && !I.uni) I.str_chunks.clear();
+  }
+  if (!I.str_chunks.empty()) {
+    if (!I.uni) I.info_vec = 0;
+    I.uni = 1;
+    I.cvec = 4;
+    if (tile_x == 0 && I.run == 4 && I.order == 2 && I.n_cells > kWideMaxCells) I.run = 2;
+    // one or two chunks (64 ordinates): a tile of 16 cells leaves half of a CTA's warps
+    // without a chunk, which costs less than larger tiles only on small grids
+    // (70^2 x 64 Heun: 35.4 us per step with 16, 38.5 with 32); the ordered form gains up to
+    // four (280^2 x 128: 103 us with 16, 96 with 32), and no more beyond (280^2 x 512: 294, 342)
+    if (tile_x == 0 && I.run == 2 && I.str_chunks.size() <= (I.ord_vec ? 4u : 2u)) {
+      double narrow, wider;
+      stream_segment(I, 2, ordered_form(I, 2), &narrow);
+      stream_segment(I, 4, ordered_form(I, 4), &wider);
+      if (wider < narrow && fits(4)) I.run = 4;
+    }
+    I.uni = ordered_form(I, I.run);
+  } else {
+    I.uni = 0;
+    I.run = 2;
+  }
+  choose_cart_tiles(I, tile_y);
+  const int stage_hi = I.integrator == RT_HEUN ? STAGE_HEUN2 : STAGE_EULER;
+  I.cart_smem = cart_smem_bytes(I.order, I.storage, I.run, I.cvec, I.ly, stage_hi, I.uni);
+  if (I.cart_smem > 227 * 1024) { set_error("tile %dx%d needs %zu bytes of shared memory", I.tx, I.ly, I.cart_smem); return RT_EINVAL; }
+  return RT_OK;
+}
+
 // ---------------------------------------------------------------- build
 rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_quadrature* quad,
                          const rt_boundary* bc, int order, int integrator, int storage, double dt_target,
@@ -795,93 +901,7 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
 
   // --- tiles and work items
   if (I.kind == RT_MESH_CARTESIAN) {
-    if (variant < 0 || variant > 2) { set_error("variant must be 0, 1 or 2"); return RT_EINVAL; }
-    // per-lane width first; the chunk-uniform variant is taken (automatically) when
-    // the same width also gives sign-uniform chunks, or when asked for
-    if (vec != 0 && vec != 1 && vec != 2 && vec != 4) { set_error("vec must be 0, 1, 2 or 4"); return RT_EINVAL; }
-    I.uni = 0;
-    I.cvec = choose_cart_vec(quad, I.Mpad);
-    if (vec != 0) {
-      if (vec > I.cvec) { set_error("vec %d: the quadrature allows at most %d ordinates per lane", vec, I.cvec); return RT_EINVAL; }
-      I.cvec = vec;
-    }
-    if (tile_x != 0 && tile_x != 16 && tile_x != 32) { set_error("tile_x must be 0, 16 or 32"); return RT_EINVAL; }
-    I.run = 2;
-    // 32-cell tiles: asked for, or taken when whole chunks of 128 ordinates mix signs but
-    // chunks of 64 do not (256 ordinates), on grids of more than kWideMinCells cells.
-    // Above kWideMaxCells cells second order takes tiles of 16 cells all the same (256
-    // ordinates, Heun: 450^2 304 us with 32, 280 with 16; 840^2 848 and 756).
-    constexpr int64_t kWideMinCells = 100000, kWideMaxCells = 1 << 17;
-    bool wide = false;
-    if (variant != 1 && (vec == 0 || vec == 2) && tile_x != 16) {
-      const bool narrow4 = tile_x == 0 && vec == 0 && I.cvec >= 4 && chunks_uniform(quad, I.Mpad, 4);
-      const bool small = tile_x == 0 && variant == 0 && vec == 0 && n_cells <= kWideMinCells;
-      wide = !narrow4 && !small && chunks_uniform(quad, I.Mpad, 2);
-    }
-    if (wide) {
-      I.uni = 1;
-      I.cvec = 2;
-      I.run = 4;
-    } else if (tile_x == 32) {
-      set_error("tile_x 32 needs chunk-uniform directions with 2 ordinates per lane");
-      return RT_EINVAL;
-    } else if (variant != 1) {
-      for (int V = (variant == 2 && vec == 0 ? 4 : I.cvec); V >= 2; V /= 2) {
-        if (chunks_uniform(quad, I.Mpad, V)) {
-          I.uni = 1;
-          I.cvec = V;
-          break;
-        }
-        if (variant == 0 || vec != 0) break;
-      }
-      if (variant == 2 && !I.uni) {
-        set_error("variant 2 needs every ordinate chunk to have one sign of xi and one of eta");
-        return RT_EINVAL;
-      }
-    }
-    // What the caller sees of the choice: chunk-uniform (2) or per-lane (1) directions.
-    // The streaming kernel runs both: always for chunk-uniform ones, and for per-lane
-    // ones unless a number of ordinates per lane was asked for (that is the general
-    // kernel's option; the streaming kernel always takes four, and vec reads 0). The
-    // general kernel is left for quadratures whose signs change too often for windows
-    // of 32: at 1000^2 x 128, where both run, it takes 0.84 ms per Heun step against
-    // 0.59, at 531^2 x 100 0.52 against 0.24, at 140^2 x 128 0.076 against 0.055.
-    I.info_variant = I.uni ? 2 : 1;
-    I.info_vec = I.cvec;
-    if (I.uni || vec == 0) I.str_chunks = plan_stream_chunks(quad, I.Mpad, storage);
-    // whether as long a segment as asked for fits the shared memory of a CTA
-    auto fits = [&](int run) {
-      const int stage_hi = integrator == RT_HEUN ? STAGE_HEUN2 : STAGE_EULER;
-      return tile_y <= 0 || cart_smem_bytes(order, storage, run, 4, std::min(tile_y, 256), stage_hi,
-                                            ordered_form(I, run)) <= 227 * 1024;
-    };
-    I.ord_vec = 0;
-    if (order == 2 && n_cells <= kOrderedMaxCells && !I.str_chunks.empty()) {
-      if (I.cvec > 1 && windows_whole(I.str_chunks, I.Mpad)) I.ord_vec = I.cvec;
-      if (I.ord_vec && !fits(I.run)) I.ord_vec = 0;
-      if (!I.ord_vec && !I.uni) I.str_chunks.clear();
-    }
-    if (!I.str_chunks.empty()) {
-      if (!I.uni) I.info_vec = 0;
-      I.uni = 1;
-      I.cvec = 4;
-      if (tile_x == 0 && I.run == 4 && I.order == 2 && n_cells > kWideMaxCells) I.run = 2;
-      // one or two chunks (64 ordinates): a tile of 16 cells leaves half of a CTA's warps
-      // without a chunk, which costs less than larger tiles only on small grids
-      // (70^2 x 64 Heun: 35.4 us per step with 16, 38.5 with 32); the ordered form gains up to
-      // four (280^2 x 128: 103 us with 16, 96 with 32), and no more beyond (280^2 x 512: 294, 342)
-      if (tile_x == 0 && I.run == 2 && I.str_chunks.size() <= (I.ord_vec ? 4u : 2u)) {
-        double narrow, wider;
-        stream_segment(I, 2, ordered_form(I, 2), &narrow);
-        stream_segment(I, 4, ordered_form(I, 4), &wider);
-        if (wider < narrow && fits(4)) I.run = 4;
-      }
-      I.uni = ordered_form(I, I.run);
-    } else {
-      I.uni = 0;
-      I.run = 2;
-    }
-    choose_cart_tiles(I, tile_y);
+    if ((s = plan_cart(I, quad, tile_x, tile_y, variant, vec)) != RT_OK) return s;
     I.stage_items.clear();
     const int n = I.n_strips * I.n_segs;
     for (int g = 0; g < I.n_segs; ++g)
@@ -890,9 +910,6 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
         w.inst = 0; w.a = st; w.b = g; w.item = (int32_t)I.stage_items.size(); w.count = n;
         I.stage_items.push_back(w);
       }
-    const int stage_hi = integrator == RT_HEUN ? STAGE_HEUN2 : STAGE_EULER;
-    I.cart_smem = cart_smem_bytes(order, storage, I.run, I.cvec, I.ly, stage_hi, I.uni);
-    if (I.cart_smem > 227 * 1024) { set_error("tile %dx%d needs %zu bytes of shared memory", I.tx, I.ly, I.cart_smem); return RT_EINVAL; }
   } else {
     // persistent work items: item g processes chunks g, g + G, ..., with as many items
     // as the kernel has CTAs resident
