@@ -28,9 +28,9 @@ def device_key() -> str:
 
 
 def shape_key(problem, M: int, order: int, integrator: int, storage: int) -> str:
-    # "stream": the kernel family; entries tuned for kernels that are gone are not used
+    # "stream2": the kernel family and its candidates; entries tuned among others are not used
     m = problem.mesh
-    return f"{device_key()}|stream|cart{m.nx}x{m.ny}|M{M}|o{order}|i{integrator}|s{storage}"
+    return f"{device_key()}|stream2|cart{m.nx}x{m.ny}|M{M}|o{order}|i{integrator}|s{storage}"
 
 
 def _load() -> dict:

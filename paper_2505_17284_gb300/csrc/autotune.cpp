@@ -2,9 +2,9 @@
 // (strip width, segment length, direction family) of one problem on the
 // current device and returns the fastest. Each candidate is a complete solver
 // built through the public entry points, so what is timed is what rt_step runs.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <tuple>
 #include <vector>
 
 #include "host_common.h"
@@ -40,7 +40,7 @@ extern "C" rt_status rt_autotune(const rt_mesh* mesh, const rt_materials* mat, c
     set_error("event creation failed");
     return RT_ECUDA;
   }
-  std::vector<std::tuple<int, int, int, int>> seen;
+  std::vector<CartKey> seen;
   double best_ms = INFINITY;
   rt_options best_opts = *opts;
   rt_status result = RT_OK;
@@ -49,30 +49,36 @@ extern "C" rt_status rt_autotune(const rt_mesh* mesh, const rt_materials* mat, c
     o.tile_x = c.tile_x;
     o.tile_y = c.tile_y;
     o.variant = c.variant;
+    // what would run is known before anything is built (each candidate is a whole state);
+    // the first one is built in any case, and so checks the problem
+    CartKey key{};
+    if (!seen.empty()) {
+      const rt_status st = cart_launch_key(mesh, quad, o, &key);
+      if (st == RT_EINVAL) continue;   // not available for this problem (quadrature, shared memory)
+      if (std::find(seen.begin(), seen.end(), key) != seen.end()) continue;
+    }
     rt_solver* s = nullptr;
     rt_status st = rt_create(mesh, mat, quad, bc, &o, &s);
-    if (st == RT_EINVAL) continue;   // not available for this problem (quadrature, shared memory)
     if (st != RT_OK) { result = st; break; }
-    rt_info_t info;
-    rt_info(s, &info);
-    const auto key = std::make_tuple(info.tile_x, info.tile_y, info.variant, info.vec);
-    bool dup = false;
-    for (const auto& k : seen) dup = dup || (k == key);
-    const int64_t n = std::min<int64_t>(steps, info.n_steps - 1);
-    if (dup || n < 1) {
+    if (seen.empty() && (st = cart_launch_key(mesh, quad, o, &key)) != RT_OK) {
       rt_destroy(s);
-      if (n < 1 && !dup && std::isinf(best_ms)) {   // too few steps to time: keep the library's choice
-        best_opts = o;
-        best_opts.tile_x = info.tile_x;
-        best_opts.tile_y = info.tile_y;
-        best_opts.variant = info.variant;
-        best_opts.vec = info.vec;
-        best_ms = 0.0;
-        break;
-      }
-      continue;
+      result = st;
+      break;
     }
     seen.push_back(key);
+    rt_info_t info;
+    rt_info(s, &info);
+    const int64_t n = std::min<int64_t>(steps, info.n_steps - 1);
+    if (n < 1) {   // too few steps to time: keep the library's choice
+      rt_destroy(s);
+      best_opts = o;
+      best_opts.tile_x = info.tile_x;
+      best_opts.tile_y = info.tile_y;
+      best_opts.variant = info.variant;
+      best_opts.vec = info.vec;
+      best_ms = 0.0;
+      break;
+    }
     float ms = 0.f;
     if ((st = rt_step(s, 1)) == RT_OK) {
       cudaEventRecord(e0, stream);

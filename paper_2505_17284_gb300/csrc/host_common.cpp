@@ -811,6 +811,28 @@ static rt_status plan_cart(Instance& I, const rt_quadrature* quad, int tile_x, i
   return RT_OK;
 }
 
+rt_status cart_launch_key(const rt_mesh* mesh, const rt_quadrature* quad, const rt_options& o, CartKey* key) {
+  Instance I;
+  I.order = o.order; I.integrator = o.integrator; I.storage = o.storage;
+  I.nx = mesh->nx; I.ny = mesh->ny;
+  I.n_cells = (int64_t)mesh->nx * mesh->ny;
+  std::vector<double> xi, eta, w;
+  std::vector<int32_t> kmap, inv;
+  rt_quadrature rq{};
+  if (o.variant != 1 && regroup_quadrature(quad, xi, eta, w, kmap, inv)) {
+    rq.M = (int64_t)xi.size();
+    rq.xi = xi.data();
+    rq.eta = eta.data();
+    rq.w = w.data();
+    quad = &rq;
+    I.regrouped = 1;
+  }
+  I.Mpad = (int32_t)((quad->M + 31) / 32 * 32);
+  const rt_status s = plan_cart(I, quad, o.tile_x, o.tile_y, o.variant, o.vec);
+  if (s == RT_OK) *key = {I.uni, I.run, I.ly, I.cvec, I.ord_vec, I.Mpad, I.regrouped};
+  return s;
+}
+
 // ---------------------------------------------------------------- build
 rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_quadrature* quad,
                          const rt_boundary* bc, int order, int integrator, int storage, double dt_target,

@@ -6,6 +6,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <array>
 #include <string>
 #include <vector>
 
@@ -87,6 +88,12 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
                          const rt_boundary* bc, int order, int integrator, int storage, double dt, double t_end,
                          int tile_x, int tile_y, DeviceArena& arena, cudaStream_t stream, Instance& inst,
                          std::vector<std::vector<char>>& host_keepalive, int variant = 0, int vec = 0);
+
+// What a Cartesian problem's launches are determined by: kernel, tile, segment and layout of
+// the ordinates. Two sets of options with the same key run the same. No device memory; the
+// arguments must be those of a problem that rt_create accepts but for the kernel options.
+using CartKey = std::array<int32_t, 7>;
+rt_status cart_launch_key(const rt_mesh* mesh, const rt_quadrature* quad, const rt_options& opts, CartKey* key);
 
 int device_sm_count();
 

@@ -1,4 +1,5 @@
-"""The kernel options that the library reports and the tuner returns can be asked for."""
+"""The kernel options that the library reports and the tuner returns can be asked for, and the
+tuner times the library's own choice and nothing twice."""
 import numpy as np
 import pytest
 
@@ -44,10 +45,25 @@ def test_reported_options_can_be_asked_for(rt, rule, n, order):
     b.close()
 
 
-@pytest.mark.parametrize("rule,n,order", [((4, 16), 140, 2), ((4, 16), 280, 1), ((16, 32), 100, 1)])
-def test_tuned_options_can_be_asked_for(rt, rule, n, order):
+@pytest.mark.parametrize("rule,n,order,most", [((4, 16), 140, 2, 24), ((4, 16), 280, 1, 24), ((16, 32), 330, 2, 24),
+                                               ((16, 32), 100, 1, 24), ((8, 16), 350, 2, 12)])
+def test_tuner_builds_each_configuration_once(rt, monkeypatch, rule, n, order, most):
+    """At most 12 segment lengths (one of them automatic) for each tile width, the library's own width among them."""
+    import torch
     p, quad = si.lattice_problem(n), rt.rt_quad_product(*rule)
+    own = rt.Solver(p, quad, order=order, integrator=rt.RT_HEUN)
+    psi_bytes, width = int(own.info.n_cells) * int(own.info.M_pad) * 4, own.info.tile_x
+    own.close()
+    sizes, alloc = [], torch.cuda.caching_allocator_alloc
+
+    def counting(size, *args):
+        sizes.append(size)
+        return alloc(size, *args)
+
+    monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", counting)
     cfg, ms = rt.rt_autotune(p, quad, order=order, integrator=rt.RT_HEUN, steps=1)
+    builds = sum(s == -(-psi_bytes // 256) * 256 for s in sizes) // 2   # two buffers of psi each
+    assert 11 <= builds <= most and (width == 16 or builds > 12)
     s = rt.Solver(p, quad, order=order, integrator=rt.RT_HEUN, **{k: cfg[k] for k in ("tile_x", "tile_y", "variant", "vec")})
     assert options(s) == (cfg["tile_x"], cfg["tile_y"], cfg["variant"], cfg["vec"])
     s.close()
