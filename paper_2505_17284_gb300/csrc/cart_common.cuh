@@ -75,18 +75,10 @@ __device__ __forceinline__ void stg_vec(T* p, const float (&in)[V]) {
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   return __ffma2_rn(b, make_float2(-1.f, -1.f), a);   // a - b, rounded once
 }
-__device__ __forceinline__ float2 minmod2(float2 a, float2 b) {
-  return make_float2(minmod_med(a.x, b.x), minmod_med(a.y, b.y));
-}
 __device__ __forceinline__ float2 relu2(float2 a) { return make_float2(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f)); }
 // minmod(a, b) = min(max(a, b), max(a, 0), max(b, 0)), the last two given: for
 // a <= b this is a when 0 <= a, 0 when a < 0 <= b and b when b < 0, i.e. the
 // median of (a, b, 0). A difference feeds two faces, so its max(., 0) is shared.
-__device__ __forceinline__ float fmin3f(float a, float b, float c) {
-  float r;
-  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
 __device__ __forceinline__ float2 minmod2r(float2 a, float2 b, float2 ra, float2 rb) {
   return make_float2(fmin3f(fmaxf(a.x, b.x), ra.x, rb.x), fmin3f(fmaxf(a.y, b.y), ra.y, rb.y));
 }

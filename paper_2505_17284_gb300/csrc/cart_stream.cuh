@@ -50,13 +50,12 @@
 // and 55 us, 280^2 x 256 163 and 180; the general kernel 111 and 320.
 //
 // Bound by: HBM on large grids (1400^2 x 512 FP32 Heun: 20 bytes per cell and ordinate
-// at 5.4 TB/s; a pair of rows is about 500 instructions for 16 values a lane, issue
+// at 5.6 TB/s; a pair of rows is about 500 instructions for 16 values a lane, issue
 // slots half used), by instruction latency and the fixed cost of a launch on small ones.
 // Per Heun step, against the kernels that it replaced (one CTA barrier per row with
 // chunk-uniform directions; for mixed directions the general kernel of
-// cart_kernel.cuh): 1400^2 x 512 4.11 -> 3.78 ms (BF16 4.42 -> 3.81, first-order Euler
-// 1.50 -> 1.36), 700^2 x 484 1.36 -> 1.17, 531^2 x 100 0.57 -> 0.26, 280^2 x 256 0.32
-// -> 0.17, 140^2 x 128 0.11 -> 0.05. Measured and not kept: 4 cells per lane (12 warps
+// cart_kernel.cuh): 1400^2 x 512 4.12 -> 3.57 ms (BF16 4.42 -> 3.69, first-order Euler
+// 1.51 -> 1.36), 700^2 x 484 1.36 -> 1.16, 531^2 x 100 0.57 -> 0.25. Measured and not kept: 4 cells per lane (12 warps
 // per SM: spills, and a loop too long for the instruction cache), scalar instead of
 // paired FP32 (24 % slower), prefetching the pair after next to L2.
 #pragma once
@@ -125,7 +124,6 @@ struct StrEdge {
   int nx, ny, periodic_x, periodic_y;
   float ghost[4];   // psi^- of the sides
 };
-constexpr size_t kStrEdgeBytes = 64;
 
 // One warp's strip: what the row walk needs from the descriptor and the tile.
 struct StrWarp {

@@ -79,8 +79,6 @@ __device__ __forceinline__ uint2 sr_bits4(uint32_t cell, uint32_t gkey) {
   h2 ^= h2 >> 13;
   return make_uint2(h, h2);
 }
-// the 32 random bits of the pair (4g + 2p, 4g + 2p + 1), p = 0 or 1
-__device__ __forceinline__ uint32_t sr_pair(uint2 b, int p) { return p ? b.y : b.x; }
 // the 16 random bits (low half) of ordinate 4g + e
 __device__ __forceinline__ uint32_t sr_elem(uint2 b, int e) {
   const uint32_t w = (e & 2) ? b.y : b.x;
@@ -185,10 +183,16 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
 }
 
 // ------------------------------------------------------------------ math
-// minmod(a, b): 0 unless a and b have the same sign, else the one of smaller magnitude.
-__device__ __forceinline__ float minmod(float a, float b) {
-  const float m = fminf(fabsf(a), fabsf(b));
-  return (a * b > 0.f) ? copysignf(m, a) : 0.f;
+// Three-operand minimum and maximum (one instruction each).
+__device__ __forceinline__ float fmin3f(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float fmax3f(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -251,12 +255,6 @@ __device__ __forceinline__ float multi_warp_sum(float (&v)[V], int lane) {
       }
     }
   }
-}
-
-// Lane that holds the total of value index u after multi_warp_sum<V>.
-template <int V>
-__device__ __forceinline__ constexpr int multi_sum_lane(int u) {
-  return u * (32 / V);
 }
 
 // ------------------------------------------------------------------ QoI finalize

@@ -469,9 +469,7 @@ static std::vector<int4> plan_stream_chunks(const rt_quadrature* quad, int Mpad,
             lx = lx ? lx : x;
           }
         }
-        const bool whole = k == base && hi == base + 32;
-        out.push_back(make_int4(base, (k - base) | (hi - base) << 8, sy < 0 ? -1 : 1,
-                                mixed || !whole ? 0 : (dx < 0 ? -1 : 1)));
+        out.push_back(make_int4(base, (k - base) | (hi - base) << 8, sy < 0 ? -1 : 1, 0));
         k = hi;
       }
     }

@@ -90,7 +90,7 @@ struct alignas(128) InstDesc {
   double dt_d, area_d, dx_d, dy_d;  // Cartesian cell area and sizes (FP64 QoIs)
   float ghost[4];               // inflow value per side (entering ordinates)
   // streaming Cartesian kernel: per chunk {first ordinate of the 32, lo | hi << 8 (the
-  // chunk's ordinates within them), sign of eta, sign of xi or 0 if the lanes differ}
+  // chunk's ordinates within them), sign of eta, 0}
   const int4* str_chunks;
   float sig_t[kMaxMat];
   float sig_s2pi[kMaxMat];      // sigma_s / (2 pi)

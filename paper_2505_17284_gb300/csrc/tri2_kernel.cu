@@ -96,17 +96,6 @@ __device__ __forceinline__ float venkat_exact(float x, float y, float eps2) {
   return den > 0.f ? (c + p) / den : 1.f;
 }
 
-__device__ __forceinline__ float fmin3f(float a, float b, float c) {
-  float r;
-  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-__device__ __forceinline__ float fmax3f(float a, float b, float c) {
-  float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-
 // Quotients a / b of pairs of positive floats, b and 1 / b in the normal range: the product
 // with the approximate reciprocal, corrected once by its residual a - q b, which a fused
 // operation gives exactly (P. Markstein, Computation of elementary functions on the IBM RISC

@@ -11,7 +11,7 @@
 // sn_2d_eqn_fv). The warp sums w_k out_k over all ordinates to phi_out of the cell.
 // Bound by the latency of the gathers: 1300^2 x 256 first-order Euler 2.36 -> 2.00 ms
 // with differences instead of selected traces, cell tables and the next cell's row
-// fetched to L2 (the staged kernel takes 1.66).
+// fetched to L2 (the staged kernel takes 1.70).
 #include <cuda_bf16.h>
 
 #include "device_common.cuh"

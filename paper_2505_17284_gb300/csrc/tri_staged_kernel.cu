@@ -33,7 +33,7 @@
 // cell of 256 ordinates, 44 % of the slots; DRAM 8.1 bytes per cell and ordinate at
 // half of its peak). 1300^2 x 256 first-order Euler, FP32: with selects between the
 // traces, two barriers per block, one thread's QoI sums per cell and per-row bulk copies
-// (which a warp issues lane by lane) 2.28 ms; now 1.66. 650^2 x 256 BF16 0.61 -> 0.42.
+// (which a warp issues lane by lane) 2.28 ms; now 1.70. 650^2 x 256 BF16 0.61 -> 0.42.
 #include <cuda_bf16.h>
 
 #include <type_traits>
@@ -483,14 +483,9 @@ __global__ void __launch_bounds__(kStgThreads, 2)
   finalize_item<kStgThreads>(d, it, red, STAGE, red + NQ);
 }
 
-// Ordinates per lane of the staged kernel: those of the instance.
-static int stg_vec(int, int vec) { return vec; }
-
 size_t tri_staged_smem_bytes(int vec, int storage, int hmax, int stage) {
-  return stg_layout(stg_vec(storage, vec), storage == 1 ? 2 : 4, hmax, stage == STAGE_HEUN2).total;
+  return stg_layout(vec, storage == 1 ? 2 : 4, hmax, stage == STAGE_HEUN2).total;
 }
-
-int tri_staged_threads() { return kStgThreads; }
 
 template <int VEC, int STAGE, typename T>
 static cudaError_t stg_prepare_one(size_t smem) {
@@ -516,7 +511,6 @@ constexpr size_t kStgSmemCap = 108 * 1024;   // two CTAs per SM
 
 cudaError_t prepare_tri_staged(int stage, int storage, int vec, int hmax) {
   if (tri_staged_smem_bytes(vec, storage, hmax, stage) > kStgSmemCap) return cudaErrorInvalidValue;
-  vec = stg_vec(storage, vec);
   const size_t smem = kStgSmemCap;
 #define RTK_P(V, ST, TT) \
   if (vec == V && stage == ST) return stg_prepare_one<V, ST, TT>(smem);
@@ -529,7 +523,6 @@ cudaError_t launch_tri_staged(const InstDesc* d_desc, const WorkItem* d_items, i
                               int vec, int hmax, cudaStream_t s, bool chained) {
   if (n_items <= 0) return cudaSuccess;
   const size_t smem = tri_staged_smem_bytes(vec, storage, hmax, stage);
-  vec = stg_vec(storage, vec);
 #define RTK_L(V, ST, TT) \
   if (vec == V && stage == ST) return stg_launch_one<V, ST, TT>(d_desc, d_items, n_items, smem, s, chained);
   if (storage == 0) { RTK_STG_ALL(RTK_L, float) } else { RTK_STG_ALL(RTK_L, __nv_bfloat16) }
