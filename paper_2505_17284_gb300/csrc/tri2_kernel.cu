@@ -28,9 +28,10 @@
 // vanish, and the rounding error is smaller (650^2 x 256, one step against FP64: 4.22e-8
 // of psi, 4.33e-8 with values). At 400^2 x 256 (FP32), with IEEE divisions in divergent
 // branches and 2 ordinates per lane in the stage pass: gradient 0.82 ms, stage 0.45 ms;
-// now 0.29 and 0.35 ms. A Heun step at 650^2 x 256: 6.65 -> 3.42 ms (3.29 with quotients that
-// were 2 ulp off).
+// now 0.27 and 0.35 ms. A Heun step at 650^2 x 256: 6.65 -> 3.27 ms.
 #include <cuda_bf16.h>
+
+#include <type_traits>
 
 #include "device_common.cuh"
 
@@ -79,6 +80,49 @@ __device__ __forceinline__ void t2_bulk_load(void* dst, const void* src, uint32_
                : "memory");
 }
 
+// Arithmetic on a pair of ordinates (FP32 pairs: two values per instruction), or on the one
+// ordinate of a lane (a pair of itself would take twice the scalar operations: 260^2 x 32
+// Heun 241 us against 222).
+__device__ __forceinline__ float t2_fma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ float2 t2_fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float t2_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float2 t2_mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float t2_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float2 t2_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float t2_neg(float a) { return -a; }
+__device__ __forceinline__ float2 t2_neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float t2_abs(float a) { return fabsf(a); }
+__device__ __forceinline__ float2 t2_abs(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
+__device__ __forceinline__ float t2_min3(float a, float b, float c) { return fmin3f(a, b, c); }
+__device__ __forceinline__ float2 t2_min3(float2 a, float2 b, float2 c) {
+  return make_float2(fmin3f(a.x, b.x, c.x), fmin3f(a.y, b.y, c.y));
+}
+__device__ __forceinline__ float t2_max3(float a, float b, float c) { return fmax3f(a, b, c); }
+__device__ __forceinline__ float2 t2_max3(float2 a, float2 b, float2 c) {
+  return make_float2(fmax3f(a.x, b.x, c.x), fmax3f(a.y, b.y, c.y));
+}
+__device__ __forceinline__ float t2_pos(float a) { return fmaxf(a, 0.f); }
+__device__ __forceinline__ float2 t2_pos(float2 a) { return make_float2(fmaxf(a.x, 0.f), fmaxf(a.y, 0.f)); }
+__device__ __forceinline__ float t2_pick(float s, float a, float b) { return s > 0.f ? a : b; }   // a where s > 0
+__device__ __forceinline__ float2 t2_pick(float2 s, float2 a, float2 b) {
+  return make_float2(s.x > 0.f ? a.x : b.x, s.y > 0.f ? a.y : b.y);
+}
+__device__ __forceinline__ float t2_least(float a) { return a; }
+__device__ __forceinline__ float t2_least(float2 a) { return fminf(a.x, a.y); }
+__device__ __forceinline__ float t2_most(float a) { return a; }
+__device__ __forceinline__ float t2_most(float2 a) { return fmaxf(a.x, a.y); }
+template <typename P>
+__device__ __forceinline__ P t2_dup(float a) {
+  if constexpr (sizeof(P) == 4) return a;
+  else return make_float2(a, a);
+}
+__device__ __forceinline__ float t2_rcp(float a) {   // approximate reciprocal of a float in the normal range
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+  return r;
+}
+__device__ __forceinline__ float2 t2_rcp(float2 a) { return make_float2(t2_rcp(a.x), t2_rcp(a.y)); }
+
 // psi^- of boundary side s for an ordinate: the side's inflow value if the
 // ordinate enters through it (outward normals x- (-1,0), x+ (1,0), y- (0,-1),
 // y+ (0,1)), else 0
@@ -96,24 +140,23 @@ __device__ __forceinline__ float venkat_exact(float x, float y, float eps2) {
   return den > 0.f ? (c + p) / den : 1.f;
 }
 
-// Quotients a / b of pairs of positive floats, b and 1 / b in the normal range: the product
-// with the approximate reciprocal, corrected once by its residual a - q b, which a fused
-// operation gives exactly (P. Markstein, Computation of elementary functions on the IBM RISC
-// System/6000 processor, 1990). Off from the rounded quotient only where a / b lies within
-// 2^-21 ulp of the middle of two floats.
-__device__ __forceinline__ float2 quotient2(float2 a, float2 b) {
-  float2 r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(b.x));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(b.y));
-  const float2 q = __fmul2_rn(a, r);
-  return __ffma2_rn(__ffma2_rn(make_float2(-q.x, -q.y), b, a), r, q);
+// Quotients a / b of positive floats, b and 1 / b in the normal range: the product with the
+// approximate reciprocal, corrected once by its residual a - q b, which a fused operation
+// gives exactly (P. Markstein, Computation of elementary functions on the IBM RISC System/6000
+// processor, 1990). Off from the rounded quotient only where a / b lies within 2^-21 ulp of the
+// middle of two floats (or, for a below 2^-102, whose residuals are subnormal, 2^-126 / a ulp).
+template <typename P>
+__device__ __forceinline__ P quotient(P a, P b) {
+  const P r = t2_rcp(b), q = t2_mul(a, r);
+  return t2_fma(t2_fma(t2_neg(q), b, a), r, q);
 }
 
-// Smallest of the three edges' limiter values outside the range of quotient2 for the values as
-// they are. Numerators below 2^-117 (they are at most twice the denominators), whose residuals
-// leave the range of floats, are formed again from x and y times 2^63, the quotient being
-// homogeneous: a state of zeros or a front's foot has them where epsilon^2 = A^6 is small
-// (10^-36 at 2 * 650^2 cells). Only states above 10^18 divide by IEEE.
+// Smallest of the three edges' limiter values outside the range of quotient for the values as
+// they are. Denominators below 2^-118 are formed again, with their numerators, from x and y
+// times 2^63, the quotient being homogeneous: a front's foot has them where epsilon^2 = A^6 is
+// small (10^-36 at 2 * 650^2 cells). (Numerators of epsilon^2 over larger denominators, at every
+// extremum of the state, are near enough as they are: testing for them too took 4 % of a step at
+// 650^2 x 256, scaling every cell's terms 3 %.) Only states above 10^18 divide by IEEE.
 __device__ __forceinline__ float limiter_rescaled(float gx, float gy, float up, float dn, const float (&rxh)[3],
                                                   const float (&ryh)[3], float eps2) {
   float x[3], y[3], den[3], L[3];
@@ -133,51 +176,49 @@ __device__ __forceinline__ float limiter_rescaled(float gx, float gy, float up, 
       const float s = den[e] < 0x1p-100f ? 0x1p63f : 1.f;
       const float xs = x[e] * s, ys = y[e] * s, p = xs * ys, c = fmaf(ys, ys, eps2 * s * s) + p;
       const float d = fmaf(xs + xs, xs, c);
-      L[e] = d > 0.f ? quotient2(make_float2(c + p, 1.f), make_float2(d, 1.f)).x : 1.f;   // 0 / 0 without a spread
+      L[e] = d > 0.f ? quotient(c + p, d) : 1.f;   // 0 / 0 without a spread
     }
   }
   return fminf(fminf(L[0], L[1]), L[2]);
 }
 
-// Limited gradient L g of a pair of ordinates from the cell's values c and its
-// neighbours' n0, n1, n2 (FP32 pairs: two values per instruction). The normals of a
-// triangle sum to zero, so the Green-Gauss sum of l n (c + n_e)/2 is that of
-// l n (n_e - c)/2, whose rounding error scales with the differences, not the values.
-__device__ __forceinline__ void limited_gradient2(float2 c, float2 n0, float2 n1, float2 n2, const float (&axh)[3],
-                                                  const float (&ayh)[3], const float (&rxh)[3], const float (&ryh)[3],
-                                                  float eps2, float2& lx, float2& ly) {
-  auto dup = [](float a) { return make_float2(a, a); };
-  const float2 mc = make_float2(-c.x, -c.y);
-  const float2 s0 = __fadd2_rn(n0, mc), s1 = __fadd2_rn(n1, mc), s2 = __fadd2_rn(n2, mc);
-  const float2 gx = __ffma2_rn(dup(axh[2]), s2, __ffma2_rn(dup(axh[1]), s1, __fmul2_rn(dup(axh[0]), s0)));
-  const float2 gy = __ffma2_rn(dup(ayh[2]), s2, __ffma2_rn(dup(ayh[1]), s1, __fmul2_rn(dup(ayh[0]), s0)));
+// Limited gradient L g of a pair of ordinates (or one) from the cell's values c and its
+// neighbours' n0, n1, n2. The normals of a triangle sum to zero, so the Green-Gauss sum of
+// l n (c + n_e)/2 is that of l n (n_e - c)/2, whose rounding error scales with the differences,
+// not the values.
+template <typename P>
+__device__ __forceinline__ void limited_gradient(P c, P n0, P n1, P n2, const float (&axh)[3], const float (&ayh)[3],
+                                                 const float (&rxh)[3], const float (&ryh)[3], float eps2, P& lx, P& ly) {
+  auto dup = [](float a) { return t2_dup<P>(a); };
+  const P mc = t2_neg(c), s0 = t2_add(n0, mc), s1 = t2_add(n1, mc), s2 = t2_add(n2, mc);
+  const P gx = t2_fma(dup(axh[2]), s2, t2_fma(dup(axh[1]), s1, t2_mul(dup(axh[0]), s0)));
+  const P gy = t2_fma(dup(ayh[2]), s2, t2_fma(dup(ayh[1]), s1, t2_mul(dup(ayh[0]), s0)));
   // beta_max and -beta_min
-  const float2 up = make_float2(fmaxf(fmax3f(s0.x, s1.x, s2.x), 0.f), fmaxf(fmax3f(s0.y, s1.y, s2.y), 0.f));
-  const float2 dn = make_float2(-fminf(fmin3f(s0.x, s1.x, s2.x), 0.f), -fminf(fmin3f(s0.y, s1.y, s2.y), 0.f));
-  float2 num[3], den[3];
+  const P up = t2_pos(t2_max3(s0, s1, s2)), dn = t2_pos(t2_neg(t2_min3(s0, s1, s2)));
+  P num[3], den[3];
 #pragma unroll
   for (int e = 0; e < 3; ++e) {
-    const float2 D = __ffma2_rn(dup(ryh[e]), gy, __fmul2_rn(dup(rxh[e]), gx));
-    const float2 x = make_float2(fabsf(D.x), fabsf(D.y));
-    const float2 y = make_float2(D.x > 0.f ? up.x : dn.x, D.y > 0.f ? up.y : dn.y);
-    const float2 p = __fmul2_rn(x, y);
-    const float2 q = __fadd2_rn(__ffma2_rn(y, y, dup(eps2)), p);
-    num[e] = __fadd2_rn(q, p);
-    den[e] = __ffma2_rn(__fadd2_rn(x, x), x, q);
+    const P D = t2_fma(dup(ryh[e]), gy, t2_mul(dup(rxh[e]), gx));
+    const P x = t2_abs(D), y = t2_pick(D, up, dn), p = t2_mul(x, y);
+    const P q = t2_add(t2_fma(y, y, dup(eps2)), p);
+    num[e] = t2_add(q, p);
+    den[e] = t2_fma(t2_add(x, x), x, q);
   }
   // The smallest of the edges' values. Three IEEE divisions in divergent branches were 200 of
   // 269 instructions per cell and ordinate.
-  float2 L;
-  const float lo = fminf(fmin3f(num[0].x, num[1].x, num[2].x), fmin3f(num[0].y, num[1].y, num[2].y));
-  const float hi = fmaxf(fmax3f(den[0].x, den[1].x, den[2].x), fmax3f(den[0].y, den[1].y, den[2].y));
-  if (lo >= 0x1p-117f && hi <= 1e36f) {
-    const float2 l0 = quotient2(num[0], den[0]), l1 = quotient2(num[1], den[1]), l2 = quotient2(num[2], den[2]);
-    L = make_float2(fmin3f(l0.x, l1.x, l2.x), fmin3f(l0.y, l1.y, l2.y));
+  P L;
+  const float lo = t2_least(t2_min3(den[0], den[1], den[2])), hi = t2_most(t2_max3(den[0], den[1], den[2]));
+  if (lo >= 0x1p-118f && hi <= 1e36f) {
+    L = t2_min3(quotient(num[0], den[0]), quotient(num[1], den[1]), quotient(num[2], den[2]));
+  } else if (t2_most(t2_max3(t2_abs(gx), t2_abs(gy), dup(0.f))) == 0.f) {
+    L = dup(1.f);   // no gradient: a state of zeros
+  } else if constexpr (sizeof(P) == 4) {
+    L = limiter_rescaled(gx, gy, up, dn, rxh, ryh, eps2);
   } else {
     L = make_float2(limiter_rescaled(gx.x, gy.x, up.x, dn.x, rxh, ryh, eps2), limiter_rescaled(gx.y, gy.y, up.y, dn.y, rxh, ryh, eps2));
   }
-  lx = __fmul2_rn(L, gx);
-  ly = __fmul2_rn(L, gy);
+  lx = t2_mul(L, gx);
+  ly = t2_mul(L, gy);
 }
 
 // Fetch the rows of a cell to L2, a 128-byte line per lane at a time: na lines at a,
@@ -293,7 +334,7 @@ __global__ void __launch_bounds__(t2_grad_threads(VEC), t2_ctas(VEC))
 #pragma unroll
           for (int l = 0; l < VEC; l += 2) {
             float2 gx, gy;
-            limited_gradient2(make_float2(c[l], c[l + 1]), make_float2(nb3[0][l], nb3[0][l + 1]),
+            limited_gradient<float2>(make_float2(c[l], c[l + 1]), make_float2(nb3[0][l], nb3[0][l + 1]),
                               make_float2(nb3[1][l], nb3[1][l + 1]), make_float2(nb3[2][l], nb3[2][l + 1]), axh, ayh, rxh,
                               ryh, eps2, gx, gy);
             ox[l] = gx.x;
@@ -302,11 +343,7 @@ __global__ void __launch_bounds__(t2_grad_threads(VEC), t2_ctas(VEC))
             oy[l + 1] = gy.y;
           }
         } else {
-          float2 gx, gy;   // the pair's second value is not used
-          limited_gradient2(make_float2(c[0], c[0]), make_float2(nb3[0][0], nb3[0][0]), make_float2(nb3[1][0], nb3[1][0]),
-                            make_float2(nb3[2][0], nb3[2][0]), axh, ayh, rxh, ryh, eps2, gx, gy);
-          ox[0] = gx.x;
-          oy[0] = gy.x;
+          limited_gradient<float>(c[0], nb3[0][0], nb3[1][0], nb3[2][0], axh, ayh, rxh, ryh, eps2, ox[0], oy[0]);
         }
         st_vec<float, VEC>(row_g, ox);
         st_vec<float, VEC>(row_g + Mpad, oy);
@@ -472,37 +509,44 @@ __global__ void __launch_bounds__(kT2Threads, t2_ctas(VEC))
         // BF16 rounding bits of the lane's ordinates kk .. kk+VEC-1 (one group of four)
         [[maybe_unused]] uint2 rb4;
         if constexpr (sizeof(T) == 2) rb4 = sr_bits4((uint32_t)cell, sr_gkey(kk >> 2, salt));
-        // ordinate pairs (two FP32 values per instruction); a single ordinate is a pair of itself
+        // ordinate pairs (two FP32 values per instruction), or the lane's one ordinate
+        using P = std::conditional_t<(VEC > 1), float2, float>;
 #pragma unroll
         for (int l = 0; l < VEC; l += 2) {
-          const int l1 = VEC > 1 ? l + 1 : l;
-          auto pair = [&](const float (&a)[VEC]) { return make_float2(a[l], a[l1]); };
-          auto dup = [](float a) { return make_float2(a, a); };
-          const float2 c2 = pair(c), xi2 = pair(xi), eta2 = pair(eta), cx2 = pair(cx), cy2 = pair(cy);
+          auto pair = [&](const float (&a)[VEC]) {
+            if constexpr (VEC > 1) return make_float2(a[l], a[l + 1]);
+            else return a[l];
+          };
+          auto dup = [](float a) { return t2_dup<P>(a); };
+          const P c2 = pair(c), xi2 = pair(xi), eta2 = pair(eta), cx2 = pair(cx), cy2 = pair(cy);
           // traces less the cell's value: omega . n l / A sums to zero over the edges
-          const float2 mc2 = make_float2(-c2.x, -c2.y);
-          float2 div = make_float2(0.f, 0.f);
+          const P mc2 = t2_neg(c2);
+          P div = dup(0.f);
 #pragma unroll
           for (int e = 0; e < 3; ++e) {
-            const float2 on = __ffma2_rn(eta2, dup(ay[e]), __fmul2_rn(xi2, dup(ax[e])));
-            const float2 mine = __ffma2_rn(cx2, dup(rx[e]), __fmul2_rn(cy2, dup(ry[e])));
-            const float2 other = __ffma2_rn(pair(nx[e]), dup(sx[e]),
-                                            __ffma2_rn(pair(ny[e]), dup(sy[e]), __fadd2_rn(pair(nbv[e]), mc2)));
-            div = __ffma2_rn(on, make_float2(on.x > 0.f ? mine.x : other.x, on.y > 0.f ? mine.y : other.y), div);
+            const P on = t2_fma(eta2, dup(ay[e]), t2_mul(xi2, dup(ax[e])));
+            const P mine = t2_fma(cx2, dup(rx[e]), t2_mul(cy2, dup(ry[e])));
+            const P other = t2_fma(pair(nx[e]), dup(sx[e]), t2_fma(pair(ny[e]), dup(sy[e]), t2_add(pair(nbv[e]), mc2)));
+            div = t2_fma(on, t2_pick(on, mine, other), div);
           }
-          const float2 F = __fadd2_rn(__ffma2_rn(dup(-sig_t), c2, make_float2(-div.x, -div.y)), dup(src));
-          float2 o;
+          const P F = t2_add(t2_fma(dup(-sig_t), c2, t2_neg(div)), dup(src));
+          P o;
           if constexpr (STAGE == STAGE_HEUN2) {
-            o = __fmul2_rn(dup(0.5f), __ffma2_rn(dup(dt), F, __fadd2_rn(pair(base), c2)));
+            o = t2_mul(dup(0.5f), t2_fma(dup(dt), F, t2_add(pair(base), c2)));
           } else {
-            o = __ffma2_rn(dup(dt), F, c2);
+            o = t2_fma(dup(dt), F, c2);
           }
-          if constexpr (sizeof(T) == 2) {
-            o.x = Store<T>::round_sr(o.x, sr_elem(rb4, (kk + l) & 3));
-            o.y = Store<T>::round_sr(o.y, sr_elem(rb4, (kk + l1) & 3));
+          if constexpr (VEC > 1) {
+            if constexpr (sizeof(T) == 2) {
+              o.x = Store<T>::round_sr(o.x, sr_elem(rb4, (kk + l) & 3));
+              o.y = Store<T>::round_sr(o.y, sr_elem(rb4, (kk + l + 1) & 3));
+            }
+            out[l] = o.x;
+            out[l + 1] = o.y;
+          } else {
+            if constexpr (sizeof(T) == 2) o = Store<T>::round_sr(o, sr_elem(rb4, kk & 3));
+            out[l] = o;
           }
-          out[l] = o.x;
-          if constexpr (VEC > 1) out[l1] = o.y;
         }
         st_vec<T, VEC>(psi_out + (size_t)cell * Mpad + kk, out);
 #pragma unroll

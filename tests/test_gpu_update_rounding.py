@@ -91,7 +91,7 @@ def second_order_euler(mesh, quad, psi, sigma, dt):
     gx, gy = (fm(h * a[:, 2:3], d3[2], fm(h * a[:, 1:2], d3[1], h * a[:, 0:1] * d3[0])) for a in (ax, ay))
     up, dn = np.maximum(np.maximum.reduce(d3), 0), -np.minimum(np.minimum.reduce(d3), 0)
     def limiter(scale):
-        """(smallest of the three edges' values, smallest numerator); x and y times 2^63 where den < 2^-100 if asked for."""
+        """(smallest of the three edges' values, smallest denominator); x and y times 2^63 where den < 2^-100 if asked for."""
         L = lo = None
         for e in range(3):
             D = fm(h * r[:, e, 1:2], gy, h * r[:, e, 0:1] * gx)
@@ -101,14 +101,15 @@ def second_order_euler(mesh, quad, psi, sigma, dt):
             x, y = x * k, y * k
             p = x * y
             q = fm(y, y, eps2 * k * k) + p
-            one, num = (q + p) / fm(x + x, x, q), q + p
-            L, lo = (one, num) if L is None else (np.minimum(L, one), np.minimum(lo, num))
+            den = fm(x + x, x, q)
+            one = (q + p) / den
+            L, lo = (one, den) if L is None else (np.minimum(L, one), np.minimum(lo, den))
         return L, lo
 
     L, lo = limiter(False)
-    if lo.min() < 2.0 ** -117:   # the kernels rescale where residuals would leave the range of floats
+    if lo.min() < 2.0 ** -118:   # the kernels rescale where residuals would leave the range of floats
         pair = M > 32            # (both values of a lane's pair together)
-        low = lo < f32(2.0 ** -117)
+        low = lo < f32(2.0 ** -118)
         low = (low | np.stack([low[:, 1::2], low[:, ::2]], 2).reshape(low.shape)) if pair else low
         L = np.where(low, limiter(True)[0], L)
     lx, ly = L * gx, L * gy
