@@ -245,7 +245,8 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
   float xsum = 0.f;
   {
     const float dt = d.dt;
-    const float half = ORD ? 1.f : STAGE == STAGE_HEUN2 ? -0.5f : -1.f;   // stage 2 averages psi^n and the update
+    // stage 2 averages psi^n and the update: the halves (of a and b, too) are exact
+    const float half = (ORD ? 1.f : -1.f) * (STAGE == STAGE_HEUN2 ? 0.5f : 1.f);
     const int lo = ch.x + (ch.y & 255), hi = ch.x + (ch.y >> 8);
     float wv[4], ax[4], ay[4];
 #pragma unroll
@@ -433,14 +434,9 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
           float2 t = __ffma2_rn(make_float2(ab.x, ab.x), C.c[r][v], make_float2(ab.y, ab.y));
-          if constexpr (ORD) {
-            t = sub2(t, out[r][v]);
-            out[r][v] = STAGE == STAGE_HEUN2 ? __fmul2_rn(make_float2(0.5f, 0.5f), __fadd2_rn(base[v], t)) : t;
-          } else if constexpr (STAGE == STAGE_HEUN2) {
-            out[r][v] = __ffma2_rn(make_float2(0.5f, 0.5f), __fadd2_rn(base[v], t), out[r][v]);
-          } else {
-            out[r][v] = __fadd2_rn(t, out[r][v]);
-          }
+          t = ORD ? sub2(t, out[r][v]) : __fadd2_rn(t, out[r][v]);
+          // (the sum of the update first: psi^n and it are of one size, and their sum rounds at twice that)
+          out[r][v] = STAGE == STAGE_HEUN2 ? __ffma2_rn(make_float2(0.5f, 0.5f), base[v], t) : t;
         }
       }
       if constexpr (sizeof(T) == 2) {
@@ -726,7 +722,7 @@ __global__ void __launch_bounds__(kStrThreads, 2)
     }
   }
   // per-cell constants of the tile: a = 1 - dt sigma_t, b = dt (sigma_s/(2 pi) phi + Q)
-  const float dt = d.dt;
+  const float dt = d.dt, half = STAGE == STAGE_HEUN2 ? 0.5f : 1.f;
   for (int i = tid; i < nrows * TX; i += kStrThreads) {
     const int gx = x0 + (i & (TX - 1));
     float a = 1.f, b = 0.f;
@@ -736,7 +732,7 @@ __global__ void __launch_bounds__(kStrThreads, 2)
       a = 1.f - dt * d.sig_t[m];
       b = dt * (d.sig_s2pi[m] * phi_in[cell] + d.q_src[m]);
     }
-    tile_ab[i] = make_float2(a, b);
+    tile_ab[i] = make_float2(half * a, half * b);
   }
   for (int i = tid; i < (ORD ? 1 : WC) * d.ly * TX; i += kStrThreads) tile_acc[i] = 0.f;
   __syncthreads();

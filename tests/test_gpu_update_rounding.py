@@ -168,3 +168,52 @@ def test_quantities_are_summed_in_64_bits(rt, vec, lane):
     s.close()
     assert np.array_equal(got[:, 0], psi.ravel())
     assert q["mass"] == 2.0 ** -23
+
+
+def test_heun_average_rounds_once_at_the_size_of_psi(rt):
+    """Above 1e5 cells the streaming kernel sums differences. Stage 2 adds the update in half its size and psi^n / 2 in
+    one fused operation (psi^n + a psi first, and the differences to their half, rounds twice at the size of psi). All
+    ordinates flow towards +x, +y; cells three or more from the sides, operation by operation."""
+    nx, ny, sigma, q, dt = 420, 250, 3.0, 0.3, 2.0 ** -6
+    xi, eta, mu, w = rt.rt_quad_product(16, 32)
+    k = np.nonzero((xi > 0) & (eta > 0))[0][:32]
+    quad = tuple(v[k] for v in (xi, eta, mu, w))
+    mesh = si.CartesianMesh(nx=nx, ny=ny, x0=0.0, y0=0.0, dx=0.04, dy=0.05)
+    mats = si.Materials(sigma_a=np.array([sigma]), sigma_s=np.zeros(1), Q=np.array([q]), cell_mat=np.zeros(nx * ny, np.int32),
+                        cell_region=np.zeros(nx * ny, np.int32), region_names=("all",))
+    s = rt.Solver(si.Problem(mesh=mesh, materials=mats, boundary=si.Boundary(), t_end=64 * dt), quad, order=2,
+                  integrator=rt.RT_HEUN, dt=dt)
+    psi0 = (0.5 + si.random_psi(nx * ny, 32, seed=2)).astype(f32)
+    s.set_psi(psi0)
+    s.step(1)
+    got = s.psi().reshape(ny, nx, 32)
+    assert s.info.dt == dt
+    s.close()
+    h, one = f32(0.5), np.float64(1)
+
+    def fm(a, b, x):
+        return (one * a * b.astype(np.float64) + x).astype(f32)
+
+    def minmod(a, b):
+        return np.where(a * b > 0, np.where(np.abs(a) < np.abs(b), a, b), f32(0))
+
+    a, b = fm(-f32(dt), np.full((1,), f32(sigma)), f32(1)), f32(dt) * f32(q)
+    ax, ay = (f32(dt) * np.asarray(v, f32)[k] * f32(1.0 / d) for v, d in ((xi, mesh.dx), (eta, mesh.dy)))
+
+    def stage(u, base):
+        c = f32(1) if base is None else h
+        dx, dy = np.diff(u, axis=1, prepend=f32(0)), np.diff(u, axis=0, prepend=f32(0))
+        mx, my = minmod(dx[:, 1:], dx[:, :-1]), minmod(dy[1:], dy[:-1])          # of cells 0 .. n - 2
+        mx, my = np.concatenate([mx, mx[:, :1]], 1), np.concatenate([my, my[:1]], 0)   # (the last cells are not looked at)
+        g = fm(h, mx - np.roll(mx, 1, 1), dx)
+        z = (-c * ax) * g
+        low = h * np.roll(my, 1, 0)
+        z = fm(np.broadcast_to(-c * ay, u.shape), dy - low, z)
+        out = fm(np.broadcast_to(-c * ay, u.shape), h * my, z)
+        t = fm(c * a, u, c * b) + out
+        return t if base is None else fm(h, base, t)
+
+    u = psi0.reshape(ny, nx, 32)
+    want = stage(stage(u, None), u)
+    inner = np.s_[6:-6, 6:-6]
+    assert np.mean(got[inner] != want[inner]) <= 1e-5   # (fused operations that the 64-bit stand-in rounds twice)
