@@ -149,12 +149,16 @@ typedef void (*rt_free_fn)(void* ptr, void* ctx);
  *     every chunk of 128 or 64 ordinates has one sign of xi and one of eta (the product
  *     quadrature's quadrants are contiguous); RT_EINVAL if it is not. The
  *     library takes chunk-uniform directions where the chunks allow them, except
- *     where only chunks of 64 would on a grid of at most 1e5 cells.
+ *     where only chunks of 64 would on a grid of at most 1e5 cells. Both families run the
+ *     streaming kernel (see vec); at second order on at most 1e5 cells they differ in the
+ *     order of operations, elsewhere in the labels of rt_info_t alone.
  *   vec: Cartesian ordinates per lane (1, 2 or 4; 0 = chosen by the library);
  *     RT_EINVAL if the quadrature does not allow it (see rt_info_t for the choice).
  *     With per-lane directions, a number asks for the general kernel (the one that
  *     rt_cart_stage_noalloc runs); 0 lets the library take the streaming kernel where the
- *     ordinates allow it (it always takes four per lane).
+ *     ordinates allow it (it always takes four per lane). With chunk-uniform directions the
+ *     streaming kernel runs whatever the number, which is checked and reported, and sets the
+ *     order in which phi is summed at second order on at most 1e5 cells.
  *   alloc/free/alloc_ctx: device allocator (NULL = cudaMalloc/cudaFree).
  *   stream: cudaStream_t for every launch and copy. */
 typedef struct {
@@ -223,7 +227,8 @@ typedef struct {
                         triangles 3 first order with each chunk's rows staged in shared memory,
                         0 otherwise (rows gathered from global memory) */
   int32_t vec;       /* ordinates per lane (Cartesian: 0 if per-lane directions run in the streaming
-                        kernel, which takes four) */
+                        kernel, which takes four; with chunk-uniform directions the 32nd part of
+                        the chunks that have one sign each) */
   int32_t regrouped; /* Cartesian: 1 if the ordinates are stored regrouped by direction quadrant, each
                         quadrant padded with zero-weight ordinates to whole chunks (done when the
                         caller's order does not give sign-uniform chunks and the padding adds at most

@@ -31,8 +31,8 @@
 //
 // Update. With a = 1 - dt sigma_t and b = dt (sigma_s/(2 pi) phi + Q) per cell:
 //   Euler / Heun stage 1: out = a psi + b - dt (div_x + div_y)
-//   Heun stage 2:         out = (psi^n + a psi1 + b - dt (div_x + div_y)) / 2
-// (Eq. sn_2d_eqn_fv and Sec. 4.3). phi_out = sum_k w_k out_k: two rows are summed over
+//   Heun stage 2:         out = psi^n / 2 + (a psi1 + b - dt (div_x + div_y)) / 2
+// (Eq. sn_2d_eqn_fv and Sec. 4.3; the halves are exact, the last sum rounds once). phi_out = sum_k w_k out_k: two rows are summed over
 // 8 lanes by shuffles, chunks in the warp's own accumulators, the WC warps of a column
 // in fixed order at the end. The boundary outflow is taken from the stored rows after
 // the walk; the epilogue writes phi_out and the FP64 QoI partials.
@@ -46,8 +46,9 @@
 // lanes leave their terms of phi in shared memory (128 bytes per cell, no shuffles in the
 // walk), which are then added in the order of a warp's butterfly over the chunk. The face
 // values take 8 more registers (spilled, mostly at sides), the terms limit a segment to 13
-// rows with two CTAs per SM. Per Heun step, sums of differences and ordered: 140^2 x 128 52
-// and 55 us, 280^2 x 256 163 and 180; the general kernel 111 and 320.
+// rows with two CTAs per SM, and rules of more than 128 ordinates meet at a barrier of the
+// column's warps per 128. Per Heun step, sums of differences and ordered: 140^2 x 128 52
+// and 56 us, 280^2 x 256 163 and 179; the general kernel 111 and 320.
 //
 // Bound by: HBM on large grids (1400^2 x 512 FP32 Heun: 20 bytes per cell and ordinate
 // at 5.6 TB/s; a pair of rows is about 500 instructions for 16 values a lane, issue
@@ -55,9 +56,9 @@
 // Per Heun step, against the kernels that it replaced (one CTA barrier per row with
 // chunk-uniform directions; for mixed directions the general kernel of
 // cart_kernel.cuh): 1400^2 x 512 4.12 -> 3.57 ms (BF16 4.42 -> 3.69, first-order Euler
-// 1.51 -> 1.36), 700^2 x 484 1.36 -> 1.16, 531^2 x 100 0.57 -> 0.25. Measured and not kept: 4 cells per lane (12 warps
-// per SM: spills, and a loop too long for the instruction cache), scalar instead of
-// paired FP32 (24 % slower), prefetching the pair after next to L2.
+// 1.51 -> 1.36), 700^2 x 484 1.36 -> 1.13, 531^2 x 100 0.57 -> 0.25. Measured and not
+// kept: 4 cells per lane (12 warps per SM: spills, and a loop too long for the instruction
+// cache), scalar instead of paired FP32 (24 % slower), prefetching the pair after next to L2.
 #pragma once
 #include <cuda_bf16.h>
 

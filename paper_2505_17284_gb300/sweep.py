@@ -119,11 +119,10 @@ def group_key(j):
 def tune_groups(jobs, storage=rt.RT_FP32, tile_ys=(0, 16, 24, 32, 48), variants=(0, 1), steps=3, by_shape=False):
     """Per-group tuner: for each group of jobs with one ordinate count, order
     and integrator (and, with by_shape, one cell count), the (tile_y, variant)
-    pair with the shortest batch step, timed on that group's jobs alone. Small
-    grids with 4 quadrants of 64 ordinates, for example, run faster on the
-    per-lane-direction kernel (variant 1) than on the chunk-uniform one the
-    library picks for large grids. Returns (per-job config dicts, {group:
-    {"tile_y/variant": ms}})."""
+    pair with the shortest batch step, timed on that group's jobs alone (the
+    variants run one kernel at different tile widths, layouts or orders of
+    operations). Returns (per-job config dicts, {group: {"tile_y/variant":
+    ms}})."""
     groups = {}
     for i, j in enumerate(jobs):
         groups.setdefault(group_key(j) + ((j.n_cells,) if by_shape else ()), []).append(i)
