@@ -23,12 +23,12 @@
 //                      and the FP64 QoI partials as the first-order kernel does.
 //
 // Bound by the latency of the gathers (24 warps per SM in the gradient pass, 16 in
-// the stage pass; DRAM at 45 - 48 % of its peak, issue slots at 62 and 47 %). Differences
+// the stage pass; DRAM at 58 - 66 % of the copy rate, issue slots at 56 and 46 %). Differences
 // to the cell's value, not values, are summed over the edges: the sums of the normals
 // vanish, and the rounding error is smaller (650^2 x 256, one step against FP64: 4.22e-8
 // of psi, 4.33e-8 with values). At 400^2 x 256 (FP32), with IEEE divisions in divergent
 // branches and 2 ordinates per lane in the stage pass: gradient 0.82 ms, stage 0.45 ms;
-// now 0.27 and 0.35 ms. A Heun step at 650^2 x 256: 6.65 -> 3.27 ms.
+// now 0.25 and 0.37 ms. A Heun step at 650^2 x 256: 6.65 -> 3.27 ms.
 #include <cuda_bf16.h>
 
 #include <type_traits>
