@@ -584,7 +584,7 @@ static int stream_segment(const Instance& I, int run, int form, double* cost) {
       const double rounds = (double)items / (2.0 * sms);
       t = (7.0 + 1.28 * chunks * rows) * (form == STREAM_PLAIN ? rounds + 0.5 : std::ceil(rounds));
     }
-    if (t < *cost) {
+    if (form == STREAM_PLAIN ? t < *cost : t <= *cost) {   // equal rounds: the fewer items
       *cost = t;
       best = ly;
     }
