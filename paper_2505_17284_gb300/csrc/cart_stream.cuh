@@ -43,12 +43,14 @@
 // scheme to amplify that, the operations of those kernels are kept, value for value: face
 // values F = u + m/2 and G, then div = ax (F_1 - F_0) + ay (G_1 - G_0) with the last product
 // fused (y for per-lane directions, x for chunk-uniform ones), out = (a c + b) - div; and the
-// lanes leave their terms of phi in shared memory (128 bytes per cell, no shuffles in the
-// walk), which are then added in the order of a warp's butterfly over the chunk. The face
-// values take 8 more registers (spilled, mostly at sides), the terms limit a segment to 13
-// rows with two CTAs per SM, and rules of more than 128 ordinates meet at a barrier of the
-// column's warps per 128. Per Heun step, sums of differences and ordered: 140^2 x 128 52
-// and 56 us, 280^2 x 256 163 and 179; the general kernel 111 and 320.
+// lanes leave their terms of phi in shared memory (128 bytes per cell, or all ordinates where
+// V = 1; no shuffles in the walk), which are then added in the order of a warp's butterfly
+// over the chunk. The face values take 8 more registers (spilled, mostly at sides), the terms
+// limit a segment to 13 rows with two CTAs per SM (fewer for V = 1, which takes one CTA per SM
+// then), and rules of more than 128 ordinates meet at a barrier of the column's warps per
+// 128. Per Heun step, sums of differences, ordered, and the general kernel: 140^2 x 128 52, 56
+// and 111 us, 280^2 x 256 163, 179 and 320, 140^2 x 100 56, 66 and 135, 272^2 x 64 52, 65 and
+// 143 (300^2).
 //
 // Bound by: HBM on large grids (1400^2 x 512 FP32 Heun: 20 bytes per cell and ordinate
 // at 5.6 TB/s; a pair of rows is about 500 instructions for 16 values a lane, issue
@@ -96,7 +98,7 @@ struct StrCfg {
 };
 
 // Floats per cell that hold the lanes' terms of phi in the ordered form (form: CartForm).
-__host__ __device__ inline int str_parts(int form) { return form & (16 | 32 | 64); }
+__host__ __device__ inline int str_parts(int form) { return form >> 1; }
 // (a, b) of every cell, and one phi accumulator per cell and chunk group; in the ordered
 // form one per cell, and the lanes' terms
 __host__ __device__ inline size_t str_tile_bytes(int tx, int ly, int parts) {
@@ -240,7 +242,8 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
   const int dys = ch.z;
   const int n = w.yb - w.ya + L::EXTRA;                // rows of the chunk
   const int npair = (n + 1) / 2;
-  const bool part = !ORD && ch.y != (32 << 8);         // a partial window
+  constexpr bool PARTIAL = !ORD || V == 1;             // windows may be partial
+  const bool part = PARTIAL && ch.y != (32 << 8);
 
   float2 w2[2], ax2[2], ay2[2];
   float xsum = 0.f;
@@ -284,7 +287,12 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
   [[maybe_unused]] float* tpart = nullptr;
   [[maybe_unused]] int poff[R], pstep = 0;
   [[maybe_unused]] bool second = false;   // the term is added to that of the window 64 ordinates before
-  if constexpr (ORD) {
+  if constexpr (ORD && V == 1) {   // one ordinate per term: all ordinates of a cell in order
+    tpart = w.part + ((start - w.ya) * w.TX - L::EXTRA * astep + w.xl + R * grp) * w.parts + k0;
+    pstep = astep * w.parts;
+#pragma unroll
+    for (int r = 0; r < R; ++r) poff[r] = (dxs > 0 ? r : 1 - r) * w.parts;
+  } else if constexpr (ORD) {
     static_assert(R == 2, "pairs of cells");
     const int wslot = c & (w.slots - 1);
     tpart = w.part + ((start - w.ya) * w.TX - L::EXTRA * astep + w.xl + R * grp) * w.parts + l8 * (4 / V);
@@ -473,7 +481,17 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
         for (int r = 0; r < R; ++r) {
           float* p = tpart + poff[r];
           const float2 p0 = __fmul2_rn(w2[0], out[r][0]);
-          if constexpr (V == 4) {
+          if constexpr (V == 1) {
+            const float2 p1 = __fmul2_rn(w2[1], out[r][1]);
+            if (!part) {
+              *reinterpret_cast<float4*>(p) = make_float4(p0.x, p0.y, p1.x, p1.y);
+            } else {
+              const int lo = ch.x + (ch.y & 255), hi = ch.x + (ch.y >> 8);
+#pragma unroll
+              for (int v = 0; v < 4; ++v)
+                if (k0 + v >= lo && k0 + v < hi) p[v] = v == 0 ? p0.x : v == 1 ? p0.y : v == 2 ? p1.x : p1.y;
+            }
+          } else if constexpr (V == 4) {
             float t;
             if constexpr (FORM == STR_UNI) {
               const float2 pw = __ffma2_rn(w2[1], out[r][1], p0);
@@ -491,12 +509,12 @@ __device__ __forceinline__ void str_chunk(const InstDesc& d, const StrWarp& w, c
         }
       }
       tpart += pstep;
-      return;
-    }
+    } else {
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const float2 pw = __ffma2_rn(w2[1], out[r][1], __fmul2_rn(w2[0], out[r][0]));
-      c[r] = pw.x + pw.y;
+      for (int r = 0; r < R; ++r) {
+        const float2 pw = __ffma2_rn(w2[1], out[r][1], __fmul2_rn(w2[0], out[r][0]));
+        c[r] = pw.x + pw.y;
+      }
     }
   };
 
@@ -585,12 +603,35 @@ __device__ __forceinline__ void str_phi_ordered(const StrWarp& w, int wc, int WC
   }
 }
 
+// The same for one ordinate per lane: n ordinates, of which a lane here takes four in a row.
+__device__ __forceinline__ void str_phi_ordered1(const StrWarp& w, int wc, int WC, int n) {
+  const int lane = threadIdx.x & 31, l8 = lane & 7, grp = lane >> 3;
+  for (int i = wc; i < kStrRun * (w.yb - w.ya); i += WC) {
+    const int cell = (i >> 1) * w.TX + w.xl + kStrRun * grp + (i & 1);
+    const float* p = w.part + cell * w.parts;
+    float a = 0.f;
+    for (int k = 4 * l8; k - 4 * l8 < n; k += 32) {
+      float4 x = *reinterpret_cast<const float4*>(p + k);
+      float2 s = make_float2(k < n ? x.x : 0.f, k + 1 < n ? x.y : 0.f), t = make_float2(k + 2 < n ? x.z : 0.f, k + 3 < n ? x.w : 0.f);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        s = __fadd2_rn(s, make_float2(__shfl_xor_sync(0xffffffffu, s.x, o), __shfl_xor_sync(0xffffffffu, s.y, o)));
+        t = __fadd2_rn(t, make_float2(__shfl_xor_sync(0xffffffffu, t.x, o), __shfl_xor_sync(0xffffffffu, t.y, o)));
+      }
+      s = __fadd2_rn(s, t);
+      a += s.x + s.y;
+    }
+    if (l8 == 0) w.acc[cell] = a;
+  }
+}
+
 // Ordered form: the chunks of a warp. The warps of a strip meet where their windows complete
 // chunks of 32 V ordinates.
 template <int STAGE, typename T, int FORM, int V>
 __device__ __forceinline__ void str_chunks_ordered(const InstDesc& d, const StrWarp& w, int wx, int wc, int WC, bool active,
                                                    bool edge, int in_buf, T* __restrict__ psi_out, uint32_t salt) {
-  const int per = max(V, WC), n_chunks = d.n_chunks;
+  const int n_chunks = d.n_chunks;
+  [[maybe_unused]] const int per = max(V, WC);
   if (active) {
     int slot = 0;
 #pragma unroll 1
@@ -598,17 +639,20 @@ __device__ __forceinline__ void str_chunks_ordered(const InstDesc& d, const StrW
       const int4 ch = d.str_chunks[c];
       if (edge) str_chunk<2, STAGE, T, true, FORM, V>(d, w, ch, c, c + WC, slot, in_buf, psi_out, salt);
       else str_chunk<2, STAGE, T, false, FORM, V>(d, w, ch, c, c + WC, slot, in_buf, psi_out, salt);
-      const int next = c - wc + WC;   // first window of the strip's next round
-      if (next % per == 0 && next < n_chunks) {
-        str_strip_barrier(wx, WC);
-        str_phi_ordered<V>(w, wc, WC, per);
-        str_strip_barrier(wx, WC);
+      [[maybe_unused]] const int next = c - wc + WC;   // first window of the strip's next round
+      if constexpr (V > 1) {
+        if (next % per == 0 && next < n_chunks) {
+          str_strip_barrier(wx, WC);
+          str_phi_ordered<V>(w, wc, WC, per);
+          str_strip_barrier(wx, WC);
+        }
       }
     }
     cp_async_wait<0>();
   }
   __syncthreads();
-  str_phi_ordered<V>(w, wc, WC, n_chunks - (n_chunks - 1) / per * per);
+  if constexpr (V > 1) str_phi_ordered<V>(w, wc, WC, n_chunks - (n_chunks - 1) / per * per);
+  else str_phi_ordered1(w, wc, WC, d.M);
   __syncthreads();
 }
 
@@ -741,7 +785,8 @@ __global__ void __launch_bounds__(kStrThreads, 2)
   const int n_chunks = d.n_chunks;
   if constexpr (ORD) {
     if (d.ord_vec == 4) str_chunks_ordered<STAGE, T, FORM, 4>(d, w, wx, wc, WC, active, edge, in_buf, psi_out, salt);
-    else str_chunks_ordered<STAGE, T, FORM, 2>(d, w, wx, wc, WC, active, edge, in_buf, psi_out, salt);
+    else if (d.ord_vec == 2) str_chunks_ordered<STAGE, T, FORM, 2>(d, w, wx, wc, WC, active, edge, in_buf, psi_out, salt);
+    else if constexpr (FORM == STR_LANE) str_chunks_ordered<STAGE, T, FORM, 1>(d, w, wx, wc, WC, active, edge, in_buf, psi_out, salt);
   } else {
     if (active) {
       int slot = 0;

@@ -559,8 +559,9 @@ static bool regroup_quadrature(const rt_quadrature* quad, std::vector<double>& x
 // 1078 at 57, 976 at 44). Against timings of 29 problems at 3 to 64 rows (70^2 x 64 to
 // 1400^2 x 512) its choice is 4 % from the best on average, 14 % at most. The ordered form's
 // few items come in whole rounds (280^2 x 256 Heun: 576 items of 9 rows 173 us, 504 of 10 rows
-// 192): 2 % from the best of 3 to 13 rows on average over 21 problems of 50^2 x 64 to
-// 280^2 x 512. *cost receives the model's time.
+// 192), of which those with one CTA per SM take 0.72 of the sum (272^2 x 64 65 us at 17 rows, 77
+// at 5): 1 % from the best of 3 to 13 rows on average over 73 problems of 50^2 x 64 to
+// 315^2 x 512. *cost receives the model's time.
 static int stream_segment(const Instance& I, int run, int form, double* cost) {
   const int sms = device_sm_count();
   const int tx = cart_tile_width(run), groups = cart_stream_chunk_groups(tx);
@@ -571,13 +572,18 @@ static int stream_segment(const Instance& I, int run, int form, double* cost) {
   *cost = INFINITY;
   const int ly_most = I.str_chunks.size() > 1 ? 40 : 64;
   for (int ly = 3; ly <= ly_most; ++ly) {
-    // two CTAs per SM by shared memory (228 KB, 1 KB of it per CTA reserved)
-    if (cart_smem_bytes(I.order, I.storage, run, I.cvec, ly, stage_hi, form) > 113 * 1024) break;
+    // two CTAs per SM by shared memory (228 KB, 1 KB of it per CTA reserved); one in the
+    // ordered form where that allows longer segments
+    const size_t smem = cart_smem_bytes(I.order, I.storage, run, I.cvec, ly, stage_hi, form);
+    const bool alone = smem > 113 * 1024;
+    if (alone && (form == STREAM_PLAIN || smem > 227 * 1024)) break;
     const int64_t items = strips * ((I.ny + ly - 1) / ly);
     const int rows = (std::min(ly, I.ny) + (I.order == 2 ? 3 : 1) + 1) / 2 * 2;
     double t;
     if (items <= sms) {
       t = 9.6 + (double)chunks * rows;
+    } else if (alone) {
+      t = 0.72 * (9.6 + (double)chunks * rows) * std::ceil((double)items / sms);
     } else if (items <= 2 * sms) {
       t = 12.0 + 1.28 * chunks * rows;
     } else {
@@ -599,8 +605,9 @@ static int stream_segment(const Instance& I, int run, int form, double* cost) {
 // differ by 1e-5 after 32 Heun steps and by up to 2e-3 after 96 on lattices of 140^2 to 280^2
 // cells (relative L2 of psi 1e-7 and 3e-6; both are as far from FP64). Small grids are those
 // that run for hundreds of steps, so there the streaming kernel takes its ordered form where
-// the windows are whole, and per-lane directions that allow no such form (one ordinate per
-// lane) stay on the general kernel. First order contracts, and keeps to rounding anyway.
+// the windows are whole or hold one ordinate per lane of that kernel, and per-lane directions
+// that allow no such form stay on the general kernel. First order contracts, and keeps to
+// rounding anyway.
 constexpr int64_t kOrderedMaxCells = 100000;
 
 // Form of the streaming kernel (CartForm) for tiles of `run`: the ordered one if I.ord_vec is
@@ -608,8 +615,9 @@ constexpr int64_t kOrderedMaxCells = 100000;
 // warps (32-cell tiles) add the four windows of 4 ordinates per lane in place, in pairs.
 static int ordered_form(const Instance& I, int run) {
   if (!I.ord_vec) return STREAM_PLAIN;
+  if (I.ord_vec == 1) return 2 * I.Mpad;   // windows need not be whole: all ordinates
   const int windows = std::min(cart_stream_chunk_groups(cart_tile_width(run)), (int)I.str_chunks.size());
-  return 32 / I.ord_vec * windows + (I.info_variant == 2 ? STREAM_UNI : 0);
+  return 2 * (32 / I.ord_vec * windows) + (I.info_variant == 2 ? STREAM_UNI : 0);
 }
 
 static void choose_cart_tiles(Instance& I, int tile_y) {
@@ -778,7 +786,10 @@ static rt_status plan_cart(Instance& I, const rt_quadrature* quad, int tile_x, i
   };
   I.ord_vec = 0;
   if (I.order == 2 && I.n_cells <= kOrderedMaxCells && !I.str_chunks.empty()) {
-    if (I.cvec > 1 && windows_whole(I.str_chunks, I.Mpad)) I.ord_vec = I.cvec;
+    if (I.cvec == 1 || windows_whole(I.str_chunks, I.Mpad)) I.ord_vec = I.cvec;
+    double cost;   // some segment must fit
+    if (I.ord_vec) stream_segment(I, I.run, ordered_form(I, I.run), &cost);
+    if (I.ord_vec && std::isinf(cost)) I.ord_vec = 0;
     if (I.ord_vec && !fits(I.run)) I.ord_vec = 0;
     if (!I.ord_vec && !I.uni) I.str_chunks.clear();
   }
@@ -1141,8 +1152,8 @@ rt_status build_instance(const rt_mesh* mesh, const rt_materials* mat, const rt_
   D.n_chunks = I.kind != RT_MESH_CARTESIAN ? I.Mpad / kChunk
                : I.uni ? (int32_t)I.str_chunks.size() : I.Mpad / (32 * I.cvec);
   D.str_chunks = d_str_chunks;
-  D.ord_vec = I.uni >= 16 ? I.ord_vec : 0;
-  D.ord_parts = I.uni & ~STREAM_UNI;
+  D.ord_vec = I.uni > STREAM_PLAIN ? I.ord_vec : 0;
+  D.ord_parts = I.uni >> 1;
   D.tx = I.tx; D.ly = I.ly; D.n_strips = I.n_strips;
   D.n_segs = I.n_segs; D.n_items = (int32_t)I.stage_items.size(); D.n_regions = I.n_regions;
   D.n_cells = n_cells; D.n_steps = I.n_steps;

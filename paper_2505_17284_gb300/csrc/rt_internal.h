@@ -31,8 +31,8 @@ constexpr int kTriStgChunk = 32;       // cells per chunk of the staged first-or
 
 enum Stage : int32_t { STAGE_EULER = 0, STAGE_HEUN1 = 1, STAGE_HEUN2 = 2, STAGE_INIT = 3 };
 // Cartesian kernels (the launchers' `uni`): the general one, the streaming one, and the
-// latter in its ordered form: 16, 32 or 64 (floats per cell that hold the lanes' terms of
-// phi in shared memory), + STREAM_UNI with the operations of chunk-uniform directions.
+// latter in its ordered form: twice the floats per cell that hold the lanes' terms of phi in
+// shared memory, + STREAM_UNI with the operations of chunk-uniform directions.
 enum CartForm : int32_t { CART_GENERAL = 0, STREAM_PLAIN = 1, STREAM_UNI = 1 };
 enum Kind : int32_t { KIND_CART = 0, KIND_TRI = 1 };
 
@@ -79,7 +79,7 @@ struct alignas(128) InstDesc {
   int32_t nx, ny, M, Mpad;
   int32_t n_chunks, tx, ly, n_strips;
   int32_t n_segs, n_items, n_regions;
-  // streaming Cartesian kernel, ordered form: ordinates per term of phi (2 or 4), floats per
+  // streaming Cartesian kernel, ordered form: ordinates per term of phi (1, 2 or 4), floats per
   // cell that hold the terms
   int32_t ord_vec, ord_parts, pad1;
   int64_t n_cells;

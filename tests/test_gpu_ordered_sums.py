@@ -59,13 +59,17 @@ def test_streaming_and_general_kernel_store_the_same_bits(rt, n_p, n_phi, vec, n
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
 
 
-@pytest.mark.parametrize("quad", ["tess-3", "tess-5", "tess-9"])
-def test_rules_of_one_ordinate_per_lane_stay_on_the_general_kernel(rt, quad):
-    p, q = problem(40, 33, seed=2), rt.rt_quad_tessellation(int(quad[5:]))
+@pytest.mark.parametrize("quad,vec", [("tess-3", 1), ("tess-5", 0), ("tess-7", 0), ("tess-9", 0), ("prod-6x16", 0)])
+@pytest.mark.parametrize("nx,ny,tile_y,periodic", [(70, 70, 0, False), (93, 41, 0, False), (31, 57, 2, True), (9, 3, 7, False),
+                                                   (61, 70, 63, False)])
+def test_rules_of_one_ordinate_per_lane(rt, quad, vec, nx, ny, tile_y, periodic):
+    """The same where quadrants are no multiples of two ordinates, so that windows are partial (tess-3 allows none)."""
+    p = problem(nx, ny, seed=2, periodic=periodic)
+    q = rt.rt_quad_tessellation(int(quad[5:])) if quad[0] == "t" else rt.rt_quad_product(*map(int, quad[5:].split("x")))
     psi0 = state(p, len(q[0]), seed=5)
-    a = after(rt, p, q, psi0, 40, integrator=rt.RT_HEUN, variant=1)
-    b = after(rt, p, q, psi0, 40, integrator=rt.RT_HEUN, variant=1, vec=1)
-    assert a[2].vec == 1
+    a = after(rt, p, q, psi0, 96, integrator=rt.RT_HEUN, variant=1, tile_y=tile_y)
+    b = after(rt, p, q, psi0, 96, integrator=rt.RT_HEUN, variant=1, vec=1, tile_y=16)
+    assert a[2].vec in (vec, 1)   # (1 where so long a segment does not fit)
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
 
 
