@@ -219,7 +219,7 @@ rt_status add_in_slot(rt_batch* b, const rt_problem& P, int i) {
 // Rebuild the work list of the unfinished problems, grouped by kernel variant.
 rt_status rebuild(rt_batch* b) {
   drop_graph(b);
-  std::map<std::tuple<int, int, int, int, int, int, int>, std::vector<int>> by_variant;
+  std::map<std::tuple<int, int, int, int, int, int, int, int>, std::vector<int>> by_variant;
   b->members.clear();
   for (int i = 0; i < (int)b->slots.size(); ++i) {
     const Slot& S = b->slots[i];
@@ -227,14 +227,17 @@ rt_status rebuild(rt_batch* b) {
     const Instance& I = S.inst;
     // (the Cartesian kernels do not depend on I.vec)
     const int vec = I.kind == RT_MESH_CARTESIAN ? 0 : I.vec;
-    by_variant[std::make_tuple(I.kind, I.order, I.integrator, I.run, I.cvec, vec, I.uni)].push_back(i);
+    // (a launch takes the shared memory of its longest segment: members whose blocks have an SM
+    // to themselves would take every other member's second block from it)
+    const int alone = I.kind == RT_MESH_CARTESIAN && I.cart_smem > 113 * 1024 ? 1 : 0;
+    by_variant[std::make_tuple(I.kind, I.order, I.integrator, I.run, I.cvec, vec, I.uni, alone)].push_back(i);
     b->members.push_back(i);
   }
   std::vector<WorkItem> items, box_items;
   b->groups.clear();
   for (auto& kv : by_variant) {
     Group g{};
-    std::tie(g.kind, g.order, g.integrator, g.run, g.cvec, g.vec, g.uni) = kv.first;
+    std::tie(g.kind, g.order, g.integrator, g.run, g.cvec, g.vec, g.uni, std::ignore) = kv.first;
     g.offset = (int)items.size();
     g.box_offset = (int)box_items.size();
     g.ly_max = 1;

@@ -150,3 +150,27 @@ def test_order_of_operations_of_a_stage(rt, n_p, n_phi, variant, tile_x, V):
     psi, phi = stage(p, quad, psi0, phi0, got[2].dt, V, variant == 2)
     psi, phi = stage(p, quad, psi, phi, got[2].dt, V, variant == 2)
     assert np.mean(got[0] != psi) <= 1e-6 and np.mean(got[1] != phi) <= 1e-6
+
+
+def test_batch_members_keep_their_bits(rt):
+    """Members of every form in one batch: ordered with two blocks and with one block per SM (272^2 x 64), with one,
+    two and four ordinates per lane, plain (330^2) and general (tess-3): psi and QoIs as alone, bit for bit."""
+    members = [(272, "4x16"), (70, "4x16"), (96, "8x16"), (64, "16x32"), (50, "t5"), (330, "4x16"), (40, "t3"), (70, "4x16")]
+    probs, quads = [], []
+    for n, rule in members:
+        p = si.lattice_problem(n)
+        p.t_end = 100.0
+        probs.append(p)
+        quads.append(rt.rt_quad_tessellation(int(rule[1:])) if rule[0] == "t" else rt.rt_quad_product(*map(int, rule.split("x"))))
+    b = rt.Batch(probs, quads, order=2, integrator=rt.RT_HEUN, dts=[0.5 * p.mesh.dx for p in probs])
+    b.step(3)
+    b.step(8)
+    for i, (p, q) in enumerate(zip(probs, quads)):
+        s = rt.Solver(p, q, order=2, integrator=rt.RT_HEUN, dt=0.5 * p.mesh.dx)
+        s.step(11)
+        mine, alone = b.qoi(i), s.qoi()
+        for k in ("abs_now", "abs_int", "mass", "outflow_now", "outflow_int", "box_out_now"):
+            assert np.array_equal(np.asarray(mine[k]), np.asarray(alone[k])), (members[i], k)
+        assert np.array_equal(b.psi(i), s.psi()), members[i]
+        s.close()
+    b.close()
