@@ -548,6 +548,9 @@ static bool regroup_quadrature(const rt_quadrature* quad, std::vector<double>& x
   return false;
 }
 
+// Dynamic shared memory that a CTA of the streaming kernel can have: 227 KB less its static part.
+constexpr size_t kMaxDynamicSmem = 227 * 1024 - 256;
+
 // Segment length of the streaming kernel for a tile of I.run, by a model of a launch in
 // units of one row of a warp that shares its SM with one CTA. A CTA costs a fixed part
 // (start, tile constants, QoI sums, about 10 rows) and chunks x rows, 1.28 times that
@@ -576,7 +579,7 @@ static int stream_segment(const Instance& I, int run, int form, double* cost) {
     // ordered form where that allows longer segments
     const size_t smem = cart_smem_bytes(I.order, I.storage, run, I.cvec, ly, stage_hi, form);
     const bool alone = smem > 113 * 1024;
-    if (alone && (form == STREAM_PLAIN || smem > 227 * 1024)) break;
+    if (alone && (form == STREAM_PLAIN || smem > kMaxDynamicSmem)) break;
     const int64_t items = strips * ((I.ny + ly - 1) / ly);
     const int rows = (std::min(ly, I.ny) + (I.order == 2 ? 3 : 1) + 1) / 2 * 2;
     double t;
@@ -782,7 +785,7 @@ static rt_status plan_cart(Instance& I, const rt_quadrature* quad, int tile_x, i
   auto fits = [&](int run) {
     const int stage_hi = I.integrator == RT_HEUN ? STAGE_HEUN2 : STAGE_EULER;
     return tile_y <= 0 || cart_smem_bytes(I.order, I.storage, run, 4, std::min(tile_y, 256), stage_hi,
-                                          ordered_form(I, run)) <= 227 * 1024;
+                                          ordered_form(I, run)) <= kMaxDynamicSmem;
   };
   I.ord_vec = 0;
   if (I.order == 2 && I.n_cells <= kOrderedMaxCells && !I.str_chunks.empty()) {

@@ -73,6 +73,19 @@ def test_rules_of_one_ordinate_per_lane(rt, quad, vec, nx, ny, tile_y, periodic)
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
 
 
+@pytest.mark.parametrize("n_p,n_phi,tile_y,integrator", [(9, 32, 8, "HEUN"), (11, 32, 8, "EULER"), (9, 32, 0, "HEUN")])
+def test_segments_at_the_limit_of_shared_memory(rt, n_p, n_phi, tile_y, integrator):
+    """8 rows of 288 ordinates (Heun; 352 in BF16 Euler) leave 112 bytes of a block's 227 KB: less than the kernel's own
+    variables, so the general kernel takes them."""
+    p, quad = problem(100, 64, seed=1), rt.rt_quad_product(n_p, n_phi)
+    psi0 = state(p, n_p * n_phi, seed=4)
+    storage = rt.RT_BF16 if integrator == "EULER" else rt.RT_FP32
+    options = dict(integrator=getattr(rt, "RT_" + integrator), variant=1, storage=storage)
+    a = after(rt, p, quad, psi0, 3, tile_y=tile_y, **options)
+    b = after(rt, p, quad, psi0, 3, tile_y=8, vec=1, **options)
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
 def fma(a, b, c):
     """a b + c in one rounding (the product of two floats is exact in 64 bits)."""
     return (a.astype(np.float64) * b.astype(np.float64) + c.astype(np.float64)).astype(f32)
